@@ -200,10 +200,6 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
                           const DecodeExtra& extra);
 // Prefill attention: codes workspace bytes, and the two launches (codes, attention).
 size_t prefill_workspace(int batch, int n_kv, int n_ctx);
-// The codes launch alone: the signed codes of every slot of `layer` for tokens [0, n_ctx) as f16
-// in the prefill workspace layout ([b][slot][K|V][n_ctx_pad][128], value tiles transposed).
-cudaError_t launch_codes(const Plan& plan, int layer, const void* cache, int batch, int n_ctx, int max_tokens,
-                         void* ws, cudaStream_t st);
 cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_start, int n_q, const void* cache,
                            int batch, int n_ctx, int max_tokens, float* out, void* ws, cudaStream_t st);
 cudaError_t launch_dequant(const Plan& plan, int layer, const void* cache, int batch, int t0, int n,

@@ -4,9 +4,9 @@
 //
 // Two launches per call:
 //   codes    per (128-token tile, kv-head x K|V, sequence): the packed records -> the signed codes
-//            code_c = u_c - 2^(b_c - 1) as f16 (exact: |code| <= 128) in a workspace of rows of 128
-//            f16, [b][h][K|V][n_ctx_pad][128]: key rows are tokens, value tiles are stored
-//            transposed ([tile][channel][token]) so both are K-major tensor-core operands;
+//            code_c = u_c - 2^(b_c - 1) as f16 (exact: |code| <= 2048) in a workspace of 32 KB tiles,
+//            [b][h][K|V][tile]: key rows are tokens, value rows channels, both K-major tensor-core
+//            operands laid out with the 128-byte swizzle, so one plain bulk copy fetches a tile;
 //   attn     per (128 query rows, kv-head, sequence), rows = (query token, head of the GQA group),
 //            everything on the tensor cores (tcgen05): q' = (U_K^T q) f^K log2(e) / sqrt(128),
 //            per 128-token tile S = alpha^K (q'_hi + q'_lo) . code^K, causal mask, lazily
@@ -31,83 +31,182 @@ struct PrefillArgs {
   const float* alpha;        // cache alpha region
   const __nv_bfloat16* q;    // [batch][n_q][H_q][128]
   float* out;                // [batch][n_q][H_q][128]
-  __half* codes;             // workspace [batch][n_kv][2][n_ctx_pad][128]
+  __half* codes;             // workspace [batch][n_kv][2][tile]: 128 x 128 operands (swizzled)
   const float* u32;          // plan: [S][128 dim][128 ch]
   const float* u32t;         // plan: [S][128 ch][128 dim]
   const float* f;            // plan: [S][128]
   const ChanEnc* enc;        // plan: [S][128] (offsets 2^(b-1))
   const StreamLayout* lay;   // plan: [S]
-  const short* entry;        // plan: [S][n_entries]
-  const short* chan_ent;     // plan: [S][128][kChanEnt]
-  int layer, n_kv, n_q_heads, group, q_start, n_q, n_ctx, n_ctx_pad, n_tiles, n_words, n_entries;
+  int layer, n_kv, n_q_heads, group, q_start, n_q, n_ctx, n_ctx_pad, n_tiles, n_words;
   int* err;
 };
 
+constexpr int kTAtom = 128 * 128;                  // one 128-row K-atom (64 16-bit values per row)
+constexpr int kTOp = 2 * kTAtom;                   // one 128 x 128 16-bit operand (two K-atoms)
+
+// byte offset of element (row, k) of a 128-row K-major operand with the 128-byte swizzle
+__device__ __forceinline__ int sw128_off(int row, int k) {
+  return (k >> 6) * kTAtom + (row >> 3) * 1024 + (row & 7) * 128 + ((((k & 63) >> 3) ^ (row & 7)) << 4) + (k & 7) * 2;
+}
+
+// Four base-4 digits (8 bits) -> the low two bits of four bytes; four single bits -> four bytes.
+__device__ __forceinline__ uint32_t spread_digits(uint32_t x) {
+  const uint32_t y = (x | (x << 12)) & 0x000F000Fu;
+  return (y | (y << 6)) & 0x03030303u;
+}
+__device__ __forceinline__ uint32_t spread_bits(uint32_t x) { return (x * 0x00204081u) & 0x01010101u; }
+__device__ __forceinline__ uint32_t low_mask(int n) { return n >= 32 ? 0xFFFFFFFFu : (1u << n) - 1u; }
+
+// One CTA per (128-token tile, kv-head x K|V, sequence), thread = token: the packed record -> the
+// signed codes as one 32 KB tensor-core operand, written as a whole by a bulk copy.
+// The record is read as the bit stream that the encode wrote (digit layers in channel order, then
+// the odd widths' top bits, then the digits moved out of the last D2 word): 16 digits or up to 32
+// bits per step, spread into the byte lanes of 32 registers (stored value u_c of channel c = byte
+// c & 3 of U[c >> 2]; kWide: UH holds the high bytes of the first 32 channels), which the run
+// bounds, uniform over the CTA, guard.  code = u - 2^(b-1) as f16: below 9 bits the byte is put
+// into the mantissa of 1024 + u, and (1024 + u) - (1024 + 2^(b-1)) is exact.
+// Bound by issue next to the write of 256 B per token and stream: 8 heads x 30011 tokens at 2.75
+// bits take 45 us (2.7 TB/s written), a single tile 6 us.  Reading each channel's entries through
+// the plan's entry lists, one field at a time in dependent loads, took 280 us and 60 us.
+template <bool kWide>
 __global__ void __launch_bounds__(TILE) aatc_prefill_codes_kernel(const PrefillArgs a) {
-  __shared__ uint32_t rec[32][TILE];           // record words of the tile's tokens (W <= 32)
+  extern __shared__ __align__(128) unsigned char smc[];
+  unsigned char* op = smc;                                        // the operand, swizzled
+  uint32_t* rec = reinterpret_cast<uint32_t*>(smc + kTOp);        // [n_words + 1][128], token-planar
+  __shared__ __align__(16) uint32_t off2[D / 2];                  // f16 pairs 1024 + 2^(b-1) of channels 2i, 2i + 1
+  __shared__ float offw[32];                                      // 2^(b-1) of the first 32 channels (kWide)
+  __shared__ StreamLayout ly;
   const int tile = blockIdx.x, hk = blockIdx.y, b = blockIdx.z, t = threadIdx.x;
   const int head = hk >> 1, kind = hk & 1;
   const size_t cs = (static_cast<size_t>(b) * a.n_kv + head) * 2 + kind;
-  const int tok = tile * TILE + t;
-  __half* dst = a.codes + (cs * a.n_ctx_pad + tok) * D;
-  if (tok >= a.n_ctx) {                        // padding rows of the last tile: zero codes
-    if (tok < a.n_ctx_pad) {
-      if (kind == 1) {
-        __half* d2 = a.codes + cs * a.n_ctx_pad * D + static_cast<size_t>(tile) * TILE * D + t;
-        for (int c = 0; c < D; ++c) d2[c * TILE] = __float2half_rn(0.0f);
-      } else {
-        for (int c = 0; c < D; c += 8) *reinterpret_cast<uint4*>(dst + c) = make_uint4(0u, 0u, 0u, 0u);
-      }
-    }
-    return;
-  }
   const int s = (a.layer * a.n_kv + head) * 2 + kind;
-  const StreamLayout ly = a.lay[s];
-  const int nw = ly.n2 / 16 + (ly.n1 + 31) / 32;
+  const int nw = a.lay[s].words;
   const uint32_t* tw = a.words + (cs * a.n_tiles + tile) * static_cast<size_t>(a.n_words) * TILE;
-  for (int w = 0; w < nw; ++w) {
-    const uint32_t* ww = tw + static_cast<size_t>(w) * TILE;
-    uint32_t x;
-    if (kind == 0) {
-      x = ww[t];
-    } else {                                   // quad-interleaved: quarter r in slot 4Q + (0, 2, 1, 3)[r]
-      const int q4 = 4 * (t >> 2), sh = 8 * (t & 3);
-      x = ((ww[q4] >> sh) & 0xFFu) | (((ww[q4 + 2] >> sh) & 0xFFu) << 8) | (((ww[q4 + 1] >> sh) & 0xFFu) << 16) |
-          (((ww[q4 + 3] >> sh) & 0xFFu) << 24);
-    }
-    rec[w][t] = x;                             // each thread reads back only its own column
+  if (t < D / 2) {
+    const __half2 o = __floats2half2_rn(1024.0f + a.enc[s * D + 2 * t].off, 1024.0f + a.enc[s * D + 2 * t + 1].off);
+    off2[t] = *reinterpret_cast<const uint32_t*>(&o);
   }
-  const short* ce = a.chan_ent + static_cast<size_t>(s) * D * kChanEnt;
-  const short* ent = a.entry + static_cast<size_t>(s) * a.n_entries;
-  // values for the tensor-core kernel: per 128-token tile [channel][token]
-  __half* dst_t = a.codes + cs * a.n_ctx_pad * D + static_cast<size_t>(tile) * TILE * D + t;
-  const bool transposed = kind == 1;
-  for (int c = 0; c < D; c += 2) {
-    float v2[2];
+  if (kWide && t < 32) offw[t] = a.enc[s * D + t].off;
+  if (t < static_cast<int>(sizeof(StreamLayout) / 4))
+    reinterpret_cast<int*>(&ly)[t] = reinterpret_cast<const int*>(a.lay + s)[t];
+  for (int w0 = 0; w0 < nw; w0 += 8) {
+    uint32_t x[8];
 #pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int cc = c + i;
-      uint32_t u = 0;
-      for (int k = 0; k < kChanEnt; ++k) {
-        const int e = ce[cc * kChanEnt + k];
-        if (e < 0) break;
-        uint32_t v;
-        if (e < ly.n2) {
-          v = (rec[e >> 4][t] >> (2 * (e & 15))) & 3u;
-        } else {
-          const int e1 = e - ly.n2;
-          v = (rec[ly.n2 / 16 + (e1 >> 5)][t] >> (e1 & 31)) & 1u;
-        }
-        u |= v << ((ent[e] >> 8) & 15);
+    for (int i = 0; i < 8; ++i) x[i] = w0 + i < nw ? tw[(w0 + i) * TILE + t] : 0u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (w0 + i < nw) rec[(w0 + i) * TILE + t] = x[i];
+  }
+  rec[nw * TILE + t] = 0u;                     // read (and masked) past the last word
+  if (kind == 1) {
+    // quad-interleaved: byte t & 3 of slots 4Q + (0, 2, 1, 3)[r] is quarter r of this token's word
+    const uint32_t lo = (t & 3) | ((4 + (t & 3)) << 4);
+    for (int w = 0; w < nw; ++w) {
+      __syncwarp();
+      const uint4 q = *reinterpret_cast<const uint4*>(rec + w * TILE + (t & ~3));
+      __syncwarp();
+      rec[w * TILE + t] = __byte_perm(__byte_perm(q.x, q.z, lo), __byte_perm(q.y, q.w, lo), 0x5410);
+    }
+  }
+  __syncthreads();                             // off2, offw, ly
+  auto get = [&](int p) {                      // the 32 record bits from bit p on (own column)
+    const uint32_t* r = rec + (p >> 5) * TILE + t;
+    return __funnelshift_r(r[0], r[TILE], p & 31);
+  };
+  uint32_t U[32], UH[8];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) U[i] = 0u;
+#pragma unroll
+  for (int i = 0; i < 8; ++i) UH[i] = 0u;
+  constexpr int kLayers = kWide ? 8 : 4;
+  int pos = 2 * ly.n2, mpos = pos;             // D1 bits; the moved digits after them
+#pragma unroll
+  for (int k = 0; k < kLayers; ++k) mpos += ly.lodd[k] - ly.l2all[k];
+  // the odd widths' top bits: channels [a, b) have width 2k + 1
+#pragma unroll 1
+  for (int k = kLayers - 1; k >= 0; --k) {
+    const int ca = ly.l2all[k], cb = ly.lodd[k];
+    if (ca >= cb) continue;
+    const int sh = 2 * (k & 3);
+    auto put = [&](int i, uint32_t (&dst)[8]) {            // 32 channels from 32 i
+      const int lo = max(ca - 32 * i, 0), n = min(cb - 32 * i, 32) - lo;
+      const uint32_t v = (get(pos) & low_mask(n)) << lo;
+      pos += n;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) dst[j] |= spread_bits((v >> (4 * j)) & 15u) << sh;
+    };
+    if (kWide && k >= 4) {
+      put(0, UH);
+      continue;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (ca < 32 * i + 32 && cb > 32 * i) put(i, *reinterpret_cast<uint32_t(*)[8]>(&U[8 * i]));
+  }
+  // digit layers: layer k has the digits of channels [0, l2all[k]), the first l2[k] of them in D2
+  pos = 0;
+#pragma unroll 1
+  for (int k = 0; k < kLayers; ++k) {
+    const int lk = ly.l2[k], la = ly.l2all[k];
+    if (la == 0) break;
+    const int sh = 2 * (k & 3);
+    auto put = [&](int c, uint32_t (&dst)[4]) {            // 16 channels from 16 c
+      const int nd = min(max(lk - 16 * c, 0), 16), nm = min(la - 16 * c, 16) - nd;
+      uint32_t v = nd > 0 ? get(pos + 32 * c) & low_mask(2 * nd) : 0u;
+      if (nm > 0) {                                        // at most 15 digits move in all
+        v |= (get(mpos) & low_mask(2 * nm)) << (2 * nd);
+        mpos += 2 * nm;
       }
-      v2[i] = static_cast<float>(u) - a.enc[s * D + cc].off;   // dropped channels: u = off = 0
-    }
-    if (transposed) {
-      dst_t[c * TILE] = __float2half_rn(v2[0]);
-      dst_t[(c + 1) * TILE] = __float2half_rn(v2[1]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) dst[j] |= spread_digits((v >> (8 * j)) & 0xFFu) << sh;
+    };
+    if (kWide && k >= 4) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+        if (16 * c < la) put(c, *reinterpret_cast<uint32_t(*)[4]>(&UH[4 * c]));
     } else {
-      *reinterpret_cast<__half2*>(dst + c) = __floats2half2_rn(v2[0], v2[1]);
+#pragma unroll
+      for (int c = 0; c < 8; ++c)
+        if (16 * c < la) put(c, *reinterpret_cast<uint32_t(*)[4]>(&U[4 * c]));
     }
+    pos += 2 * lk;
+  }
+  // f16 codes into the operand: keys K = channel, row = token; values K = token, row = channel
+#pragma unroll
+  for (int g8 = 0; g8 < 16; ++g8) {                        // eight channels
+    const uint4 o4 = *reinterpret_cast<const uint4*>(off2 + 4 * g8);
+    const uint32_t ov[4] = {o4.x, o4.y, o4.z, o4.w};
+    uint32_t h[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t u = U[2 * g8 + (j >> 1)];
+      if (kWide && g8 < 4) {
+        const uint32_t uh = UH[2 * g8 + (j >> 1)], i0 = 16 * (j & 1);
+        const float u0 = static_cast<float>(((u >> i0) & 0xFFu) | (((uh >> i0) & 0xFFu) << 8));
+        const float u1 = static_cast<float>(((u >> (i0 + 8)) & 0xFFu) | (((uh >> (i0 + 8)) & 0xFFu) << 8));
+        const __half2 c2 = __floats2half2_rn(u0 - offw[8 * g8 + 2 * j], u1 - offw[8 * g8 + 2 * j + 1]);
+        h[j] = *reinterpret_cast<const uint32_t*>(&c2);
+      } else {
+        const uint32_t m = __byte_perm(u, 0x64646464u, (j & 1) ? 0x4342 : 0x4140);   // 1024 + u, twice
+        const __half2 c2 = __hsub2(*reinterpret_cast<const __half2*>(&m), *reinterpret_cast<const __half2*>(&ov[j]));
+        h[j] = *reinterpret_cast<const uint32_t*>(&c2);
+      }
+    }
+    if (kind == 0) {
+      *reinterpret_cast<uint4*>(op + sw128_off(t, 8 * g8)) = make_uint4(h[0], h[1], h[2], h[3]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        *reinterpret_cast<uint16_t*>(op + sw128_off(8 * g8 + 2 * j, t)) = static_cast<uint16_t>(h[j]);
+        *reinterpret_cast<uint16_t*>(op + sw128_off(8 * g8 + 2 * j + 1, t)) = static_cast<uint16_t>(h[j] >> 16);
+      }
+    }
+  }
+  ptx::fence_proxy_async_smem();
+  __syncthreads();
+  if (t == 0) {
+    ptx::bulk_store(a.codes + (cs * (a.n_ctx_pad / TILE) + tile) * static_cast<size_t>(TILE * D), op, kTOp);
+    ptx::bulk_store_drain();
   }
 }
 
@@ -143,8 +242,6 @@ constexpr int kTRows = 128;
 constexpr int kTSoftmax = 256;                     // softmax threads (warps 0-7)
 constexpr int kTThreads = kTSoftmax + 32;          // + the control warp
 constexpr int kTCtl = kTSoftmax;                   // the thread that issues copies and MMAs
-constexpr int kTAtom = 128 * 128;                  // one 128-row K-atom (64 16-bit values per row)
-constexpr int kTOp = 2 * kTAtom;                   // one 128 x 128 16-bit operand (two K-atoms)
 constexpr float kLazyLog2 = 8.0f;
 constexpr uint32_t kIdescTT = ptx::idesc_f16_f32(128, 128);
 constexpr uint32_t kIdescBB = ptx::idesc_bf16_f32(128, 128);
@@ -164,11 +261,6 @@ struct PrefillTcSmem {
 };
 // kt and vt together hold the four projection operands (prologue, epilogue)
 static_assert(offsetof(PrefillTcSmem, vt) == offsetof(PrefillTcSmem, kt) + 2 * kTOp, "operand slots contiguous");
-
-// byte offset of element (row, k) of a 128-row K-major operand with the 128-byte swizzle
-__device__ __forceinline__ int sw128_off(int row, int k) {
-  return (k >> 6) * kTAtom + (row >> 3) * 1024 + (row & 7) * 128 + ((((k & 63) >> 3) ^ (row & 7)) << 4) + (k & 7) * 2;
-}
 
 __device__ __forceinline__ uint32_t pack_bf2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
   return static_cast<uint32_t>(__bfloat16_as_ushort(lo)) | (static_cast<uint32_t>(__bfloat16_as_ushort(hi)) << 16);
@@ -198,7 +290,7 @@ __device__ __forceinline__ void store_split_bf16(unsigned char* dst, const float
 __device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTSoftmax) : "memory"); }
 
 __global__ void __launch_bounds__(kTThreads, 1)
-    aatc_prefill_tc_kernel(const __grid_constant__ CUtensorMap tm, const PrefillArgs a) {
+    aatc_prefill_tc_kernel(const PrefillArgs a) {
   extern __shared__ unsigned char smraw[];
   PrefillTcSmem& sm =
       *reinterpret_cast<PrefillTcSmem*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
@@ -237,7 +329,6 @@ __global__ void __launch_bounds__(kTThreads, 1)
     ptx::mbar_init(&sm.bar_p, 1);
     sm.abort_flag = 0;
     ptx::fence_mbar_init();
-    ptx::prefetch_tmap(&tm);
   }
   if (warp == 0) {
     ptx::tmem_alloc(&sm.tmem, 512);
@@ -343,19 +434,17 @@ __global__ void __launch_bounds__(kTThreads, 1)
     // ---- control thread: TMA copies and MMAs.  Every wait below is on a phase that cannot be
     // overtaken: the next arrival on that barrier needs an action this thread takes later.
     if (lane == 0 && n_kv_tiles > 0) {
+      const __half* ck = a.codes + csk * a.n_ctx_pad * D;    // tiles of this head's keys, values: 32 KB operands
+      const __half* cv = a.codes + csv * a.n_ctx_pad * D;
       auto load_k = [&](int t) {
         const int buf = t & 1;
-        const int krow = static_cast<int>(csk * a.n_ctx_pad) + t * TILE;
         ptx::mbar_arrive_expect_tx(&sm.bar_k[buf], kTOp);
-        ptx::tma_load_2d(sm.kt[buf], &tm, &sm.bar_k[buf], 0, krow);
-        ptx::tma_load_2d(sm.kt[buf] + kTAtom, &tm, &sm.bar_k[buf], 64, krow);
+        ptx::bulk_load(sm.kt[buf], ck + static_cast<size_t>(t) * TILE * D, kTOp, &sm.bar_k[buf]);
       };
       auto load_v = [&](int t) {
         const int buf = t & 1;
-        const int vrow = static_cast<int>(csv * a.n_ctx_pad) + t * TILE;
         ptx::mbar_arrive_expect_tx(&sm.bar_v[buf], kTOp);
-        ptx::tma_load_2d(sm.vt[buf], &tm, &sm.bar_v[buf], 0, vrow);
-        ptx::tma_load_2d(sm.vt[buf] + kTAtom, &tm, &sm.bar_v[buf], 64, vrow);
+        ptx::bulk_load(sm.vt[buf], cv + static_cast<size_t>(t) * TILE * D, kTOp, &sm.bar_v[buf]);
       };
       auto issue_s = [&](int t) {                       // S = q'_hi . code_K + q'_lo . code_K, A from TMEM
         const uint32_t kt_a = ptx::smem_u32(sm.kt[t & 1]);
@@ -586,31 +675,6 @@ size_t prefill_workspace(int batch, int n_kv, int n_ctx) {
   return static_cast<size_t>(batch) * n_kv * 2 * pad * D * sizeof(__half);
 }
 
-cudaError_t launch_codes(const Plan& plan, int layer, const void* cache, int batch, int n_ctx, int max_tokens,
-                         void* ws, cudaStream_t st) {
-  const CacheGeom g = cache_geom(batch, plan.dims.n_kv_heads, max_tokens, plan.n_words);
-  PrefillArgs a{};
-  a.words = static_cast<const uint32_t*>(cache);
-  a.alpha = reinterpret_cast<const float*>(static_cast<const uint32_t*>(cache) + g.words_elems);
-  a.codes = static_cast<__half*>(ws);
-  a.f = plan.dev.f;
-  a.enc = plan.dev.enc;
-  a.lay = plan.dev.lay;
-  a.entry = plan.dev.entry;
-  a.chan_ent = plan.dev.chan_ent;
-  a.layer = layer;
-  a.n_kv = plan.dims.n_kv_heads;
-  a.n_ctx = n_ctx;
-  a.n_ctx_pad = (n_ctx + TILE - 1) / TILE * TILE;
-  a.n_tiles = g.n_tiles;
-  a.n_words = plan.n_words;
-  a.n_entries = plan.n_entries;
-  a.err = plan.dev.err;
-  if (plan.n_words > 32) return cudaErrorNotSupported;
-  aatc_prefill_codes_kernel<<<dim3(a.n_ctx_pad / TILE, a.n_kv * 2, batch), TILE, 0, st>>>(a);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_start, int n_q, const void* cache,
                            int batch, int n_ctx, int max_tokens, float* out, void* ws, cudaStream_t st) {
   const CacheGeom g = cache_geom(batch, plan.dims.n_kv_heads, max_tokens, plan.n_words);
@@ -625,8 +689,6 @@ cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_sta
   a.f = plan.dev.f;
   a.enc = plan.dev.enc;
   a.lay = plan.dev.lay;
-  a.entry = plan.dev.entry;
-  a.chan_ent = plan.dev.chan_ent;
   a.layer = layer;
   a.n_kv = plan.dims.n_kv_heads;
   a.n_q_heads = plan.dims.n_q_heads;
@@ -637,23 +699,21 @@ cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_sta
   a.n_ctx_pad = (n_ctx + TILE - 1) / TILE * TILE;
   a.n_tiles = g.n_tiles;
   a.n_words = plan.n_words;
-  a.n_entries = plan.n_entries;
   a.err = plan.dev.err;
   if (plan.n_words > 32) return cudaErrorNotSupported;
-  aatc_prefill_codes_kernel<<<dim3(a.n_ctx_pad / TILE, a.n_kv * 2, batch), TILE, 0, st>>>(a);
-  cudaError_t e = cudaGetLastError();
+  // one instantiation for plans with a channel wider than 8 bits (high bytes kept), one without
+  auto* codes = plan.max_bits > 8 ? aatc_prefill_codes_kernel<true> : aatc_prefill_codes_kernel<false>;
+  const size_t csm = kTOp + static_cast<size_t>(plan.n_words + 1) * TILE * 4;
+  cudaError_t e = ensure_smem_optin(reinterpret_cast<const void*>(codes), csm);
   if (e != cudaSuccess) return e;
-  // one 2D map over the whole codes workspace: rows of 128 f16 (a key token, or a value channel
-  // of a 128-token tile), box 64 x 128
-  alignas(64) unsigned char tmap[128];
-  e = make_tensor_map_2d(tmap, true, ws, D, static_cast<uint64_t>(batch) * a.n_kv * 2 * a.n_ctx_pad, D * 2, 64, TILE);
+  codes<<<dim3(a.n_ctx_pad / TILE, a.n_kv * 2, batch), TILE, csm, st>>>(a);
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t smem = sizeof(PrefillTcSmem) + 1024;
   e = ensure_smem_optin(reinterpret_cast<const void*>(aatc_prefill_tc_kernel), smem);
   if (e != cudaSuccess) return e;
   const int n_rows = n_q * a.group;
-  aatc_prefill_tc_kernel<<<dim3((n_rows + kTRows - 1) / kTRows, a.n_kv, batch), kTThreads, smem, st>>>(
-      *reinterpret_cast<const CUtensorMap*>(tmap), a);
+  aatc_prefill_tc_kernel<<<dim3((n_rows + kTRows - 1) / kTRows, a.n_kv, batch), kTThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 

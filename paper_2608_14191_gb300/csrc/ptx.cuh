@@ -78,6 +78,16 @@ __device__ __forceinline__ void bulk_load_hint(void* dst, const void* src, uint3
       "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
       : "memory");
 }
+// Plain bulk copy shared -> global (the caller has fenced its shared-memory writes for the async
+// proxy), and the wait until every bulk store of this thread has read its shared memory.
+__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(reinterpret_cast<uint64_t>(dst)),
+               "r"(smem_u32(src)), "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_store_drain() {
+  asm volatile("cp.async.bulk.commit_group;\n\tcp.async.bulk.wait_group.read 0;" ::: "memory");
+}
 // L2 policy: lines fetched under it are the first to be evicted.
 __device__ __forceinline__ uint64_t l2_policy_evict_first() {
   uint64_t p;
