@@ -221,46 +221,56 @@ __device__ __forceinline__ uint32_t pack_h2(float lo, float hi) {
 }
 
 // ---------------------------------------------------------------- tensor-core (tcgen05) attention
-// Per CTA 128 query rows (= TMEM lanes) of one (kv-head, sequence).  Warps 0-7 do the softmax:
-// warp w owns TMEM lanes 32 (w & 3) .. + 31 and the column half w >> 2 of every 128-column TMEM
-// block.  Warp 8 is the control warp: one thread issues every TMA copy and tensor-core MMA and
-// talks to the softmax warps through mbarriers only.
+// Per CTA 128 query rows (= TMEM lanes) of one (kv-head, sequence).  Warps 0-15 do the softmax:
+// warp w owns TMEM lanes 32 (w & 3) .. + 31 and column quarter w >> 2 of every 128-column TMEM
+// block.  Warp 16 issues every tensor-core MMA, one thread of warp 17 every copy; the roles talk
+// through mbarriers only.
 //   prologue  q' = (q U_K) f^K log2(e) / sqrt(128) on the tensor cores: q (bf16, exact) against
 //             U_K split into three bf16 parts (about 2^-25 relative), rows scaled to 2^14 and
 //             split into f16 hi / lo operands kept in TMEM (the A operand of the score MMA, so
 //             only the key tile is read from shared memory)
-//   per 128-token tile (TMA, 128-byte swizzle, key and value tiles double-buffered):
-//             S = q'_hi . code_K + q'_lo . code_K   tcgen05.mma M = N = 128, K = 128; the softmax
-//             keeps its scores in registers, so S of tile t + 1 is computed into the same TMEM
-//             columns as soon as every warp has read S(t)
-//             softmax from TMEM with the scores held in registers between the maximum and the
-//             exponent: s = S rs alpha^K (causal mask), lazy maximum (O rescaled only when a
-//             row's maximum grows by more than 2^8, so P' = 2^(s - m) alpha^V stays inside f16)
-//             P' stored to TMEM as f16 pairs: the A operand of O += P' . code_V^T
+//   per 128-token tile (key and value tiles in rings of three):
+//             S = q'_hi . code_K + q'_lo . code_K   tcgen05.mma M = N = 128, K = 128 into score
+//             buffer t & 1, one tile ahead of the softmax;
+//             softmax with the scores held in registers: x = S alpha^K (causal mask), the row
+//             maximum over the four quarters through shared memory and one barrier, lazy reference
+//             maximum (O rescaled only when a row's maximum grows by more than 2^8, so
+//             P' = 2^(s - m) alpha^V stays inside f16);
+//             P' as f16 pairs over the first half of the score buffer it came from: the A operand
+//             of O += P' . code_V^T.  S(t + 2), which reuses the buffer, is issued behind PV(t) and
+//             the MMAs run in issue order.
 //   epilogue  out = (f^V O / l) U_V^T on the tensor cores, both operands split hi / lo in bf16.
+// Bound by the softmax's latency: the tensor pipe needs ~1600 cycles a tile (24 MMAs of 64 and
+// more), a tile takes ~2600 (4 x 8192 x 28 heads: 2.5 ms, 3.2 ms before this split of the roles).
+// Sixteen warps, four a scheduler, hide more of it than eight; halving the MMAs, dropping the
+// exponentials or the copies changes nothing, dropping the reads of alpha saves a sixth (a column's
+// alpha is one shared-memory word for every row).
 constexpr int kTRows = 128;
-constexpr int kTSoftmax = 256;                     // softmax threads (warps 0-7)
-constexpr int kTThreads = kTSoftmax + 32;          // + the control warp
-constexpr int kTCtl = kTSoftmax;                   // the thread that issues copies and MMAs
+constexpr int kTSoftmax = 512;                     // softmax threads (warps 0-15)
+constexpr int kTThreads = kTSoftmax + 64;          // + the MMA warp and the copy warp
+constexpr int kTMma = kTSoftmax;                   // first thread of the warp that issues MMAs
+constexpr int kTCopy = kTSoftmax + 32;             // the thread that issues copies
 constexpr float kLazyLog2 = 8.0f;
 constexpr uint32_t kIdescTT = ptx::idesc_f16_f32(128, 128);
 constexpr uint32_t kIdescBB = ptx::idesc_bf16_f32(128, 128);
-constexpr uint32_t kColS = 0;                      // score buffer; projection results
-constexpr uint32_t kColO = 128;                    // O accumulator
-constexpr uint32_t kColP = 256;                    // two P' buffers (256, 320): 64 columns of f16 pairs
+constexpr int kTRing = 3;                          // key tiles, value tiles in flight
+constexpr uint32_t kColS = 0;                      // two score buffers (0, 128), P' over their first 64
+                                                   // columns; projection results (0)
+constexpr uint32_t kColO = 256;                    // O accumulator
 constexpr uint32_t kColQ = 384;                    // q' hi (384) and lo (448): A operands of the score MMA
 
 struct PrefillTcSmem {
-  alignas(1024) unsigned char kt[2][kTOp];         // key codes: K-atoms = channels, rows = tokens
-  alignas(1024) unsigned char vt[2][kTOp];         // value codes: K-atoms = tokens 0-63 | 64-127, rows = channels
-  float al[3][2][TILE];                            // alpha^K, alpha^V of three tiles
-  float xch[2][2][kTRows];                         // per-row partials of the two column halves (two slots)
-  uint64_t bar_k[2], bar_v[2], ofree[2], bar_s, sfree, pready, bar_p;
+  alignas(1024) unsigned char kt[kTRing][kTOp];    // key codes: K-atoms = channels, rows = tokens
+  alignas(1024) unsigned char vt[kTRing][kTOp];    // value codes: K-atoms = tokens 0-63 | 64-127, rows = channels
+  alignas(16) float al[kTRing][2][TILE];           // alpha^K, alpha^V of the tiles in the value ring
+  float xch[2][4][kTRows];                         // per-row partials of the column quarters (two slots)
+  uint64_t bar_k[kTRing], bar_v[kTRing], bar_a[kTRing], kfree[kTRing], vfree[kTRing], bar_s[2], pready[2], ofree[2],
+      bar_p;
   uint32_t tmem;
-  int abort_flag;
+  int abort_flag, never;
 };
 // kt and vt together hold the four projection operands (prologue, epilogue)
-static_assert(offsetof(PrefillTcSmem, vt) == offsetof(PrefillTcSmem, kt) + 2 * kTOp, "operand slots contiguous");
+static_assert(offsetof(PrefillTcSmem, vt) == offsetof(PrefillTcSmem, kt) + kTRing * kTOp, "operand slots contiguous");
 
 __device__ __forceinline__ uint32_t pack_bf2(__nv_bfloat16 lo, __nv_bfloat16 hi) {
   return static_cast<uint32_t>(__bfloat16_as_ushort(lo)) | (static_cast<uint32_t>(__bfloat16_as_ushort(hi)) << 16);
@@ -286,7 +296,8 @@ __device__ __forceinline__ void store_split_bf16(unsigned char* dst, const float
     if (p < parts) *reinterpret_cast<uint4*>(dst + p * kTOp) = make_uint4(w[p][0], w[p][1], w[p][2], w[p][3]);
 }
 
-// barrier among the softmax warps only
+// barriers among the softmax warps only, and among the four warps that share 32 rows
+__device__ __forceinline__ void row_sync(int wq) { asm volatile("bar.sync %0, 128;" ::"r"(2 + wq) : "memory"); }
 __device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTSoftmax) : "memory"); }
 
 __global__ void __launch_bounds__(kTThreads, 1)
@@ -298,6 +309,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
   const int rb = gridDim.x - 1 - blockIdx.x, head = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool softmax = tid < kTSoftmax;
+  const int wu = ptx::warp_uniform(warp);
   const int G = a.group, n_rows = a.n_q * G;
   const int sk = (a.layer * a.n_kv + head) * 2, sv = sk + 1;
   const size_t csk = (static_cast<size_t>(b) * a.n_kv + head) * 2, csv = csk + 1;
@@ -305,7 +317,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
   const int r_last = min(n_rows - 1, R0 + kTRows - 1) - R0;
   const int kv_end = min(a.n_ctx, a.q_start + (R0 + r_last) / G + 1);
   const int n_kv_tiles = (kv_end + TILE - 1) / TILE;
-  const int r = 32 * (warp & 3) + lane, half = (warp >> 2) & 1, hc = 64 * half;
+  const int r = 32 * (warp & 3) + lane, quarter = (warp >> 2) & 3, qc = 32 * quarter;
   const uint32_t lane_base = static_cast<uint32_t>(32 * (warp & 3)) << 16;
   const int R = R0 + r;
   unsigned char* const pj = sm.kt[0];              // projection operand i at pj + i * kTOp
@@ -317,17 +329,22 @@ __global__ void __launch_bounds__(kTThreads, 1)
     }
   };
 
-  if (tid == kTCtl) {
-    for (int i = 0; i < 2; ++i) {
+  if (tid == kTMma) {
+    for (int i = 0; i < kTRing; ++i) {
       ptx::mbar_init(&sm.bar_k[i], 1);
       ptx::mbar_init(&sm.bar_v[i], 1);
-      ptx::mbar_init(&sm.ofree[i], 1);          // PV of tiles i, i + 2, ... done
+      ptx::mbar_init(&sm.bar_a[i], 1);               // alpha of the value slot's tile
+      ptx::mbar_init(&sm.kfree[i], 1);               // the MMAs have read key slot i, value slot i
+      ptx::mbar_init(&sm.vfree[i], 1);
     }
-    ptx::mbar_init(&sm.bar_s, 1);                    // S(t) computed
-    ptx::mbar_init(&sm.sfree, kTSoftmax / 32);       // S(t) read out by every softmax warp
-    ptx::mbar_init(&sm.pready, kTSoftmax / 32);
+    for (int i = 0; i < 2; ++i) {
+      ptx::mbar_init(&sm.bar_s[i], 1);               // S of tiles i, i + 2, ... computed
+      ptx::mbar_init(&sm.pready[i], kTSoftmax / 32); // their P' written (one arrival per warp)
+      ptx::mbar_init(&sm.ofree[i], 1);               // their PV done
+    }
     ptx::mbar_init(&sm.bar_p, 1);
     sm.abort_flag = 0;
+    sm.never = 0;
     ptx::fence_mbar_init();
   }
   if (warp == 0) {
@@ -362,253 +379,261 @@ __global__ void __launch_bounds__(kTThreads, 1)
   ptx::tc_fence_after();
   const uint32_t tmem = sm.tmem;
   const uint32_t pj_a = ptx::smem_u32(pj);
-  if (tid == kTCtl) {
-#pragma unroll 1
+  if (wu == kTMma / 32) {
+    const uint32_t el = ptx::elect_one(), tm = ptx::warp_uniform(tmem);
+    const uint64_t ad = ptx::sdesc_kmajor_sw128(pj_a);
+#pragma unroll
     for (int part = 0; part < 3; ++part)
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk) {
         const uint32_t off = (kk >> 2) * kTAtom + (kk & 3) * 32;
-        ptx::umma_bf16(tmem + kColS, ptx::sdesc_kmajor_sw128(pj_a + off),
-                       ptx::sdesc_kmajor_sw128(pj_a + (1 + part) * kTOp + off), kIdescBB, (part | kk) ? 1u : 0u);
+        ptx::umma_bf16_w(tm + kColS, ad + (off >> 4), ad + (((1 + part) * kTOp + off) >> 4), kIdescBB,
+                         (part | kk) ? 1u : 0u, el);
       }
-    ptx::umma_commit(&sm.bar_p);
+    ptx::umma_commit_w(&sm.bar_p, el);
   }
   // ---- q' rows scaled to 2^14, f16 hi / lo into the score operands
   float rsr = 1.0f;
   if (softmax) {
     wait(&sm.bar_p, 0);
     ptx::tc_fence_after();
-    uint32_t q0[32], q1[32];
-    ptx::tmem_ld_32raw(tmem + lane_base + kColS + hc, q0);
-    ptx::tmem_ld_32raw(tmem + lane_base + kColS + hc + 32, q1);
+    uint32_t q0[32];
+    ptx::tmem_ld_32raw(tmem + lane_base + kColS + qc, q0);
     ptx::tmem_ld_wait();
     ptx::tmem_regs_ready(q0);
-    ptx::tmem_regs_ready(q1);
     const float sc = kPLog2e * 0.08838834764831845f;
-    const float* fk = a.f + sk * D + hc;
-    float x[64];
+    const float* fk = a.f + sk * D + qc;
+    float x[32];
     float m = 0.0f;
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
       x[i] = __uint_as_float(q0[i]) * fk[i] * sc;
-      x[32 + i] = __uint_as_float(q1[i]) * fk[32 + i] * sc;
-      m = fmaxf(m, fmaxf(fabsf(x[i]), fabsf(x[32 + i])));
+      m = fmaxf(m, fabsf(x[i]));
     }
-    sm.xch[0][half][r] = m;
+    sm.xch[0][quarter][r] = m;
     softmax_sync();
-    m = fmaxf(sm.xch[0][0][r], sm.xch[0][1][r]);
+    m = fmaxf(fmaxf(sm.xch[0][0][r], sm.xch[0][1][r]), fmaxf(sm.xch[0][2][r], sm.xch[0][3][r]));
     const float inv = m > 0.0f ? kPOpMax / m : 0.0f;
     rsr = m > 0.0f ? m / kPOpMax : 1.0f;             // > 0, so the mask's -inf survives the scaling
-    // this thread's 64 channels as 32 f16 pairs of hi and of lo: TMEM columns kColQ + 32 half ..
-    // (hi) and kColQ + 64 + 32 half .. (lo), row = lane
-    uint32_t hw[32], lw[32];
+    // this thread's 32 channels as 16 f16 pairs of hi and of lo: TMEM columns kColQ + 16 quarter ..
+    // (hi) and kColQ + 64 + 16 quarter .. (lo), row = lane
+    uint32_t hw[16], lw[16];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
+    for (int j = 0; j < 16; ++j) {
       const float y0 = x[2 * j] * inv, y1 = x[2 * j + 1] * inv;
       const __half2 h = __floats2half2_rn(y0, y1);
       const float2 hf = __half22float2(h);
       hw[j] = *reinterpret_cast<const uint32_t*>(&h);
       lw[j] = pack_h2(y0 - hf.x, y1 - hf.y);
     }
-    ptx::tmem_st32(tmem + lane_base + kColQ + 32 * half, hw);
-    ptx::tmem_st32(tmem + lane_base + kColQ + 64 + 32 * half, lw);
+    ptx::tmem_st16(tmem + lane_base + kColQ + 16 * quarter, hw);
+    ptx::tmem_st16(tmem + lane_base + kColQ + 64 + 16 * quarter, lw);
     ptx::tmem_wait_st();
-  }
-  // alpha^K / alpha^V of one tile: thread tid < 256 owns entry tid (K for tid < 128)
-  auto alpha_of = [&](int t) -> float {
-    const int tl = tid & (TILE - 1), tok = t * TILE + tl;
-    const size_t cs = tid < TILE ? csk : csv;
-    return tok < a.n_ctx ? a.alpha[cs * a.n_tiles * TILE + tok] : 0.0f;
-  };
-  float a_next = 0.0f;
-  if (softmax && n_kv_tiles > 0) {
-    sm.al[0][tid >> 7][tid & (TILE - 1)] = alpha_of(0);
-    if (n_kv_tiles > 1) a_next = alpha_of(1);
   }
   ptx::fence_proxy_async_smem();
   ptx::tc_fence_before();
-  __syncthreads();                                        // q' and alpha of tile 0 complete; slots, S free
+  __syncthreads();                                        // q' complete; operand slots, score buffers free
   ptx::tc_fence_after();
 
-  if (!softmax) {
-    // ---- control thread: TMA copies and MMAs.  Every wait below is on a phase that cannot be
-    // overtaken: the next arrival on that barrier needs an action this thread takes later.
-    if (lane == 0 && n_kv_tiles > 0) {
-      const __half* ck = a.codes + csk * a.n_ctx_pad * D;    // tiles of this head's keys, values: 32 KB operands
-      const __half* cv = a.codes + csv * a.n_ctx_pad * D;
-      auto load_k = [&](int t) {
-        const int buf = t & 1;
-        ptx::mbar_arrive_expect_tx(&sm.bar_k[buf], kTOp);
-        ptx::bulk_load(sm.kt[buf], ck + static_cast<size_t>(t) * TILE * D, kTOp, &sm.bar_k[buf]);
-      };
-      auto load_v = [&](int t) {
-        const int buf = t & 1;
-        ptx::mbar_arrive_expect_tx(&sm.bar_v[buf], kTOp);
-        ptx::bulk_load(sm.vt[buf], cv + static_cast<size_t>(t) * TILE * D, kTOp, &sm.bar_v[buf]);
-      };
-      auto issue_s = [&](int t) {                       // S = q'_hi . code_K + q'_lo . code_K, A from TMEM
-        const uint32_t kt_a = ptx::smem_u32(sm.kt[t & 1]);
-        ptx::tc_fence_after();
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint32_t off = (kk >> 2) * kTAtom + (kk & 3) * 32;
-          ptx::umma_f16_ta(tmem + kColS, tmem + kColQ + 8 * kk, ptx::sdesc_kmajor_sw128(kt_a + off), kIdescTT,
-                           kk > 0 ? 1u : 0u);
-        }
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint32_t off = (kk >> 2) * kTAtom + (kk & 3) * 32;
-          ptx::umma_f16_ta(tmem + kColS, tmem + kColQ + 64 + 8 * kk, ptx::sdesc_kmajor_sw128(kt_a + off), kIdescTT,
-                           1u);
-        }
-        ptx::umma_commit(&sm.bar_s);
-      };
-      load_k(0);
-      load_v(0);
-      if (n_kv_tiles > 1) {
-        load_k(1);
-        load_v(1);
-      }
-      wait(&sm.bar_k[0], 0);
-      issue_s(0);
-      for (int t = 0; t < n_kv_tiles; ++t) {
-        const int buf = t & 1;
-        if (t + 1 < n_kv_tiles) {
-          wait(&sm.sfree, t & 1);                       // S(t) read out: the S buffer and kt[buf] are free
-          if (t + 2 < n_kv_tiles) load_k(t + 2);
-          wait(&sm.bar_k[buf ^ 1], ((t + 1) >> 1) & 1);
-          issue_s(t + 1);
-          if (t >= 1) {                                 // PV(t - 1) has read vt[buf ^ 1]
-            wait(&sm.ofree[buf ^ 1], ((t - 1) >> 1) & 1);
-            load_v(t + 1);
-          }
-        }
-        wait(&sm.pready, t & 1);
-        wait(&sm.bar_v[buf], (t >> 1) & 1);
-        ptx::tc_fence_after();
-        const uint32_t vt_a = ptx::smem_u32(sm.vt[buf]);
-#pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const uint32_t off = (kk >> 2) * kTAtom + (kk & 3) * 32;
-          ptx::umma_f16_ta(tmem + kColO, tmem + kColP + 64 * buf + 8 * kk, ptx::sdesc_kmajor_sw128(vt_a + off),
-                           kIdescTT, (t > 0 || kk > 0) ? 1u : 0u);
-        }
-        ptx::umma_commit(&sm.ofree[buf]);
+  if (tid == kTCopy) {
+    // ---- copies: a slot is refilled once the MMAs that read it are complete
+    auto load = [&](int t, unsigned char* dst, const __half* src, uint64_t* bar, uint64_t* freed) {
+      const int st = t % kTRing;
+      if (t >= kTRing) wait(freed + st, (t / kTRing - 1) & 1);
+      if (*abort_flag) return false;
+      ptx::mbar_arrive_expect_tx(bar + st, kTOp);
+      ptx::bulk_load(dst + st * kTOp, src + static_cast<size_t>(t) * TILE * D, kTOp, bar + st);
+      return true;
+    };
+    const __half* ck = a.codes + csk * a.n_ctx_pad * D;    // tiles of this head's keys, values: 32 KB operands
+    const __half* cv = a.codes + csv * a.n_ctx_pad * D;
+    int nk = 0, nv = 0;                                   // tiles requested
+    while (nv < n_kv_tiles) {
+      if (!load(nk, sm.kt[0], ck, sm.bar_k, sm.kfree)) break;
+      ++nk;
+      if (!load(nv, sm.vt[0], cv, sm.bar_v, sm.vfree)) break;
+      // alpha of the tile, into the slot of a tile whose PV is complete (so its softmax is too);
+      // past the context it may hold any bits
+      const int st = nv % kTRing;
+      const size_t tok = static_cast<size_t>(nv) * TILE;
+      ptx::mbar_arrive_expect_tx(&sm.bar_a[st], 2 * TILE * 4);
+      ptx::bulk_load(sm.al[st][0], a.alpha + csk * a.n_tiles * TILE + tok, TILE * 4, &sm.bar_a[st]);
+      ptx::bulk_load(sm.al[st][1], a.alpha + csv * a.n_tiles * TILE + tok, TILE * 4, &sm.bar_a[st]);
+      ++nv;
+    }
+    if (*abort_flag) {                                    // a wait gave up: let the copies in flight land (bounded)
+      for (int t = max(0, nk - kTRing); t < nk; ++t)
+        ptx::mbar_wait_bounded(&sm.bar_k[t % kTRing], (t / kTRing) & 1, &sm.never);
+      for (int t = max(0, nv - kTRing); t < nv; ++t) {
+        ptx::mbar_wait_bounded(&sm.bar_v[t % kTRing], (t / kTRing) & 1, &sm.never);
+        ptx::mbar_wait_bounded(&sm.bar_a[t % kTRing], (t / kTRing) & 1, &sm.never);
       }
     }
-    __syncwarp();                                         // the control warp reconverges
-  } else {
+  } else if (wu == kTMma / 32 && n_kv_tiles > 0) {
+    // ---- MMAs, issued by the converged warp
+    const uint32_t el = ptx::elect_one();
+    const uint32_t tm = ptx::warp_uniform(tmem);
+    const uint64_t kdesc = ptx::sdesc_kmajor_sw128(ptx::smem_u32(sm.kt[0]));
+    const uint64_t vdesc = ptx::sdesc_kmajor_sw128(ptx::smem_u32(sm.vt[0]));
+    auto issue_s = [&](int t) {                           // S = q'_hi . code_K + q'_lo . code_K, A from TMEM
+      const int st = t % kTRing;
+      wait(&sm.bar_k[st], (t / kTRing) & 1);
+      const uint32_t ts = tm + kColS + 128 * (t & 1);
+      const uint64_t kd = kdesc + static_cast<uint64_t>(st * (kTOp >> 4));
+      ptx::tc_fence_after();
+#pragma unroll
+      for (int kk = 0; kk < 16; ++kk) {                   // hi, then lo
+        const uint32_t off = ((kk >> 2) & 1) * kTAtom + (kk & 3) * 32;
+        ptx::umma_f16_ta_w(ts, tm + kColQ + 8 * kk, kd + (off >> 4), kIdescTT, kk > 0 ? 1u : 0u, el);
+      }
+      ptx::umma_commit_w(&sm.bar_s[t & 1], el);
+      ptx::umma_commit_w(&sm.kfree[st], el);
+    };
+    issue_s(0);
+    if (n_kv_tiles > 1) issue_s(1);
+    for (int t = 0; t < n_kv_tiles; ++t) {
+      const int st = t % kTRing;
+      wait(&sm.bar_v[st], (t / kTRing) & 1);
+      wait(&sm.pready[t & 1], (t >> 1) & 1);
+      ptx::tc_fence_after();
+      const uint64_t vd = vdesc + static_cast<uint64_t>(st * (kTOp >> 4));
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        const uint32_t off = (kk >> 2) * kTAtom + (kk & 3) * 32;
+        ptx::umma_f16_ta_w(tm + kColO, tm + kColS + 128 * (t & 1) + 8 * kk, vd + (off >> 4), kIdescTT,
+                           (t > 0 || kk > 0) ? 1u : 0u, el);
+      }
+      ptx::umma_commit_w(&sm.ofree[t & 1], el);
+      ptx::umma_commit_w(&sm.vfree[st], el);
+      if (t + 2 < n_kv_tiles) issue_s(t + 2);
+    }
+  }
+  __syncwarp();                                           // the MMA and copy warps reconverge
+  if (softmax) {
     // ---- softmax warps
     const int pos = R < n_rows ? a.q_start + R / G : -1;   // padding rows attend to nothing
     const int last = min(pos, a.n_ctx - 1);               // last token this row attends to
-    float m_used = -INFINITY, l = 0.0f;
+    float m_used = -INFINITY;
+    uint64_t l2 = ptx::f2_pack(0.0f, 0.0f);
+    const uint64_t rs2 = ptx::f2_pack(rsr, rsr);
     for (int t = 0; t < n_kv_tiles; ++t) {
       const int buf = t & 1;
-      // alpha one tile ahead: store tile t + 1 (fetched last iteration), fetch tile t + 2
-      if (t + 1 < n_kv_tiles) sm.al[(t + 1) % 3][tid >> 7][tid & (TILE - 1)] = a_next;
-      if (t + 2 < n_kv_tiles) a_next = alpha_of(t + 2);
-      const float* akt = sm.al[t % 3][0] + hc;
-      const float* avt = sm.al[t % 3][1] + hc;
-      wait(&sm.bar_s, t & 1);
+      const float* akt = sm.al[t % kTRing][0] + qc;
+      const float* avt = sm.al[t % kTRing][1] + qc;
+      wait(&sm.bar_a[t % kTRing], (t / kTRing) & 1);
+      const uint32_t ts = tmem + lane_base + kColS + 128 * buf;
+      wait(&sm.bar_s[buf], (t >> 1) & 1);
       ptx::tc_fence_after();
-      // pass 1: x = S alpha^K over this thread's 64 tokens (masked), partial row maximum
-      const int lim = last - t * TILE - hc;                 // tokens i <= lim are attended
-      float x[64];
-      {
-        uint32_t s0[32], s1[32];
-        ptx::tmem_ld_32raw(tmem + lane_base + kColS + hc, s0);
-        ptx::tmem_ld_32raw(tmem + lane_base + kColS + hc + 32, s1);
-        ptx::tmem_ld_wait();
-        ptx::tmem_regs_ready(s0);
-        ptx::tmem_regs_ready(s1);
-        ptx::tc_fence_before();
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(&sm.sfree);         // this warp's part of S(t) read out
+      // x = S alpha^K over this thread's 32 tokens (masked), partial row maximum
+      uint32_t x[32];
+      ptx::tmem_ld_32raw(ts + qc, x);
+      const int lim = last - t * TILE - qc;                 // tokens i <= lim are attended
+      const bool full = __all_sync(0xffffffffu, lim >= 31);
+      ptx::tmem_ld_wait();
+      ptx::tmem_regs_ready(x);
+      float mt0 = -INFINITY, mt1 = -INFINITY;
+#pragma unroll
+      for (int i = 0; i < 32; i += 4) {
+        const float4 al = *reinterpret_cast<const float4*>(akt + i);
+        float y0, y1, y2, y3;
+        ptx::f2_unpack(ptx::f2_mul(ptx::f2_pack(__uint_as_float(x[i]), __uint_as_float(x[i + 1])), ptx::f2_pack(al.x, al.y)),
+                       y0, y1);
+        ptx::f2_unpack(ptx::f2_mul(ptx::f2_pack(__uint_as_float(x[i + 2]), __uint_as_float(x[i + 3])),
+                                   ptx::f2_pack(al.z, al.w)), y2, y3);
+        mt0 = ptx::fmax3(mt0, y0, y1);
+        mt1 = ptx::fmax3(mt1, y2, y3);
+        x[i] = __float_as_uint(y0);
+        x[i + 1] = __float_as_uint(y1);
+        x[i + 2] = __float_as_uint(y2);
+        x[i + 3] = __float_as_uint(y3);
+      }
+      if (!full) {
+        mt0 = mt1 = -INFINITY;
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
-          x[i] = __uint_as_float(s0[i]) * akt[i];
-          x[32 + i] = __uint_as_float(s1[i]) * akt[32 + i];
+          x[i] = i <= lim ? x[i] : 0xFF800000u;             // -inf
+          mt0 = fmaxf(mt0, __uint_as_float(x[i]));
         }
       }
-      const bool full = __all_sync(0xffffffffu, lim >= 63);
-      if (!full) {
-#pragma unroll
-        for (int i = 0; i < 64; ++i) x[i] = i <= lim ? x[i] : -INFINITY;
+      // alpha^V past the context may hold any bits, and would meet p = 0 below
+      // (the warps of a column quarter write the same zeros)
+      if ((t + 1) * TILE > a.n_ctx) {
+        if (t * TILE + qc + lane >= a.n_ctx) sm.al[t % kTRing][1][qc + lane] = 0.0f;
+        __syncwarp();
       }
-      float mt = -INFINITY;
-#pragma unroll
-      for (int i = 0; i < 64; ++i) mt = fmaxf(mt, x[i]);
-      sm.xch[buf][half][r] = mt;
-      softmax_sync();                                       // partial maxima exchanged
-      mt = fmaxf(sm.xch[buf][0][r], sm.xch[buf][1][r]) * rsr;
+      sm.xch[buf][quarter][r] = fmaxf(mt0, mt1);
+      ptx::tc_fence_before();
+      row_sync(warp & 3);                                   // partial maxima exchanged; S(t) of these rows read out
+      ptx::tc_fence_after();
+      const float mt = fmaxf(ptx::fmax3(sm.xch[buf][0][r], sm.xch[buf][1][r], sm.xch[buf][2][r]), sm.xch[buf][3][r]) * rsr;
       const bool need = mt > m_used + kLazyLog2;
-      if (__any_sync(0xffffffffu, need && t > 0)) {         // rescale this half of O once PV(t - 1) is done
-        wait(&sm.ofree[buf ^ 1], ((t - 1) >> 1) & 1);
-        ptx::tc_fence_after();
+      if (__any_sync(0xffffffffu, need)) {
         const float c = need ? (m_used == -INFINITY ? 0.0f : ex2(m_used - mt)) : 1.0f;
-#pragma unroll 1
-        for (int ch = 0; ch < 2; ++ch) {
+        if (t > 0) {                                        // rescale this quarter of O once PV(t - 1) is done
+          wait(&sm.ofree[buf ^ 1], ((t - 1) >> 1) & 1);
+          ptx::tc_fence_after();
           uint32_t o[32];
-          ptx::tmem_ld_32raw(tmem + lane_base + kColO + hc + 32 * ch, o);
+          ptx::tmem_ld_32raw(tmem + lane_base + kColO + qc, o);
           ptx::tmem_ld_wait();
           ptx::tmem_regs_ready(o);
 #pragma unroll
           for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * c);
-          ptx::tmem_st32(tmem + lane_base + kColO + hc + 32 * ch, o);
+          ptx::tmem_st32(tmem + lane_base + kColO + qc, o);
         }
+        l2 = ptx::f2_mul(l2, ptx::f2_pack(c, c));
+        if (need) m_used = mt;
       }
-      if (need) {
-        l = m_used == -INFINITY ? 0.0f : l * ex2(m_used - mt);
-        m_used = mt;
-      }
-      // pass 2: P' = 2^(x rs - m) alpha^V, f16 pairs into P' buffer `buf` once PV(t - 2) has read it
-      if (t >= 2) {
-        wait(&sm.ofree[buf], ((t - 2) >> 1) & 1);
-        ptx::tc_fence_after();
-      }
+      // P' = 2^(x rs - m) alpha^V as f16 pairs over the first half of the score buffer
       {
-        const float msub = m_used == -INFINITY ? 0.0f : m_used;
-        uint32_t pw[32];
+        const float msub = m_used == -INFINITY ? 0.0f : -m_used;
+        const uint64_t ms2 = ptx::f2_pack(msub, msub);
+        uint32_t pw[16];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float e0 = ex2(fmaf(x[2 * i], rsr, -msub)), e1 = ex2(fmaf(x[2 * i + 1], rsr, -msub));
-          l += e0 + e1;
-          pw[i] = pack_h2(e0 * avt[2 * i], e1 * avt[2 * i + 1]);
+        for (int i = 0; i < 32; i += 4) {
+          const float4 al = *reinterpret_cast<const float4*>(avt + i);
+          float e0, e1, e2, e3;
+          ptx::f2_unpack(ptx::f2_fma(ptx::f2_pack(__uint_as_float(x[i]), __uint_as_float(x[i + 1])), rs2, ms2), e0, e1);
+          ptx::f2_unpack(ptx::f2_fma(ptx::f2_pack(__uint_as_float(x[i + 2]), __uint_as_float(x[i + 3])), rs2, ms2), e2, e3);
+          const uint64_t p01 = ptx::f2_pack(ex2(e0), ex2(e1)), p23 = ptx::f2_pack(ex2(e2), ex2(e3));
+          l2 = ptx::f2_add(l2, ptx::f2_add(p01, p23));
+          ptx::f2_unpack(ptx::f2_mul(p01, ptx::f2_pack(al.x, al.y)), e0, e1);
+          ptx::f2_unpack(ptx::f2_mul(p23, ptx::f2_pack(al.z, al.w)), e2, e3);
+          pw[i / 2] = pack_h2(e0, e1);
+          pw[i / 2 + 1] = pack_h2(e2, e3);
         }
-        ptx::tmem_st32(tmem + lane_base + kColP + 64 * buf + 32 * half, pw);
+        ptx::tmem_st16(ts + 16 * quarter, pw);
       }
       ptx::tmem_wait_st();
       ptx::tc_fence_before();
       __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&sm.pready);
+      if (lane == 0) ptx::mbar_arrive(&sm.pready[buf]);
     }
     if (n_kv_tiles > 0) wait(&sm.ofree[(n_kv_tiles - 1) & 1], ((n_kv_tiles - 1) >> 1) & 1);
     ptx::tc_fence_after();
+    float l, lb;
+    ptx::f2_unpack(l2, l, lb);
+    softmax_sync();                                       // every warp is past its last maximum exchange
+    sm.xch[0][quarter][r] = l + lb;
+    softmax_sync();
+    const float lt = (sm.xch[0][0][r] + sm.xch[0][1][r]) + (sm.xch[0][2][r] + sm.xch[0][3][r]);
     // ---- o_hat = f^V O / l, hi / lo bf16 in slots 0 / 1; U_V (rows = dim, K = channel) hi / lo
     // in slots 2 / 3
-    softmax_sync();                                       // every warp is past its last maximum exchange
-    sm.xch[0][half][r] = l;
-    softmax_sync();
-    const float lt = sm.xch[0][0][r] + sm.xch[0][1][r];
     {
       const float il = lt > 0.0f ? 1.0f / lt : 0.0f;
-      uint32_t o0[32], o1[32];
-      ptx::tmem_ld_32raw(tmem + lane_base + kColO + hc, o0);
-      ptx::tmem_ld_32raw(tmem + lane_base + kColO + hc + 32, o1);
+      uint32_t o0[32];
+      ptx::tmem_ld_32raw(tmem + lane_base + kColO + qc, o0);
       ptx::tmem_ld_wait();
       ptx::tmem_regs_ready(o0);
-      ptx::tmem_regs_ready(o1);
-      const float* fv = a.f + sv * D + hc;
+      const float* fv = a.f + sv * D + qc;
 #pragma unroll
-      for (int g8 = 0; g8 < 8; ++g8) {
+      for (int g8 = 0; g8 < 4; ++g8) {
         float u[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
           const int i = 8 * g8 + j;
-          const float ov = __uint_as_float(i < 32 ? o0[i & 31] : o1[i & 31]);
-          u[j] = lt > 0.0f ? ov * il * fv[i] : 0.0f;
+          u[j] = lt > 0.0f ? __uint_as_float(o0[i]) * il * fv[i] : 0.0f;
         }
-        store_split_bf16(pj + sw128_off(r, hc + 8 * g8), u, 2);
+        store_split_bf16(pj + sw128_off(r, qc + 8 * g8), u, 2);
       }
     }
     const float* uv = a.u32 + static_cast<size_t>(sv) * D * D;
@@ -625,39 +650,36 @@ __global__ void __launch_bounds__(kTThreads, 1)
   __syncthreads();
   ptx::tc_fence_after();
   // ---- out = o_hat U_V^T = hi.hi + hi.lo + lo.hi
-  if (tid == kTCtl) {
-#pragma unroll 1
+  if (wu == kTMma / 32) {
+    const uint32_t el = ptx::elect_one(), tm = ptx::warp_uniform(tmem);
+    const uint64_t ad = ptx::sdesc_kmajor_sw128(pj_a);
+#pragma unroll
     for (int pr = 0; pr < 3; ++pr) {
       const uint32_t as = pr == 2 ? 1u : 0u, bs = pr == 1 ? 3u : 2u;
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk) {
         const uint32_t off = (kk >> 2) * kTAtom + (kk & 3) * 32;
-        ptx::umma_bf16(tmem + kColS, ptx::sdesc_kmajor_sw128(pj_a + as * kTOp + off),
-                       ptx::sdesc_kmajor_sw128(pj_a + bs * kTOp + off), kIdescBB, (pr | kk) ? 1u : 0u);
+        ptx::umma_bf16_w(tm + kColS, ad + ((as * kTOp + off) >> 4), ad + ((bs * kTOp + off) >> 4), kIdescBB,
+                         (pr | kk) ? 1u : 0u, el);
       }
     }
-    ptx::umma_commit(&sm.bar_p);
+    ptx::umma_commit_w(&sm.bar_p, el);
   }
   if (softmax) {
     wait(&sm.bar_p, 1);
     ptx::tc_fence_after();
-    uint32_t o0[32], o1[32];
-    ptx::tmem_ld_32raw(tmem + lane_base + kColS + hc, o0);
-    ptx::tmem_ld_32raw(tmem + lane_base + kColS + hc + 32, o1);
+    uint32_t o0[32];
+    ptx::tmem_ld_32raw(tmem + lane_base + kColS + qc, o0);
     ptx::tmem_ld_wait();
     ptx::tmem_regs_ready(o0);
-    ptx::tmem_regs_ready(o1);
     if (R < n_rows) {
       const int qi = R / G, qh2 = head * G + R % G;
       float4* dst =
-          reinterpret_cast<float4*>(a.out + ((static_cast<size_t>(b) * a.n_q + qi) * a.n_q_heads + qh2) * D + hc);
+          reinterpret_cast<float4*>(a.out + ((static_cast<size_t>(b) * a.n_q + qi) * a.n_q_heads + qh2) * D + qc);
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < 8; ++i)
         dst[i] = make_float4(__uint_as_float(o0[4 * i]), __uint_as_float(o0[4 * i + 1]), __uint_as_float(o0[4 * i + 2]),
                              __uint_as_float(o0[4 * i + 3]));
-        dst[8 + i] = make_float4(__uint_as_float(o1[4 * i]), __uint_as_float(o1[4 * i + 1]),
-                                 __uint_as_float(o1[4 * i + 2]), __uint_as_float(o1[4 * i + 3]));
-      }
     }
   }
   ptx::tc_fence_before();
