@@ -65,7 +65,9 @@ struct PlanDevice {
   const float* f;         // [S][128] f_c (0 for dropped)
   const StreamLayout* lay;  // [S]
   const short* entry;     // [S][n_entries]
-  const short* chan_ent;  // [S][128][8]: entries of each channel (-1 padded)
+  const short* chan_ent;  // [S][128][kChanEnt]: entries of each channel (-1 padded)
+  const short* ce8;       // [S][128][8]: the first eight of them (0 padded)
+  const float* cw8;       // [S][128][8]: 2^shift of those (0: none)
   int* err;               // [4] sticky device flags
 };
 
@@ -152,9 +154,9 @@ struct DecodeWs {
 DecodeWs decode_ws_layout(int batch, int n_q, int n_kv, int n_entries, int n_words, const DecodeSplit& sp);
 size_t decode_workspace(int batch, int n_q, int n_kv, int n_entries, int n_words, const DecodeSplit& sp);
 // The decode has two launch plans: the fused kernel (query rotation and split streaming in CTAs of
-// 8-16 warps, FUSED_CTAS_PER_SM per SM, one wave) then the merge kernel, for layers whose streams
-// share one of the record shapes it is built for; the query, split and merge kernels (about 5 CTAs
-// per SM, at most 16 tiles per split) for any other layer.  `range` = the packed tokens a call covers, counted from the first tile it reads.
+// 8-16 warps, FUSED_CTAS_PER_SM per SM, one wave) then the merge kernel, for layers whose records it
+// holds; the query, split and merge kernels (about 5 CTAs per SM, at most 16 tiles per split) for
+// any other layer.  `range` = the packed tokens a call covers, counted from the first tile it reads.
 constexpr int FUSED_CTAS_PER_SM = 1;
 DecodeSplit decode_split_for(int batch, int n_kv, int range, int num_sms, bool fused);
 // Workspace bytes that serve a decode of `range` tokens on any layer of the plan, whichever path

@@ -259,6 +259,8 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   const size_t o_lay = off;  off = align_up(off + static_cast<size_t>(S) * sizeof(StreamLayout), 256);
   const size_t o_ent = off;  off = align_up(off + static_cast<size_t>(S) * E * sizeof(short), 256);
   const size_t o_che = off;  off = align_up(off + SD * kChanEnt * sizeof(short), 256);
+  const size_t o_ce8 = off;  off = align_up(off + SD * 8 * sizeof(short), 256);
+  const size_t o_cw8 = off;  off = align_up(off + SD * 8 * sizeof(float), 256);
   const size_t o_err = off;  off = align_up(off + 16, 256);
   const size_t total = off;
   std::vector<unsigned char> host;
@@ -276,6 +278,8 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   auto* lay = reinterpret_cast<StreamLayout*>(host.data() + o_lay);
   auto* ent = reinterpret_cast<short*>(host.data() + o_ent);
   auto* che = reinterpret_cast<short*>(host.data() + o_che);
+  auto* ce8 = reinterpret_cast<short*>(host.data() + o_ce8);       // zeros where a channel has fewer
+  auto* cw8 = reinterpret_cast<float*>(host.data() + o_cw8);
   if (!basis) {
     // group tables, channels in slice-major order: j' = 128 s + c holds storage channel c g_h + s
     auto* gubf = reinterpret_cast<uint16_t*>(host.data() + o_gubf);
@@ -332,6 +336,11 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
     int fill[D] = {0};
     for (int e = 0; e < static_cast<int>(entries[s].size()); ++e) {
       const int c = entries[s][e] & 0xFF;
+      if (fill[c] < 8) {
+        const size_t i = (static_cast<size_t>(s) * D + c) * 8 + fill[c];
+        ce8[i] = static_cast<short>(e);
+        cw8[i] = std::ldexp(1.0f, entries[s][e] >> 8);
+      }
       if (fill[c] < kChanEnt) ce[c * kChanEnt + fill[c]++] = static_cast<short>(e);
     }
   }
@@ -367,6 +376,8 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   plan->dev.lay = reinterpret_cast<const StreamLayout*>(base + o_lay);
   plan->dev.entry = reinterpret_cast<const short*>(base + o_ent);
   plan->dev.chan_ent = reinterpret_cast<const short*>(base + o_che);
+  plan->dev.ce8 = reinterpret_cast<const short*>(base + o_ce8);
+  plan->dev.cw8 = reinterpret_cast<const float*>(base + o_cw8);
   plan->dev.err = reinterpret_cast<int*>(base + o_err);
   plan->group_heads = g_h;
   if (basis) {

@@ -2,11 +2,11 @@
 // uncompressed bf16 reference decode (Def. sdpa with one query row; Algorithm 1
 // "Reconstruct", "softmax", "Output" lines, computed without rebuilding the keys).
 //
-// Two launch plans, each a chain of programmatic dependents.  For layers whose key and value
-// streams share one record shape (every per-stream plan at 1.5, 2, 2.75 or 4 bits) two launches
-// per call: aatc_decode_fused_kernel (see there) rotates the queries and streams each split's
-// tiles through per-warp-group rings, then the merge kernel below.  Any other layer takes three
-// launches (flash-decoding split over the context):
+// Two launch plans, each a chain of programmatic dependents.  Two launches per call for nearly every
+// layer: aatc_decode_fused_kernel (see there) rotates the queries and streams each split's tiles
+// through per-warp-group rings, then the merge kernel below.  Layers whose records are too large for
+// it (fused_kernel_for), or have channels wider than 14 bits, take three launches (flash-decoding
+// split over the context):
 //   query    per (sequence, kv-head, query slot): q' = (U_K^T q) f^K log2(e)/sqrt(128) for the
 //            G query heads of the GQA group, the offset corrections C_g = sum_c q'_c 2^(b_c-1),
 //            and q' per record entry as f16 hi/lo tensor-core fragments (mma.sync m16n8k16);
@@ -82,6 +82,8 @@ struct DecodeArgs {
   const StreamLayout* lay; // plan: [S]
   const short* entry;      // plan: [S][n_entries]
   const short* chan_ent;   // plan: [S][128][kChanEnt] record entries of each channel (-1 padded)
+  const short* ce8;        // plan: [S][128][8] the first eight of them (0 padded)
+  const float* cw8;        // plan: [S][128][8] 2^shift of those (0: none)
   int* err;
   uint4* qfrag;            // workspace: score A fragments [batch][n_kv][ks_stride]
   float* qcorr;            // workspace: [batch][n_kv][16]: offset corrections C_g, score scales
@@ -92,6 +94,7 @@ struct DecodeArgs {
   const __nv_bfloat16* v_full;
   int n_full, full_cap;
   int n_stages;             // fused kernel: tile ring depth
+  int stage_bytes, nks_max; // fused kernel: bytes of a ring stage, score k-steps of the layer's widest streams
 };
 
 // 2^x with the hardware approximation (relative error ~2^-22; -inf -> 0)
@@ -620,6 +623,7 @@ __global__ void __launch_bounds__(kThreads)
       ssum[p] += __shfl_xor_sync(0xffffffffu, ssum[p], o);
     }
   float* oe = reinterpret_cast<float*>(ring);                  // [G][n_entries]: the ring is drained
+  if (nw_v == 0 && tid < G) oe[tid * a.n_entries] = 0.0f;      // an empty stream: its channels all point at entry 0
   if ((lane & 7) == 0)
 #pragma unroll
     for (int p = 0; p < NP; ++p) {
@@ -702,8 +706,9 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // ---------------------------------------------------------------- fused split + merge kernel
-// For plans whose key and value streams of the layer share one record shape (N2W D2 words, N1W D1
-// words).  CTA = (split, kv-head, sequence) with WG warp groups of four warps, one CTA per SM in
+// Record shape of a stream: D2 words, D1 words.  kExact: every key and value stream of the layer has
+// the shape (N2W, N1W); otherwise each stream has its own, the value streams' at most (N2W, N1W) (the
+// size of the accumulators, guarded tile by tile), the key streams' as they are (loops).  CTA = (split, kv-head, sequence) with WG warp groups of four warps, one CTA per SM in
 // one wave; the query rotation is folded in (every CTA rotates its group's queries itself, while
 // its first tiles are in flight) and the split's partial (o, m, l) per query goes to the
 // workspace for the merge kernel, which follows as this grid's programmatic dependent.  (A merge
@@ -720,7 +725,7 @@ __global__ void __launch_bounds__(kThreads)
 //    and p = 2^(s - m) below 2^72 whatever the scales, so the split needs no pass over its alpha
 //    values first.  m is only a reference point: o = sum P' code and l = sum p share it, and the
 //    merge rescales both alike.
-__host__ __device__ constexpr int fused_stage_bytes(int wu) { return 2 * wu * TILE * 4 + 2 * TILE * 4; }
+__host__ __device__ constexpr int fused_stage_bytes(int wk, int wv) { return (wk + wv) * TILE * 4 + 2 * TILE * 4; }
 // row pitch of the per-query entry sums in the epilogue: = 8 (mod 16), so the four queries of a
 // lane quad (rows t = 0..3) fall in distinct banks
 __host__ __device__ constexpr int fused_entry_pitch(int n_entries) { return ((n_entries + 7) / 8 * 8) | 8; }
@@ -728,7 +733,7 @@ constexpr float kPScale = 32.0f;            // P' < 2^9 times 2^5: f16 operands 
 
 struct FusedSmem {
   int bars, cnt, qf, qc, pf, cetab, cw8, ketab, fold, ring, total;
-  __host__ __device__ FusedSmem(int wu, int nks, int np, int wg, int n_entries, int n_stages) {
+  __host__ __device__ FusedSmem(int stage_bytes, int nks, int np, int wg, int n_entries, int n_stages) {
     const int gmax = 4 * np, warps = 4 * wg;
     int o = 0;
     bars = o;  o = align16(o + 8 * wg * n_stages);
@@ -736,13 +741,13 @@ struct FusedSmem {
     qf = o;    o += nks * np * 32 * 8;                        // query B fragments [ks][p][lane]
     qc = o;    o += 2 * MAX_GROUP * 4 + D * 4;                // C_g, score scales; value offsets 2^(b_c - 1)
     pf = o;    o += warps * 2 * np * 32 * 8;                  // P' B fragments [warp][ks][p][lane]
-    cetab = o; o += D * 8 * 2;                                // value channel -> its record entries (clamped)
+    cetab = o; o += D * 8 * 2;                                // value channel -> its record entries
     cw8 = o;   o += D * 8 * 4;                                // 2^shift of those entries (0: none)
     ketab = o; o = align16(o + n_entries * 2);                // key entry table
     fold = o;  o += ((2 + wg) * gmax * D + 2 * warps * gmax) * 4;   // q, q', partial q' [wg]; reductions
     o = (o + 127) & ~127;
     ring = o;
-    const int rings = wg * n_stages * fused_stage_bytes(wu);
+    const int rings = wg * n_stages * stage_bytes;
     // after the loop the rings hold each warp's (m, l, S', entry sums) per query, the warps'
     // factors 2^(m_w - M), the totals (M, l, S') and the entry sums over the warps
     const int nep = fused_entry_pitch(n_entries);
@@ -751,19 +756,20 @@ struct FusedSmem {
   }
 };
 
-template <int N2W, int N1W, int NP, int WG>
-__global__ void __launch_bounds__(128 * WG, 1)
-    aatc_decode_fused_kernel(const DecodeArgs a) {
-  constexpr int WU = N2W + N1W;                  // record words the streams use
-  constexpr int NKS = N2W + 2 * N1W;             // score k16-steps
+struct FusedShared {
+  uint64_t tab;             // table copies
+  int abort, never, issued[4];
+};
+
+template <int N2W, int N1W, int NP, int WG, bool kExact>
+__device__ __forceinline__ void decode_fused(const DecodeArgs& a, FusedShared& fs) {
   constexpr int NJ = N2W + 2 * N1W;              // value M-tiles (16 record entries each)
   constexpr int GMAX = 4 * NP;
   constexpr int NW = 4 * WG;                     // warps
   constexpr int NT = 32 * NW;                    // threads
-  constexpr uint32_t kTileWords = WU * TILE;
-  constexpr uint32_t kStage = fused_stage_bytes(WU);
   extern __shared__ __align__(128) unsigned char smb[];
-  __shared__ int s_abort, s_never, s_issued[WG];
+  int &s_abort = fs.abort, &s_never = fs.never, *const s_issued = fs.issued;
+  uint64_t& s_tab = fs.tab;
   int item = blockIdx.x;
   if (a.cta_per_sm > 0) item = (item % a.num_sms) * a.cta_per_sm + item / a.num_sms;
   const int split = item % a.n_splits, head = (item / a.n_splits) % a.n_kv, b = item / (a.n_splits * a.n_kv);
@@ -773,7 +779,13 @@ __global__ void __launch_bounds__(128 * WG, 1)
   const int G = a.group;
   const int NS = a.n_stages;
   const int sk = (a.layer * a.n_kv + head) * 2, sv = sk + 1;
-  const FusedSmem L(WU, NKS, NP, WG, a.n_entries, NS);
+  const StreamLayout lk = a.lay[sk];
+  const int n2k = kExact ? N2W : lk.n2 >> 4, n1k = kExact ? N1W : (lk.n1 + 31) >> 5;          // key record words
+  const int n2v = kExact ? N2W : a.lay[sv].n2 >> 4, n1v = kExact ? N1W : (a.lay[sv].n1 + 31) >> 5;   // value's
+  const int NKS = n2k + 2 * n1k;                 // score k16-steps
+  const uint32_t kWords = (n2k + n1k) * TILE, vWords = (n2v + n1v) * TILE;       // of one tile
+  const uint32_t kStage = kExact ? fused_stage_bytes(N2W + N1W, N2W + N1W) : a.stage_bytes;
+  const FusedSmem L(kStage, a.nks_max, NP, WG, a.n_entries, NS);
   uint64_t* full = reinterpret_cast<uint64_t*>(smb + L.bars) + wg * NS;   // this group's ring barriers
   int* cnt = reinterpret_cast<int*>(smb + L.cnt) + wg * NS;
   const uint2* qf = reinterpret_cast<const uint2*>(smb + L.qf);
@@ -804,11 +816,11 @@ __global__ void __launch_bounds__(128 * WG, 1)
     const size_t ta = static_cast<size_t>(tile) * TILE;
     // the cache is read once per call: evict-first keeps the plan tables in L2
     const uint64_t pol = ptx::l2_policy_evict_first();
-    ptx::mbar_arrive_expect_tx(full + s, kStage);
-    ptx::bulk_load_hint(st, kwords + tw, kTileWords * 4, full + s, pol);
-    ptx::bulk_load_hint(st + kTileWords * 4, vwords + tw, kTileWords * 4, full + s, pol);
-    ptx::bulk_load_hint(st + 2 * kTileWords * 4, kalpha + ta, TILE * 4, full + s, pol);
-    ptx::bulk_load_hint(st + 2 * kTileWords * 4 + TILE * 4, valpha + ta, TILE * 4, full + s, pol);
+    ptx::mbar_arrive_expect_tx(full + s, 4 * (kWords + vWords + 2 * TILE));
+    if (kExact || kWords) ptx::bulk_load_hint(st, kwords + tw, kWords * 4, full + s, pol);
+    if (kExact || vWords) ptx::bulk_load_hint(st + kWords * 4, vwords + tw, vWords * 4, full + s, pol);
+    ptx::bulk_load_hint(st + (kWords + vWords) * 4, kalpha + ta, TILE * 4, full + s, pol);
+    ptx::bulk_load_hint(st + (kWords + vWords + TILE) * 4, valpha + ta, TILE * 4, full + s, pol);
     s_issued[wg] = j + 1;
   };
   const bool leader = (tid & 127) == 0;          // thread 0 of a warp group
@@ -821,18 +833,17 @@ __global__ void __launch_bounds__(128 * WG, 1)
     s_abort = 0;
     s_never = 0;
   }
-  // plan constants (never written by a kernel): the streams' entry tables, key channel constants
-  // (the first 8 entries of each channel: all of them for widths up to 8, the only plans this
-  // kernel is launched for)
-  for (int i = tid; i < D * 8; i += NT) {
-    const int ce = a.chan_ent[(static_cast<size_t>(sv) * D + (i >> 3)) * kChanEnt + (i & 7)];
-    const int e = min(max(ce, 0), a.n_entries - 1);
-    reinterpret_cast<short*>(smb + L.cetab)[i] = static_cast<short>(e);
-    reinterpret_cast<float*>(smb + L.cw8)[i] =
-        ce >= 0 ? pow2i((a.entry[static_cast<size_t>(sv) * a.n_entries + e] >> 8) & 15) : 0.0f;
+  // plan constants (never written by a kernel): the value stream's entries per channel (the first 8:
+  // all of them for widths up to 14, the only plans this kernel is launched for), the key stream's
+  // entry table; key channel constants
+  if (tid == 0) {
+    ptx::mbar_init(&s_tab, 1);
+    ptx::fence_mbar_init();
+    ptx::mbar_arrive_expect_tx(&s_tab, D * 8 * 6 + a.n_entries * 2);
+    ptx::bulk_load(smb + L.cetab, a.ce8 + static_cast<size_t>(sv) * D * 8, D * 8 * 2, &s_tab);
+    ptx::bulk_load(smb + L.cw8, a.cw8 + static_cast<size_t>(sv) * D * 8, D * 8 * 4, &s_tab);
+    ptx::bulk_load(smb + L.ketab, a.entry + static_cast<size_t>(sk) * a.n_entries, a.n_entries * 2, &s_tab);
   }
-  for (int i = tid; i < a.n_entries; i += NT)
-    reinterpret_cast<short*>(smb + L.ketab)[i] = a.entry[static_cast<size_t>(sk) * a.n_entries + i];
   const int c = tid & (D - 1), part = tid >> 7;                 // channel, part of the fold (WG parts)
   // U_K rows of this thread's part of the fold: plan constants, requested before the wait
   constexpr int DR = D / WG, RR = DR < 64 ? DR : 64;
@@ -843,7 +854,6 @@ __global__ void __launch_bounds__(128 * WG, 1)
   const float fk = a.f[sk * D + c];
   const float offk = a.enc[sk * D + c].off;                     // 2^(b_c - 1), 0 if b_c = 0
   if (tid < D) reinterpret_cast<float*>(smb + L.qc)[2 * MAX_GROUP + tid] = a.enc[sv * D + tid].off;
-  const StreamLayout lk = a.lay[sk];
   if (tid < WG * NS) reinterpret_cast<int*>(smb + L.cnt)[tid] = 0;
   // everything below may read what the preceding grid in the stream wrote (cache, q, workspace)
   ptx::grid_dependency_wait();
@@ -908,6 +918,10 @@ __global__ void __launch_bounds__(128 * WG, 1)
     }
   }
   __syncthreads();
+  if (!ptx::mbar_wait_sleep(&s_tab, 0, &s_never, 20)) {          // (its own limit: nothing else stops this wait)
+    s_abort = 1;
+    atomicOr(a.err, 2);
+  }
   {
     float* qcw = reinterpret_cast<float*>(smb + L.qc);
     if (tid < GMAX) {
@@ -922,7 +936,7 @@ __global__ void __launch_bounds__(128 * WG, 1)
       qcw[MAX_GROUP + q] = q < G && m > 0.0f ? m * (kDigitScale / kOpMax) : 0.0f;   // raw sum -> sum q' u
     }
     // lane t of k-step ks holds fields (k 2t, 2t+1, 2t+8, 2t+9) = D2 (t, t+8, t+4, t+12) of word
-    // ks, or D1 bits (t, t+16, t+4, t+20) + 8 hs of word u for k-step ks = N2W + 2u + hs; the
+    // ks, or D1 bits (t, t+16, t+4, t+20) + 8 hs of word u for k-step ks = n2k + 2u + hs; the
     // split loop masks them in place (times 4^t, or 2^t and 2^(t+4)), the fragments divide it out
     uint2* qfw = reinterpret_cast<uint2*>(smb + L.qf);
     for (int i = tid; i < NKS * 4 * GMAX; i += NT) {
@@ -933,13 +947,13 @@ __global__ void __launch_bounds__(128 * WG, 1)
       const float invq = mq > 0.0f ? kOpMax / mq : 0.0f;
       int f[4], base, lim;
       float s01, s89;
-      if (ks < N2W) {
+      if (ks < n2k) {
         f[0] = tt; f[1] = tt + 8; f[2] = tt + 4; f[3] = tt + 12;
         base = 16 * ks;
         lim = 16;
         s01 = s89 = pow2i(-2 * tt);
       } else {
-        const int u = (ks - N2W) >> 1, sh = 8 * ((ks - N2W) & 1);
+        const int u = (ks - n2k) >> 1, sh = 8 * ((ks - n2k) & 1);
         f[0] = tt + sh; f[1] = tt + sh + 16; f[2] = tt + 4 + sh; f[3] = tt + 4 + sh + 16;
         base = lk.n2 + 32 * u;
         lim = min(32, lk.n1 - 32 * u);
@@ -1008,8 +1022,8 @@ __global__ void __launch_bounds__(128 * WG, 1)
     const int ti = wg + WG * j;                  // tile of the split
     const unsigned char* st = ring + s * kStage;
     const uint32_t* kt = reinterpret_cast<const uint32_t*>(st);
-    const uint32_t* vt = kt + kTileWords;
-    const float* ak = reinterpret_cast<const float*>(vt + kTileWords);
+    const uint32_t* vt = kt + kWords;
+    const float* ak = reinterpret_cast<const float*>(vt + vWords);
     const float* av = ak + TILE;
     // ---- scores of the warp's 32 tokens: M-tile 0 rows (g, g + 8) = tokens 4g, 4g + 1, M-tile 1
     // tokens 4g + 2, 4g + 3; N = 8 columns of query group p (hi, lo of queries 4p .. 4p + 3)
@@ -1021,8 +1035,8 @@ __global__ void __launch_bounds__(128 * WG, 1)
 #pragma unroll
         for (int z = 0; z < 4; ++z) kacc[m][p][z] = 0.0f;
     const uint4* kp = reinterpret_cast<const uint4*>(kt + tq);
-#pragma unroll
-    for (int ks = 0; ks < N2W; ++ks) {
+#pragma unroll(kExact ? N2W : 4)
+    for (int ks = 0; ks < n2k; ++ks) {
       const uint4 x = kp[ks * (TILE / 4)];
 #pragma unroll
       for (int p = 0; p < NP; ++p) {
@@ -1031,15 +1045,15 @@ __global__ void __launch_bounds__(128 * WG, 1)
         mma_f16(kacc[1][p], make_uint4(x.z & km2, x.w & km2, (x.z >> 8) & km2, (x.w >> 8) & km2), bf.x, bf.y);
       }
     }
-#pragma unroll
-    for (int u = 0; u < N1W; ++u) {
-      const uint4 x = kp[(N2W + u) * (TILE / 4)];
+#pragma unroll(kExact ? N1W : 2)
+    for (int u = 0; u < n1k; ++u) {
+      const uint4 x = kp[(n2k + u) * (TILE / 4)];
 #pragma unroll
       for (int hs = 0; hs < 2; ++hs) {
         const uint4 y = hs ? make_uint4(x.x >> 8, x.y >> 8, x.z >> 8, x.w >> 8) : x;
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-          const uint2 bf = qf[((N2W + 2 * u + hs) * NP + p) * 32 + lane];
+          const uint2 bf = qf[((n2k + 2 * u + hs) * NP + p) * 32 + lane];
           mma_f16(kacc[0][p], make_uint4(y.x & km1a, y.y & km1a, y.x & km1b, y.y & km1b), bf.x, bf.y);
           mma_f16(kacc[1][p], make_uint4(y.z & km1a, y.w & km1a, y.z & km1b, y.w & km1b), bf.x, bf.y);
         }
@@ -1125,6 +1139,7 @@ __global__ void __launch_bounds__(128 * WG, 1)
       const uint32_t* vq = vt + 4 * (8 * wq + 4 * kv + t);
 #pragma unroll
       for (int jw = 0; jw < N2W; ++jw) {
+        if (!kExact && jw >= n2v) break;
         const uint2 xx = *reinterpret_cast<const uint2*>(vq + jw * TILE + d2off);
         const uint4 af = make_uint4(xx.x & vm2, xx.y & vm2, (xx.x >> 8) & vm2, (xx.y >> 8) & vm2);
 #pragma unroll
@@ -1132,7 +1147,8 @@ __global__ void __launch_bounds__(128 * WG, 1)
       }
 #pragma unroll
       for (int u = 0; u < N1W; ++u) {
-        const uint4 s4 = *reinterpret_cast<const uint4*>(vq + (N2W + u) * TILE);
+        if (!kExact && u >= n1v) break;
+        const uint4 s4 = *reinterpret_cast<const uint4*>(vq + (n2v + u) * TILE);
         const uint4 afa = make_uint4(s4.x & vm1, s4.z & vm1, (s4.x >> 8) & vm1, (s4.z >> 8) & vm1);  // fields 0..15
         const uint4 afb = make_uint4(s4.y & vm1, s4.w & vm1, (s4.y >> 8) & vm1, (s4.w >> 8) & vm1);  // 16..31
 #pragma unroll
@@ -1162,6 +1178,7 @@ __global__ void __launch_bounds__(128 * WG, 1)
   __syncthreads();
   if (s_abort) {
     // a wait gave up: let every copy still in flight land (bounded) before leaving
+    if (tid == 0) ptx::mbar_wait_sleep(&s_tab, 0, &s_never, 20);
     if (leader)
       for (int j = max(0, s_issued[wg] - NS); j < s_issued[wg]; ++j)
         ptx::mbar_wait_sleep(full + j % NS, (j / NS) & 1, &s_never, 20);
@@ -1191,16 +1208,21 @@ __global__ void __launch_bounds__(128 * WG, 1)
   {
     // lane (g, t) holds entry rows g (c0 + c1) and g + 8 (c2 + c3) of every M-tile for query
     // 4p + t; raw sums times 2^24 / (row scale) / 2^5 = sum P' digit
+    if (!kExact && n2v + n1v == 0 && g == 0)       // an empty stream: its channels all point at entry 0
+#pragma unroll
+      for (int p = 0; p < NP; ++p) wE[(4 * p + t) * NEP] = 0.0f;
 #pragma unroll
     for (int jj = 0; jj < NJ; ++jj) {
       int e;
       float sc;
       if (jj < N2W) {
+        if (!kExact && jj >= n2v) continue;
         e = 16 * jj + g;
         sc = pow2i(19 - 2 * (g & 3));
       } else {
         const int u = (jj - N2W) >> 1, half = (jj - N2W) & 1;
-        e = 16 * N2W + 32 * u + 16 * half + g;
+        if (!kExact && u >= n1v) continue;
+        e = 16 * n2v + 32 * u + 16 * half + g;
         sc = pow2i(19 - g);
       }
 #pragma unroll
@@ -1283,6 +1305,34 @@ __global__ void __launch_bounds__(128 * WG, 1)
       }
     }
   }
+}
+
+// One record shape for the whole layer.
+template <int N2W, int N1W, int NP, int WG>
+__global__ void __launch_bounds__(128 * WG, 1) aatc_decode_fused_kernel(const DecodeArgs a) {
+  __shared__ FusedShared fs;
+  decode_fused<N2W, N1W, NP, WG, true>(a, fs);
+}
+// Streams that differ: each CTA takes the smallest value record its stream fits (kAccTiles value tiles
+// at most: 128 registers a thread hold no more accumulators beside the loop's operands).
+constexpr int kAccTiles = 21;
+template <int NP, int WG>
+__global__ void __launch_bounds__(128 * WG, 1) aatc_decode_fused_mixed_kernel(const DecodeArgs a) {
+  __shared__ FusedShared fs;
+  int item = blockIdx.x;
+  if (a.cta_per_sm > 0) item = (item % a.num_sms) * a.cta_per_sm + item / a.num_sms;
+  const StreamLayout& lv = a.lay[(a.layer * a.n_kv + (item / a.n_splits) % a.n_kv) * 2 + 1];
+  const int n2v = lv.n2 >> 4, n1v = (lv.n1 + 31) >> 5;
+  if (n2v <= 8 && n1v <= 3) decode_fused<8, 3, NP, WG, false>(a, fs);
+  else if (n1v <= 2) decode_fused<kAccTiles - 4, 2, NP, WG, false>(a, fs);
+  else if (n1v <= 3) decode_fused<kAccTiles - 6, 3, NP, WG, false>(a, fs);
+  else if (n1v <= 4) decode_fused<kAccTiles - 8, 4, NP, WG, false>(a, fs);
+  else decode_fused<kAccTiles - 10, 5, NP, WG, false>(a, fs);
+}
+// Records beyond that (up to four query heads per kv-head): half the warps, twice the registers.
+__global__ void __launch_bounds__(256, 1) aatc_decode_fused_large_kernel(const DecodeArgs a) {
+  __shared__ FusedShared fs;
+  decode_fused<32, 5, 1, 2, false>(a, fs);
 }
 
 // Merge of the splits of one (sequence, query head): M = max_s m_s, w_s = 2^(m_s - M),
@@ -1740,39 +1790,62 @@ cudaError_t launch_bf16_split(const Bf16Args& a, int batch, cudaStream_t st) {
 
 }  // namespace
 
-// Record shape shared by every key and value stream of `layer` (D2 words, D1 words), or false.
-static bool layer_shape(const Plan& plan, int layer, int* n2w, int* n1w) {
-  const int hk = plan.dims.n_kv_heads;
-  for (int s = 0; s < 2 * hk; ++s) {
-    const StreamLayout& l = plan.layout[layer * 2 * hk + s];
-    const int a = l.n2 / 16, b = (l.n1 + 31) / 32;
-    if (s == 0) {
-      *n2w = a;
-      *n1w = b;
-    } else if (a != *n2w || b != *n1w) {
-      return false;
+// Record shapes (D2 words, D1 words) of one layer's streams.
+struct LayerShape {
+  bool same = true;               // every key and value stream has the shape (n2v, n1v)
+  bool mixed = true;              // every value stream fits the mixed kernel's accumulators
+  int n2v = 0, n1v = 0;           // largest over the value streams
+  int nks = 0;                    // most score k-steps of a key stream
+  int stage = 0;                  // bytes of the largest tile stage (keys, values, alpha)
+};
+static LayerShape layer_shape(const Plan& plan, int layer) {
+  LayerShape r;
+  const StreamLayout* l = plan.layout.data() + static_cast<size_t>(layer) * 2 * plan.dims.n_kv_heads;
+  for (int h = 0; h < plan.dims.n_kv_heads; ++h) {
+    const int n2k = l[2 * h].n2 / 16, n1k = (l[2 * h].n1 + 31) / 32;
+    const int n2v = l[2 * h + 1].n2 / 16, n1v = (l[2 * h + 1].n1 + 31) / 32;
+    if (h == 0) {
+      r.n2v = n2v;
+      r.n1v = n1v;
     }
+    r.same = r.same && n2k == r.n2v && n1k == r.n1v && n2v == r.n2v && n1v == r.n1v;
+    r.mixed = r.mixed && n2v + 2 * std::max(n1v, 2) <= kAccTiles && n1v <= 5;
+    r.n2v = std::max(r.n2v, n2v);
+    r.n1v = std::max(r.n1v, n1v);
+    r.nks = std::max(r.nks, n2k + 2 * n1k);
+    r.stage = std::max(r.stage, fused_stage_bytes(n2k + n1k, n2v + n1v));
   }
-  return true;
+  return r;
 }
 
 using FusedKernel = void (*)(const DecodeArgs);
+struct FusedChoice {
+  FusedKernel kernel = nullptr;
+  int groups = 0;                 // warp groups per CTA
+};
 
-// The record shapes the fused kernel is built for: (D2 words, D1 words) of the per-stream plans at
-// 1.5, 2, 2.75 and 4 bits per channel.
-// Warp groups per CTA (one CTA per SM): four for up to four query heads per kv-head (16 warps, at
-// most 128 registers), two for five to eight (twice the value accumulators).
+// The fused kernel for a layer.  Warp groups per CTA (one CTA per SM): four for up to four query heads
+// per kv-head (16 warps, at most 128 registers), two for five to eight (twice the value accumulators)
+// and for records past kAccTiles value tiles.  The exact shapes are those of the per-stream plans at
+// 1.5, 2, 2.75 and 4 bits per channel.  Streams that differ take the mixed kernel once every SM has
+// some four tiles (`tiles` = 128-token tiles of all sequences and kv-heads): its CTAs each rotate the
+// queries and choose their code, which a few tiles do not pay for (two layers of 152 tiles: 22.0 us
+// against 19.9 of the three launches; 960 tiles: 19.9 against 24.7; 1256 tiles, four kv-head widths
+// apart: 22.0 against 26.7 a layer).  Records beyond the last (more than 32 + 2 x 5 value tiles, or
+// kAccTiles with more than four query heads per kv-head): the query / split / merge launches.
 template <int NP>
-constexpr int fused_groups() { return NP == 1 ? 4 : 2; }
-
-template <int NP>
-static FusedKernel fused_kernel_for(int n2w, int n1w) {
-  constexpr int WG = fused_groups<NP>();
-  if (n2w == 9 && n1w == 2) return aatc_decode_fused_kernel<9, 2, NP, WG>;
-  if (n2w == 3 && n1w == 3) return aatc_decode_fused_kernel<3, 3, NP, WG>;
-  if (n2w == 5 && n1w == 3) return aatc_decode_fused_kernel<5, 3, NP, WG>;
-  if (n2w == 13 && n1w == 3) return aatc_decode_fused_kernel<13, 3, NP, WG>;
-  return nullptr;
+static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, int num_sms) {
+  constexpr int WG = NP == 1 ? 4 : 2;
+  if (sh.same) {
+    if (sh.n2v == 9 && sh.n1v == 2) return {aatc_decode_fused_kernel<9, 2, NP, WG>, WG};
+    if (sh.n2v == 3 && sh.n1v == 3) return {aatc_decode_fused_kernel<3, 3, NP, WG>, WG};
+    if (sh.n2v == 5 && sh.n1v == 3) return {aatc_decode_fused_kernel<5, 3, NP, WG>, WG};
+    if (sh.n2v == 13 && sh.n1v == 3) return {aatc_decode_fused_kernel<13, 3, NP, WG>, WG};
+  }
+  if (tiles < 4L * num_sms) return {};
+  if (sh.mixed) return {aatc_decode_fused_mixed_kernel<NP, WG>, WG};
+  if (NP == 1 && sh.n2v <= 32 && sh.n1v <= 5) return {aatc_decode_fused_large_kernel, 2};
+  return {};
 }
 
 cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void* cache, int batch, int n_ctx,
@@ -1791,6 +1864,8 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
   a.lay = plan.dev.lay;
   a.entry = plan.dev.entry;
   a.chan_ent = plan.dev.chan_ent;
+  a.ce8 = plan.dev.ce8;
+  a.cw8 = plan.dev.cw8;
   a.err = plan.dev.err;
   a.layer = layer;
   a.n_kv = plan.dims.n_kv_heads;
@@ -1806,14 +1881,28 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
   a.n_full = extra.n_full;
   a.full_cap = extra.full_cap;
   const int np = (a.group + 3) / 4;
-  // the fused kernel: a packed range and one record shape (uncompressed tokens, if any, join in
-  // the merge kernel)
-  int n2w = 0, n1w = 0;
-  FusedKernel fk = nullptr;
-  if (extra.t_first < n_ctx && plan.max_bits <= 8 && layer_shape(plan, layer, &n2w, &n1w))
-    fk = np == 1 ? fused_kernel_for<1>(n2w, n1w) : fused_kernel_for<2>(n2w, n1w);
+  // the fused kernel: a packed range, records it holds (widths up to 14: at most 8 entries a channel)
+  // and at least two ring stages in one SM's shared memory (uncompressed tokens, if any, join in the
+  // merge kernel)
+  FusedChoice fk;
+  size_t fsm = 0;
+  if (extra.t_first < n_ctx && plan.max_bits <= 14) {
+    const LayerShape sh = layer_shape(plan, layer);
+    const long tiles = static_cast<long>(batch) * a.n_kv * ((n_ctx + TILE - 1) / TILE - extra.t_first / TILE);
+    fk = np == 1 ? fused_kernel_for<1>(sh, tiles, plan.num_sms) : fused_kernel_for<2>(sh, tiles, plan.num_sms);
+    a.stage_bytes = sh.stage;
+    a.nks_max = sh.nks;
+    if (fk.kernel) {
+      // the deepest ring (up to 3 stages per warp group) that fits
+      for (a.n_stages = 3; a.n_stages >= 2; --a.n_stages) {
+        fsm = static_cast<size_t>(FusedSmem(sh.stage, sh.nks, np, fk.groups, plan.n_entries, a.n_stages).total);
+        if (fsm <= 227 * 1024) break;
+      }
+      if (a.n_stages < 2) fk.kernel = nullptr;
+    }
+  }
   const int range = n_ctx - (extra.t_first / TILE) * TILE;
-  const DecodeSplit sp = decode_split_for(batch, a.n_kv, range, plan.num_sms, fk != nullptr);
+  const DecodeSplit sp = decode_split_for(batch, a.n_kv, range, plan.num_sms, fk.kernel != nullptr);
   a.n_splits = extra.t_first < n_ctx ? sp.n_splits : 0;     // no packed range: merge kernel only
   a.split_len = sp.split_len;
   {
@@ -1831,20 +1920,11 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
   const size_t msm = 4 * (static_cast<size_t>(D) * D + kMWarps * D + D + static_cast<size_t>((a.n_full + 3) & ~3));
   if (msm > 227 * 1024) return cudaErrorNotSupported;
   cudaError_t e = cudaSuccess;
-  if (fk) {
-    const int wu = n2w + n1w, nks = n2w + 2 * n1w;
-    const int wg = np == 1 ? fused_groups<1>() : fused_groups<2>();
-    // the deepest ring (up to 3 stages per warp group) that fits the shared memory of one SM
-    size_t smem = 0;
-    for (a.n_stages = 3; a.n_stages >= 2; --a.n_stages) {
-      smem = static_cast<size_t>(FusedSmem(wu, nks, np, wg, plan.n_entries, a.n_stages).total);
-      if (smem <= 227 * 1024) break;
-    }
-    if (a.n_stages < 2) return cudaErrorNotSupported;
-    e = ensure_smem_optin(reinterpret_cast<const void*>(fk), smem);
+  if (fk.kernel) {
+    e = ensure_smem_optin(reinterpret_cast<const void*>(fk.kernel), fsm);
     if (e != cudaSuccess) return e;
     const unsigned n_cta = static_cast<unsigned>(static_cast<long>(sp.n_splits) * a.n_kv * batch);
-    e = launch_pdl(fk, dim3(n_cta), dim3(128 * wg), smem, st, a);
+    e = launch_pdl(fk.kernel, dim3(n_cta), dim3(128 * fk.groups), fsm, st, a);
     if (e != cudaSuccess) return e;
     e = ensure_smem_optin(reinterpret_cast<const void*>(aatc_decode_merge_kernel), msm);
     if (e != cudaSuccess) return e;

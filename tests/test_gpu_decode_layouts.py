@@ -1,0 +1,66 @@
+"""Decode attention over record layouts at the edges of the fused kernel's choice (value records of
+each instantiation, streams that differ within a layer, empty streams, widths above 8 bits) and of its
+tiling, against 64-bit attention over the dequantized coefficients (aatc_dequantize, itself checked
+bit for bit against the oracle).  Tolerances: the acceptance bounds of harness.py, and a relative L2
+of 1e-4 (operands of ~22 bits, fp32 sums: 1e-5 and below was measured)."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import harness as Hn
+from test_gpu_prefill_layouts import random_plan, tokens
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def attention(coef, basis, q, group, first=0):
+    """64-bit attention of q bf16 [batch][H_q][128] over tokens [first, n) of coef [batch][n][n_kv][2][128]."""
+    k = torch.einsum("bnhc,hdc->bnhd", coef[:, first:, :, 0].double(), torch.from_numpy(basis[0, :, 0]).to(DEV).double())
+    v = torch.einsum("bnhc,hdc->bnhd", coef[:, first:, :, 1].double(), torch.from_numpy(basis[0, :, 1]).to(DEV).double())
+    k, v = k.repeat_interleave(group, 2), v.repeat_interleave(group, 2)
+    p = torch.softmax(torch.einsum("bhd,bnhd->bhn", q.double(), k) / math.sqrt(128), -1)
+    return torch.einsum("bhn,bnhd->bhd", p, v)
+
+
+CASES = [
+    # n_kv, group, b_max, bit totals of the heads, batch, n_ctx, first
+    (2, 4, 8, (0, 352), 1, 1, 0),                    # one token; a head whose streams hold no bits
+    (8, 4, 8, (352, 200, 97, 288), 1, 127, 0),       # differing streams, value records up to 8 + 3 words
+    (3, 3, 8, (352, 420, 131), 2, 129, 5),           # up to 13 + 4 words; the range starts inside a tile
+    (2, 1, 8, (900, 611), 1, 1000, 0),               # past 13 + 4 words
+    (1, 8, 8, (352,), 3, 4097, 130),                 # eight query heads
+    (2, 7, 8, (420, 255), 1, 700, 0),                # seven, differing streams
+    (2, 6, 8, (900, 700), 1, 300, 0),                # more than four query heads and large records
+    (4, 4, 12, (352, 449, 300), 1, 515, 0),          # channels above 8 bits
+    (1, 4, 16, (500,), 2, 260, 0),                   # channels above 14 bits
+]
+
+
+@pytest.mark.parametrize("many", [False, True])
+@pytest.mark.parametrize("n_kv,group,b_max,total,batch,n_ctx,first", CASES)
+def test_decode_record_layouts(aatc, n_kv, group, b_max, total, batch, n_ctx, first, many):
+    if many:                                          # sequences enough for four tiles per SM (and a few more)
+        batch = 620 // (n_kv * ((n_ctx + 127) // 128)) + 1
+    rng = np.random.default_rng([n_ctx, n_kv, b_max])
+    plan, basis, bits = random_plan(aatc, rng, n_kv, group, b_max, total)
+    k, v = tokens(rng, basis, batch, n_ctx, n_kv)
+    cap = n_ctx + 70
+    cache = plan.new_cache(batch, cap, DEV)
+    cache.fill_(-1)                                   # whatever the cache held before
+    aatc.encode(plan, 0, k, v, cache, 0, cap)
+    q = torch.from_numpy(rng.standard_normal((batch, n_kv * group, 128))).to(DEV).to(torch.bfloat16)
+    if first:
+        out = aatc.decode_attention_sw(plan, 0, q, cache, first, n_ctx, cap)
+    else:
+        out = aatc.decode_attention(plan, 0, q, cache, n_ctx, cap)
+    coef = aatc.dequantize(plan, 0, cache, batch, 0, n_ctx, cap)
+    ref = attention(coef, basis, q, group, first)
+    if not torch.any(ref):
+        assert not torch.any(out)
+        return
+    _, rel = Hn.check_decode(out.cpu().numpy().reshape(-1, 128), ref.cpu().numpy().reshape(-1, 128))
+    assert rel <= 1e-4, rel
+    assert plan.device_error() == 0

@@ -30,11 +30,13 @@ def random_plan(aatc, rng, n_kv, group, b_max, total):
 
 
 def tokens(rng, basis, batch, n, n_kv):
+    g = torch.Generator(DEV).manual_seed(int(rng.integers(1 << 30)))
+    std = torch.arange(1, 129, device=DEV) ** -0.7
     out = []
     for kind in (0, 1):
-        z = rng.standard_normal((batch, n, n_kv, 128)) * np.arange(1, 129) ** -0.7
-        x = np.einsum("bnhc,hdc->bnhd", z, basis[0, :, kind])
-        out.append(torch.from_numpy(x.astype(np.float32)).to(DEV).to(torch.bfloat16).contiguous())
+        z = torch.randn((batch, n, n_kv, 128), generator=g, device=DEV) * std
+        x = torch.einsum("bnhc,hdc->bnhd", z, torch.from_numpy(basis[0, :, kind]).to(DEV))
+        out.append(x.to(torch.bfloat16).contiguous())
     return out
 
 
