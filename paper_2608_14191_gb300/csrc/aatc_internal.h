@@ -200,10 +200,13 @@ constexpr int MAX_FULL_TOKENS = 8192;   // shared-memory scores of the uncompres
 cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void* cache, int batch,
                           int n_ctx, int max_tokens, float* out, void* ws, cudaStream_t st,
                           const DecodeExtra& extra);
-// Prefill attention: codes workspace bytes, and the two launches (codes, attention).
-size_t prefill_workspace(int batch, int n_kv, int n_ctx);
+// Prefill attention: the bytes of the codes (the least workspace), those with room for the partial rows
+// of a split context, and the launches (codes, attention, merge of the splits).
+size_t prefill_codes_bytes(int batch, int n_kv, int n_ctx);
+size_t prefill_workspace(const Plan& plan, int batch, int n_ctx);
 cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_start, int n_q, const void* cache,
-                           int batch, int n_ctx, int max_tokens, float* out, void* ws, cudaStream_t st);
+                           int batch, int n_ctx, int max_tokens, float* out, void* ws, size_t ws_bytes,
+                           cudaStream_t st);
 cudaError_t launch_dequant(const Plan& plan, int layer, const void* cache, int batch, int t0, int n,
                            int max_tokens, float* out, cudaStream_t st);
 // Head-group plans (group.cu): encode of every group stream of a layer; decode workspace and

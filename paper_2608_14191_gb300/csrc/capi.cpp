@@ -505,7 +505,7 @@ aatc_status_t aatc_encode_hidden(aatc_plan_t p, int32_t layer, const void* x, in
 aatc_status_t aatc_prefill_workspace_bytes(aatc_plan_t p, int32_t batch, int32_t n_ctx, size_t* bytes) {
   aatc::Plan* plan = as_plan(p);
   if (!plan || !bytes || batch < 1 || n_ctx < 1) return AATC_ERR_INVALID_ARG;
-  *bytes = aatc::prefill_workspace(batch, plan->dims.n_kv_heads, n_ctx);
+  *bytes = aatc::prefill_workspace(*plan, batch, n_ctx);
   return AATC_OK;
 }
 
@@ -522,9 +522,9 @@ aatc_status_t aatc_prefill_attention(aatc_plan_t p, int32_t layer, const void* q
   if (plan->n_words > 32) return AATC_ERR_UNSUPPORTED;
   if (plan->max_bits > 12) return AATC_ERR_UNSUPPORTED;   // f16 code operands are exact up to |code| = 2048
   if (plan->group_heads > 1) return AATC_ERR_UNSUPPORTED;
-  if (workspace_bytes < aatc::prefill_workspace(batch, plan->dims.n_kv_heads, n_ctx)) return AATC_ERR_WORKSPACE;
+  if (workspace_bytes < aatc::prefill_codes_bytes(batch, plan->dims.n_kv_heads, n_ctx)) return AATC_ERR_WORKSPACE;
   return cuda_status(aatc::launch_prefill(*plan, layer, q, q_start, n_q, cache, batch, n_ctx, max_tokens, out,
-                                          workspace, static_cast<cudaStream_t>(stream)));
+                                          workspace, workspace_bytes, static_cast<cudaStream_t>(stream)));
 }
 
 aatc_status_t aatc_decode_workspace_bytes(aatc_plan_t p, int32_t batch, int32_t n_ctx, size_t* bytes) {

@@ -2,7 +2,7 @@
 // cached tokens (Def. sdpa for every query row; Algorithm 1's reconstruct / attend lines, computed
 // in the transformed space as the decode does: q . (U h) = (U^T q) . h).
 //
-// Two launches per call:
+// Two or three launches per call:
 //   codes    per (128-token tile, kv-head x K|V, sequence): the packed records -> the signed codes
 //            code_c = u_c - 2^(b_c - 1) as f16 (exact: |code| <= 2048) in a workspace of 32 KB tiles,
 //            [b][h][K|V][tile]: key rows are tokens, value rows channels, both K-major tensor-core
@@ -11,7 +11,8 @@
 //            everything on the tensor cores (tcgen05): q' = (U_K^T q) f^K log2(e) / sqrt(128),
 //            per 128-token tile S = alpha^K (q'_hi + q'_lo) . code^K, causal mask, lazily
 //            rescaled softmax, P' = 2^(S - m) alpha^V (f16) and O += P' code^V, finally
-//            out = U_V (f^V O / l).
+//            out = U_V (f^V O / l).  Few row blocks over a long context are split over the context;
+//   merge    then adds the splits' outputs, weighted by their l 2^m.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -38,6 +39,9 @@ struct PrefillArgs {
   const ChanEnc* enc;        // plan: [S][128] (offsets 2^(b-1))
   const StreamLayout* lay;   // plan: [S]
   int layer, n_kv, n_q_heads, group, q_start, n_q, n_ctx, n_ctx_pad, n_tiles, n_words;
+  float* part;               // splits of the context: [split][batch][n_kv][row][128] outputs of the split alone
+  float2* part_ml;           // and [split][batch][n_kv][row] (reference maximum, l)
+  int n_split;
   int* err;
 };
 
@@ -306,7 +310,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
   PrefillTcSmem& sm =
       *reinterpret_cast<PrefillTcSmem*>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~uintptr_t(1023));
   // row blocks in reverse: the longest causal ranges start first, the shortest fill the tail
-  const int rb = gridDim.x - 1 - blockIdx.x, head = blockIdx.y, b = blockIdx.z;
+  const int split = blockIdx.x % a.n_split, rb = (gridDim.x - 1 - blockIdx.x) / a.n_split;
+  const int head = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const bool softmax = tid < kTSoftmax;
   const int wu = ptx::warp_uniform(warp);
@@ -316,7 +321,10 @@ __global__ void __launch_bounds__(kTThreads, 1)
   const int R0 = rb * kTRows;
   const int r_last = min(n_rows - 1, R0 + kTRows - 1) - R0;
   const int kv_end = min(a.n_ctx, a.q_start + (R0 + r_last) / G + 1);
-  const int n_kv_tiles = (kv_end + TILE - 1) / TILE;
+  const int all_tiles = (kv_end + TILE - 1) / TILE;
+  const int tile0 = static_cast<int>(static_cast<long>(all_tiles) * split / a.n_split);   // this split's tiles
+  const int n_kv_tiles = static_cast<int>(static_cast<long>(all_tiles) * (split + 1) / a.n_split) - tile0;
+  const int tok0 = tile0 * TILE, ctx_left = a.n_ctx - tok0;
   const int r = 32 * (warp & 3) + lane, quarter = (warp >> 2) & 3, qc = 32 * quarter;
   const uint32_t lane_base = static_cast<uint32_t>(32 * (warp & 3)) << 16;
   const int R = R0 + r;
@@ -445,8 +453,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
       ptx::bulk_load(dst + st * kTOp, src + static_cast<size_t>(t) * TILE * D, kTOp, bar + st);
       return true;
     };
-    const __half* ck = a.codes + csk * a.n_ctx_pad * D;    // tiles of this head's keys, values: 32 KB operands
-    const __half* cv = a.codes + csv * a.n_ctx_pad * D;
+    const __half* ck = a.codes + (csk * a.n_ctx_pad + tok0) * D;    // tiles of this head's keys, values: 32 KB
+    const __half* cv = a.codes + (csv * a.n_ctx_pad + tok0) * D;
     int nk = 0, nv = 0;                                   // tiles requested
     while (nv < n_kv_tiles) {
       if (!load(nk, sm.kt[0], ck, sm.bar_k, sm.kfree)) break;
@@ -455,7 +463,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
       // alpha of the tile, into the slot of a tile whose PV is complete (so its softmax is too);
       // past the context it may hold any bits
       const int st = nv % kTRing;
-      const size_t tok = static_cast<size_t>(nv) * TILE;
+      const size_t tok = static_cast<size_t>(tok0) + static_cast<size_t>(nv) * TILE;
       ptx::mbar_arrive_expect_tx(&sm.bar_a[st], 2 * TILE * 4);
       ptx::bulk_load(sm.al[st][0], a.alpha + csk * a.n_tiles * TILE + tok, TILE * 4, &sm.bar_a[st]);
       ptx::bulk_load(sm.al[st][1], a.alpha + csv * a.n_tiles * TILE + tok, TILE * 4, &sm.bar_a[st]);
@@ -509,10 +517,11 @@ __global__ void __launch_bounds__(kTThreads, 1)
     }
   }
   __syncwarp();                                           // the MMA and copy warps reconverge
+  float m_row = -INFINITY, l_row = 0.0f;                  // of row r, over this split
   if (softmax) {
     // ---- softmax warps
     const int pos = R < n_rows ? a.q_start + R / G : -1;   // padding rows attend to nothing
-    const int last = min(pos, a.n_ctx - 1);               // last token this row attends to
+    const int last = min(pos, a.n_ctx - 1) - tok0;        // last token this row attends to, from the split's first
     float m_used = -INFINITY;
     uint64_t l2 = ptx::f2_pack(0.0f, 0.0f);
     const uint64_t rs2 = ptx::f2_pack(rsr, rsr);
@@ -557,8 +566,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
       }
       // alpha^V past the context may hold any bits, and would meet p = 0 below
       // (the warps of a column quarter write the same zeros)
-      if ((t + 1) * TILE > a.n_ctx) {
-        if (t * TILE + qc + lane >= a.n_ctx) sm.al[t % kTRing][1][qc + lane] = 0.0f;
+      if ((t + 1) * TILE > ctx_left) {
+        if (t * TILE + qc + lane >= ctx_left) sm.al[t % kTRing][1][qc + lane] = 0.0f;
         __syncwarp();
       }
       sm.xch[buf][quarter][r] = fmaxf(mt0, mt1);
@@ -616,6 +625,8 @@ __global__ void __launch_bounds__(kTThreads, 1)
     sm.xch[0][quarter][r] = l + lb;
     softmax_sync();
     const float lt = (sm.xch[0][0][r] + sm.xch[0][1][r]) + (sm.xch[0][2][r] + sm.xch[0][3][r]);
+    m_row = m_used;
+    l_row = lt;
     // ---- o_hat = f^V O / l, hi / lo bf16 in slots 0 / 1; U_V (rows = dim, K = channel) hi / lo
     // in slots 2 / 3
     {
@@ -674,8 +685,13 @@ __global__ void __launch_bounds__(kTThreads, 1)
     ptx::tmem_regs_ready(o0);
     if (R < n_rows) {
       const int qi = R / G, qh2 = head * G + R % G;
-      float4* dst =
-          reinterpret_cast<float4*>(a.out + ((static_cast<size_t>(b) * a.n_q + qi) * a.n_q_heads + qh2) * D + qc);
+      float* o = a.out + ((static_cast<size_t>(b) * a.n_q + qi) * a.n_q_heads + qh2) * D;
+      if (a.n_split > 1) {
+        const size_t prow = ((static_cast<size_t>(split) * gridDim.z + b) * a.n_kv + head) * n_rows + R;
+        o = a.part + prow * D;
+        if (quarter == 0) a.part_ml[prow] = make_float2(m_row, l_row);
+      }
+      float4* dst = reinterpret_cast<float4*>(o + qc);
 #pragma unroll
       for (int i = 0; i < 8; ++i)
         dst[i] = make_float4(__uint_as_float(o0[4 * i]), __uint_as_float(o0[4 * i + 1]), __uint_as_float(o0[4 * i + 2]),
@@ -690,15 +706,74 @@ __global__ void __launch_bounds__(kTThreads, 1)
   }
 }
 
+// One warp per query row: out = sum_s w_s out_s / sum_s w_s with w_s = l_s 2^(m_s - max m) over the
+// splits of the context (a split's output is already divided by its l; no tokens: l = 0).
+constexpr int kPMergeRows = 8;
+__global__ void __launch_bounds__(32 * kPMergeRows) aatc_prefill_merge_kernel(const PrefillArgs a, int batch) {
+  const int n_rows = a.n_q * a.group, lane = threadIdx.x & 31;
+  const long row = static_cast<long>(blockIdx.x) * kPMergeRows + (threadIdx.x >> 5), all = static_cast<long>(batch) * a.n_kv * n_rows;
+  if (row >= all) return;
+  float M = -INFINITY;
+  for (int s = 0; s < a.n_split; ++s) M = fmaxf(M, a.part_ml[s * all + row].x);
+  float den = 0.0f;
+  float4 o = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 4
+  for (int s = 0; s < a.n_split; ++s) {
+    const float2 ml = a.part_ml[s * all + row];
+    const float4 v = *reinterpret_cast<const float4*>(a.part + (s * all + row) * D + 4 * lane);
+    const float w = ml.y > 0.0f ? ml.y * ex2(ml.x - M) : 0.0f;
+    den += w;
+    o.x = fmaf(w, v.x, o.x);
+    o.y = fmaf(w, v.y, o.y);
+    o.z = fmaf(w, v.z, o.z);
+    o.w = fmaf(w, v.w, o.w);
+  }
+  const float inv = den > 0.0f ? 1.0f / den : 0.0f;
+  const int R = static_cast<int>(row % n_rows), head = static_cast<int>(row / n_rows % a.n_kv);
+  const size_t b = static_cast<size_t>(row / n_rows / a.n_kv);
+  *reinterpret_cast<float4*>(a.out + ((b * a.n_q + R / a.group) * a.n_q_heads + head * a.group + R % a.group) * D +
+                             4 * lane) = make_float4(o.x * inv, o.y * inv, o.z * inv, o.w * inv);
+}
+
+// Splits of the context for a call whose row blocks leave SMs idle or a last wave nearly empty: the
+// fewest rounds of one CTA per SM over (tiles of a split + the ~8 tiles' worth of time a CTA spends
+// outside its tiles, and ~3 more for the merge), counted on the blocks' mean causal range.  At least
+// four tiles a split.  333 queries x 4 heads over 30011 tokens on 8 kv-heads (88 row blocks on 152
+// SMs): one split 330 us, five 228 us with the merge; 78 queries over 60710 tokens (24 row blocks) 641
+// against 130 us.
+constexpr int kPMaxSplits = 16, kPCtaTiles = 8, kPMergeTiles = 3;
+int prefill_splits(long ctas, int mean_tiles, int num_sms, size_t room_rows) {
+  int best = 1;
+  long cost = (ctas + num_sms - 1) / num_sms * (mean_tiles + kPCtaTiles);
+  for (int n = 2; n <= std::min(kPMaxSplits, mean_tiles / 4); ++n) {
+    if (static_cast<size_t>(ctas) * n * kTRows > room_rows) break;
+    const long c = (ctas * n + num_sms - 1) / num_sms * ((mean_tiles + n - 1) / n + kPCtaTiles) + kPMergeTiles;
+    if (c < cost) {
+      cost = c;
+      best = n;
+    }
+  }
+  return best;
+}
+constexpr size_t kPRowBytes = (D + 2) * sizeof(float);     // of one row's partial
+
 }  // namespace
 
-size_t prefill_workspace(int batch, int n_kv, int n_ctx) {
+size_t prefill_codes_bytes(int batch, int n_kv, int n_ctx) {
   const size_t pad = (static_cast<size_t>(n_ctx) + TILE - 1) / TILE * TILE;
   return static_cast<size_t>(batch) * n_kv * 2 * pad * D * sizeof(__half);
 }
+// The codes, then room for the partial rows of up to four rounds of split CTAs (none for contexts
+// that are never split).
+size_t prefill_workspace(const Plan& plan, int batch, int n_ctx) {
+  const int most = std::min(kPMaxSplits, (n_ctx + TILE - 1) / TILE / 4);
+  const size_t rows = most < 2 ? 0 : static_cast<size_t>(std::min(4, most)) * plan.num_sms * kTRows;
+  return prefill_codes_bytes(batch, plan.dims.n_kv_heads, n_ctx) + rows * kPRowBytes;
+}
 
 cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_start, int n_q, const void* cache,
-                           int batch, int n_ctx, int max_tokens, float* out, void* ws, cudaStream_t st) {
+                           int batch, int n_ctx, int max_tokens, float* out, void* ws, size_t ws_bytes,
+                           cudaStream_t st) {
   const CacheGeom g = cache_geom(batch, plan.dims.n_kv_heads, max_tokens, plan.n_words);
   PrefillArgs a;
   a.words = static_cast<const uint32_t*>(cache);
@@ -734,8 +809,21 @@ cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_sta
   const size_t smem = sizeof(PrefillTcSmem) + 1024;
   e = ensure_smem_optin(reinterpret_cast<const void*>(aatc_prefill_tc_kernel), smem);
   if (e != cudaSuccess) return e;
-  const int n_rows = n_q * a.group;
-  aatc_prefill_tc_kernel<<<dim3((n_rows + kTRows - 1) / kTRows, a.n_kv, batch), kTThreads, smem, st>>>(a);
+  const int n_rows = n_q * a.group, blocks = (n_rows + kTRows - 1) / kTRows;
+  // splits of the context, as far as the workspace has room for their partial rows
+  const size_t codes_bytes = prefill_codes_bytes(batch, a.n_kv, n_ctx);
+  const size_t room = (ws_bytes - codes_bytes) / kPRowBytes;
+  const int mean_tiles = (q_start + n_q / 2) / TILE + 1;
+  a.n_split = prefill_splits(static_cast<long>(blocks) * a.n_kv * batch, mean_tiles, std::max(1, plan.num_sms), room);
+  const size_t rows = static_cast<size_t>(a.n_split) * batch * a.n_kv * n_rows;
+  a.part = reinterpret_cast<float*>(static_cast<char*>(ws) + codes_bytes);
+  a.part_ml = reinterpret_cast<float2*>(a.part + rows * D);
+  aatc_prefill_tc_kernel<<<dim3(blocks * a.n_split, a.n_kv, batch), kTThreads, smem, st>>>(a);
+  e = cudaGetLastError();
+  if (e != cudaSuccess || a.n_split == 1) return e;
+  const long all = static_cast<long>(batch) * a.n_kv * n_rows;
+  aatc_prefill_merge_kernel<<<static_cast<unsigned>((all + kPMergeRows - 1) / kPMergeRows), 32 * kPMergeRows, 0, st>>>(
+      a, batch);
   return cudaGetLastError();
 }
 

@@ -79,3 +79,35 @@ def test_prefill_record_layouts(aatc, n_kv, group, b_max, total, batch, n_ctx, n
     ref = reference(coef, basis, q, n_ctx - n_q, group)
     Hn.check_decode(out.cpu().numpy().reshape(-1, 128), ref.cpu().numpy().reshape(-1, 128))
     assert plan.device_error() == 0
+
+
+SPLITS = [
+    # n_kv, group, batch, n_ctx, n_q: a split context (few row blocks, many tiles)
+    (1, 1, 1, 1024, 1),                              # eight tiles, one row
+    (1, 4, 1, 2049, 70),                             # splits of unequal lengths, a last tile of one token
+    (2, 3, 2, 1500, 700),                            # causal ranges that end in different splits
+    (1, 2, 1, 4200, 2500),                           # rows that end before the later splits begin
+]
+
+
+@pytest.mark.parametrize("room", ["full", "codes only"])
+@pytest.mark.parametrize("n_kv,group,batch,n_ctx,n_q", SPLITS)
+def test_prefill_split_context(aatc, n_kv, group, batch, n_ctx, n_q, room):
+    """The split context against 64 bits, and the same call with a workspace that holds the codes
+    alone (accepted, not split)."""
+    rng = np.random.default_rng([n_ctx, n_q])
+    plan, basis, _ = random_plan(aatc, rng, n_kv, group, 8, (352,))
+    k, v = tokens(rng, basis, batch, n_ctx, n_kv)
+    cache = plan.new_cache(batch, n_ctx, DEV)
+    aatc.encode(plan, 0, k, v, cache, 0, n_ctx)
+    q = torch.from_numpy(rng.standard_normal((batch, n_q, n_kv * group, 128))).to(DEV).to(torch.bfloat16)
+    codes = batch * n_kv * 2 * ((n_ctx + 127) // 128) * 128 * 128 * 2
+    ws = None if room == "full" else torch.empty(codes // 4, device=DEV)
+    out = aatc.prefill_attention(plan, 0, q, n_ctx - n_q, cache, n_ctx, n_ctx, workspace=ws)
+    coef = aatc.dequantize(plan, 0, cache, batch, 0, n_ctx, n_ctx)
+    ref = reference(coef, basis, q, n_ctx - n_q, group)
+    Hn.check_decode(out.cpu().numpy().reshape(-1, 128), ref.cpu().numpy().reshape(-1, 128))
+    assert plan.device_error() == 0
+    if ws is not None:
+        with pytest.raises(aatc.AatcError):
+            aatc.prefill_attention(plan, 0, q, n_ctx - n_q, cache, n_ctx, n_ctx, workspace=ws[:-1])
