@@ -68,6 +68,7 @@ struct PlanDevice {
   const short* chan_ent;  // [S][128][kChanEnt]: entries of each channel (-1 padded)
   const short* ce8;       // [S][128][8]: the first eight of them (0 padded)
   const float* cw8;       // [S][128][8]: 2^shift of those (0: none)
+  const unsigned char* proj;  // projection operands of the prefill (per-kv-head plans)
   int* err;               // [4] sticky device flags
 };
 
@@ -203,6 +204,9 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
 // Prefill attention: the bytes of the codes (the least workspace), those with room for the partial rows
 // of a split context, and the launches (codes, attention, merge of the splits).
 size_t prefill_codes_bytes(int batch, int n_kv, int n_ctx);
+// Plan constants of the prefill: their bytes, and the launch that writes them from the plan's bases.
+size_t prefill_operand_bytes(int n_layers, int n_kv);
+cudaError_t launch_prefill_operands(const Plan& plan, void* proj, cudaStream_t st);
 size_t prefill_workspace(const Plan& plan, int batch, int n_ctx);
 cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_start, int n_q, const void* cache,
                            int batch, int n_ctx, int max_tokens, float* out, void* ws, size_t ws_bytes,

@@ -358,14 +358,15 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaGetDevice(&plan->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&plan->num_sms, cudaDevAttrMultiProcessorCount, plan->device);
-  if (e == cudaSuccess) e = cudaMalloc(&plan->block, total);
+  // the prefill's projection operands follow the staged tables; a kernel writes them
+  const size_t proj_bytes = basis ? prefill_operand_bytes(dims->n_layers, dims->n_kv_heads) : 0;
+  if (e == cudaSuccess) e = cudaMalloc(&plan->block, total + proj_bytes);
   if (e != cudaSuccess) {
     delete plan;
     return e == cudaErrorMemoryAllocation ? AATC_ERR_NOMEM : cuda_status(e);
   }
-  plan->block_bytes = total;
+  plan->block_bytes = total + proj_bytes;
   e = cudaMemcpyAsync(plan->block, host.data(), total, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   auto* base = static_cast<unsigned char*>(plan->block);
   plan->dev.ubf16_t = base + o_ubf;
   plan->dev.u32 = reinterpret_cast<const float*>(base + o_u32);
@@ -381,6 +382,8 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   plan->dev.err = reinterpret_cast<int*>(base + o_err);
   plan->group_heads = g_h;
   if (basis) {
+    plan->dev.proj = base + total;
+    if (e == cudaSuccess) e = launch_prefill_operands(*plan, base + total, st);
     if (e == cudaSuccess) e = encode_tensor_maps_u(*plan);
   } else {
     plan->dev.ubf16_t = nullptr;
@@ -393,6 +396,8 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
       e = make_tensor_map_2d(plan->tmap_g, false, plan->gdev.ubf, static_cast<uint64_t>(n_g), GB / n_g,
                              static_cast<uint64_t>(n_g) * 2, 64, 256);
   }
+  const cudaError_t es = cudaStreamSynchronize(st);         // also on an error: the copy reads `host`
+  if (e == cudaSuccess) e = es;
   if (e != cudaSuccess) {
     cudaFree(plan->block);
     delete plan;

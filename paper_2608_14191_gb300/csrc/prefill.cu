@@ -33,8 +33,7 @@ struct PrefillArgs {
   const __nv_bfloat16* q;    // [batch][n_q][H_q][128]
   float* out;                // [batch][n_q][H_q][128]
   __half* codes;             // workspace [batch][n_kv][2][tile]: 128 x 128 operands (swizzled)
-  const float* u32;          // plan: [S][128 dim][128 ch]
-  const float* u32t;         // plan: [S][128 ch][128 dim]
+  const unsigned char* proj; // plan: [S / 2][5] projection operands (aatc_prefill_operands_kernel)
   const float* f;            // plan: [S][128]
   const ChanEnc* enc;        // plan: [S][128] (offsets 2^(b-1))
   const StreamLayout* lay;   // plan: [S]
@@ -269,7 +268,7 @@ struct PrefillTcSmem {
   alignas(16) float al[kTRing][2][TILE];           // alpha^K, alpha^V of the tiles in the value ring
   float xch[2][4][kTRows];                         // per-row partials of the column quarters (two slots)
   uint64_t bar_k[kTRing], bar_v[kTRing], bar_a[kTRing], kfree[kTRing], vfree[kTRing], bar_s[2], pready[2], ofree[2],
-      bar_p;
+      bar_p, bar_u;
   uint32_t tmem;
   int abort_flag, never;
 };
@@ -304,6 +303,24 @@ __device__ __forceinline__ void store_split_bf16(unsigned char* dst, const float
 __device__ __forceinline__ void row_sync(int wq) { asm volatile("bar.sync %0, 128;" ::"r"(2 + wq) : "memory"); }
 __device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kTSoftmax) : "memory"); }
 
+// Plan constants of the attention kernel, per (layer, kv-head) five 32 KB operands in the layout the
+// tensor cores read: U_K^T (rows = channel, K = dim) in three bf16 parts, U_V (rows = dim, K =
+// channel) in two.  Splitting them in every CTA took a third of the time a CTA spends outside its
+// tiles.
+__global__ void __launch_bounds__(256) aatc_prefill_operands_kernel(const float* u32, const float* u32t, unsigned char* proj) {
+  const int sk = 2 * blockIdx.x, g = blockIdx.y * 256 + threadIdx.x;
+  const int row = g >> 4, k8 = (g & 15) * 8;
+  unsigned char* dst = proj + static_cast<size_t>(blockIdx.x) * 5 * kTOp + sw128_off(row, k8);
+#pragma unroll
+  for (int kind = 0; kind < 2; ++kind) {
+    const float* src = (kind == 0 ? u32t + static_cast<size_t>(sk) * D * D : u32 + static_cast<size_t>(sk + 1) * D * D) +
+                       row * D + k8;
+    const float4 u0 = *reinterpret_cast<const float4*>(src), u1 = *reinterpret_cast<const float4*>(src + 4);
+    const float u[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
+    store_split_bf16(dst + 3 * kind * kTOp, u, 3 - kind);
+  }
+}
+
 __global__ void __launch_bounds__(kTThreads, 1)
     aatc_prefill_tc_kernel(const PrefillArgs a) {
   extern __shared__ unsigned char smraw[];
@@ -329,6 +346,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
   const uint32_t lane_base = static_cast<uint32_t>(32 * (warp & 3)) << 16;
   const int R = R0 + r;
   unsigned char* const pj = sm.kt[0];              // projection operand i at pj + i * kTOp
+  const unsigned char* proj = a.proj + static_cast<size_t>(sk / 2) * 5 * kTOp;
   volatile int* abort_flag = &sm.abort_flag;
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     if (!ptx::mbar_wait_bounded(bar, parity, abort_flag)) {
@@ -351,16 +369,19 @@ __global__ void __launch_bounds__(kTThreads, 1)
       ptx::mbar_init(&sm.ofree[i], 1);               // their PV done
     }
     ptx::mbar_init(&sm.bar_p, 1);
+    ptx::mbar_init(&sm.bar_u, 1);
     sm.abort_flag = 0;
     sm.never = 0;
     ptx::fence_mbar_init();
+    ptx::mbar_arrive_expect_tx(&sm.bar_u, 3 * kTOp);
+    ptx::bulk_load(pj + kTOp, proj, 3 * kTOp, &sm.bar_u);
   }
   if (warp == 0) {
     ptx::tmem_alloc(&sm.tmem, 512);
     ptx::tmem_relinquish();
   }
-  // ---- projection operands: q rows (bf16) in slot 0, U_K^T (rows = channel, K = dim) in three
-  // bf16 parts in slots 1-3
+  // ---- projection operands: q rows (bf16) in slot 0; U_K^T (rows = channel, K = dim) in three bf16
+  // parts in slots 1-3, a bulk copy
   if (softmax) {
     for (int g = tid; g < kTRows * 16; g += kTSoftmax) {
       const int row = g >> 4, k8 = (g & 15) * 8, RR = R0 + row;
@@ -372,14 +393,6 @@ __global__ void __launch_bounds__(kTThreads, 1)
       }
       *reinterpret_cast<uint4*>(pj + sw128_off(row, k8)) = v;
     }
-    const float* ukt = a.u32t + static_cast<size_t>(sk) * D * D;
-    for (int g = tid; g < D * 16; g += kTSoftmax) {
-      const int c = g >> 4, k8 = (g & 15) * 8;
-      const float4 u0 = *reinterpret_cast<const float4*>(ukt + c * D + k8);
-      const float4 u1 = *reinterpret_cast<const float4*>(ukt + c * D + k8 + 4);
-      const float u[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-      store_split_bf16(pj + kTOp + sw128_off(c, k8), u, 3);
-    }
   }
   ptx::fence_proxy_async_smem();
   ptx::tc_fence_before();
@@ -390,6 +403,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
   if (wu == kTMma / 32) {
     const uint32_t el = ptx::elect_one(), tm = ptx::warp_uniform(tmem);
     const uint64_t ad = ptx::sdesc_kmajor_sw128(pj_a);
+    wait(&sm.bar_u, 0);
 #pragma unroll
     for (int part = 0; part < 3; ++part)
 #pragma unroll
@@ -516,6 +530,15 @@ __global__ void __launch_bounds__(kTThreads, 1)
       if (t + 2 < n_kv_tiles) issue_s(t + 2);
     }
   }
+  if (wu == kTMma / 32) {
+    // U_V (rows = dim, K = channel) hi / lo into slots 2 / 3, once the last PV (and with it every MMA
+    // that reads the rings) is complete
+    if (n_kv_tiles > 0) wait(&sm.ofree[(n_kv_tiles - 1) & 1], ((n_kv_tiles - 1) >> 1) & 1);
+    if (lane == 0) {
+      ptx::mbar_arrive_expect_tx(&sm.bar_u, 2 * kTOp);
+      ptx::bulk_load(pj + 2 * kTOp, proj + 3 * kTOp, 2 * kTOp, &sm.bar_u);
+    }
+  }
   __syncwarp();                                           // the MMA and copy warps reconverge
   float m_row = -INFINITY, l_row = 0.0f;                  // of row r, over this split
   if (softmax) {
@@ -627,8 +650,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
     const float lt = (sm.xch[0][0][r] + sm.xch[0][1][r]) + (sm.xch[0][2][r] + sm.xch[0][3][r]);
     m_row = m_used;
     l_row = lt;
-    // ---- o_hat = f^V O / l, hi / lo bf16 in slots 0 / 1; U_V (rows = dim, K = channel) hi / lo
-    // in slots 2 / 3
+    // ---- o_hat = f^V O / l, hi / lo bf16 in slots 0 / 1
     {
       const float il = lt > 0.0f ? 1.0f / lt : 0.0f;
       uint32_t o0[32];
@@ -647,14 +669,6 @@ __global__ void __launch_bounds__(kTThreads, 1)
         store_split_bf16(pj + sw128_off(r, qc + 8 * g8), u, 2);
       }
     }
-    const float* uv = a.u32 + static_cast<size_t>(sv) * D * D;
-    for (int g = tid; g < D * 16; g += kTSoftmax) {
-      const int d = g >> 4, k8 = (g & 15) * 8;
-      const float4 u0 = *reinterpret_cast<const float4*>(uv + d * D + k8);
-      const float4 u1 = *reinterpret_cast<const float4*>(uv + d * D + k8 + 4);
-      const float u[8] = {u0.x, u0.y, u0.z, u0.w, u1.x, u1.y, u1.z, u1.w};
-      store_split_bf16(pj + 2 * kTOp + sw128_off(d, k8), u, 2);
-    }
   }
   ptx::fence_proxy_async_smem();
   ptx::tc_fence_before();
@@ -664,6 +678,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
   if (wu == kTMma / 32) {
     const uint32_t el = ptx::elect_one(), tm = ptx::warp_uniform(tmem);
     const uint64_t ad = ptx::sdesc_kmajor_sw128(pj_a);
+    if (!ptx::mbar_wait_bounded(&sm.bar_u, 1, &sm.never)) atomicOr(a.err, 2);
 #pragma unroll
     for (int pr = 0; pr < 3; ++pr) {
       const uint32_t as = pr == 2 ? 1u : 0u, bs = pr == 1 ? 3u : 2u;
@@ -759,6 +774,14 @@ constexpr size_t kPRowBytes = (D + 2) * sizeof(float);     // of one row's parti
 
 }  // namespace
 
+size_t prefill_operand_bytes(int n_layers, int n_kv) { return static_cast<size_t>(n_layers) * n_kv * 5 * kTOp; }
+
+cudaError_t launch_prefill_operands(const Plan& plan, void* proj, cudaStream_t st) {
+  aatc_prefill_operands_kernel<<<dim3(plan.n_streams / 2, D * 16 / 256), 256, 0, st>>>(
+      plan.dev.u32, plan.dev.u32t, static_cast<unsigned char*>(proj));
+  return cudaGetLastError();
+}
+
 size_t prefill_codes_bytes(int batch, int n_kv, int n_ctx) {
   const size_t pad = (static_cast<size_t>(n_ctx) + TILE - 1) / TILE * TILE;
   return static_cast<size_t>(batch) * n_kv * 2 * pad * D * sizeof(__half);
@@ -781,8 +804,7 @@ cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_sta
   a.q = static_cast<const __nv_bfloat16*>(q);
   a.out = out;
   a.codes = static_cast<__half*>(ws);
-  a.u32 = plan.dev.u32;
-  a.u32t = plan.dev.u32t;
+  a.proj = plan.dev.proj;
   a.f = plan.dev.f;
   a.enc = plan.dev.enc;
   a.lay = plan.dev.lay;
