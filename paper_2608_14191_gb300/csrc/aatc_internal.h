@@ -176,6 +176,26 @@ aatc_status_t status_from_cuda(cudaError_t e);
 // drives several GPUs, both get the opt-in on every device they launch on (defined in capi.cpp).
 cudaError_t ensure_smem_optin(const void* kernel, size_t bytes);
 
+#if defined(__CUDACC__)
+// Launch with programmatic stream serialization: the kernel may start before the preceding
+// grid in the stream completes; it synchronizes with griddepcontrol.wait before touching
+// anything that grid produces.
+template <typename... Args>
+cudaError_t launch_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#endif
+
 // Kernel launchers (defined in the .cu files); return the CUDA error of the launch.
 // 2D tiled tensor map with 128-byte swizzle (16-bit elements): `map` is a 128-byte, 64-aligned
 // CUtensorMap; rows of `inner` elements, `row_bytes` apart; box box_inner x box_rows.

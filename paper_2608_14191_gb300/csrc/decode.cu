@@ -1747,24 +1747,6 @@ __global__ void aatc_dequant_kernel(const uint32_t* words, const float* alpha, c
   }
 }
 
-// Launch with programmatic stream serialization: the kernel may start before the preceding
-// grid in the stream completes; it synchronizes with griddepcontrol.wait before touching
-// anything that grid produces.
-template <typename... Args>
-cudaError_t launch_pdl(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 template <int JPW, int NP>
 cudaError_t launch_split_t(const DecodeArgs& a, int batch, size_t smem, cudaStream_t st) {
   cudaError_t e = ensure_smem_optin(reinterpret_cast<const void*>(aatc_decode_split_kernel<JPW, NP>), smem);

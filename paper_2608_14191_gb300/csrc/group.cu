@@ -7,7 +7,8 @@
 // (kv-head block m = j / group) sees the embedded query q~ (q at block m, zeros elsewhere):
 //   score_t = (U_K^T q~) . h_hat_t / sqrt(128) = alpha_t sum_c q'_c f_c code_tc,
 //   out     = rows of block m of U_V applied to sum_t p_t h_hat^V_t.
-// Three launches per call:
+// Three launches per call, each a programmatic dependent of the one before (plan constants, and in the
+// attention kernel the first record chunks, are requested before it waits):
 //   query  per (query row < 16, slice, group, sequence): q'' = (U_K^T q~) f log2(e) / sqrt(128)
 //          over the slice's 128 channels, the slice's scale and part of the offset correction, and
 //          the row's words of the slice's score A fragments (entry order of its key records)
@@ -107,16 +108,22 @@ __global__ void __launch_bounds__(kGQThreads) aatc_group_query_kernel(const Grou
   const bool live = i < a.nq;
   const int m = i / a.group, hq = g * a.nq + i;
   const size_t bg = static_cast<size_t>(b) * a.n_groups + g;
-  if (s == 0 && tid == 0) a.ticket[bg * 16 + i] = 0;
-  if (live && tid < D) qv[tid] = __bfloat162float(a.q[(static_cast<size_t>(b) * a.n_q_heads + hq) * D + tid]);
-  __syncthreads();
   const int pslot = (a.layer * a.n_kv + g * a.gh + s) * 2;   // plan slot of the slice's keys
+  float x[32];
   if (live) {
     const float* u = a.uk + (static_cast<size_t>(a.layer) * a.n_groups + g) * a.n * a.n +
                      static_cast<size_t>(m * D + 32 * dq) * a.n + s * D + c;
-    float x[32];
 #pragma unroll
     for (int k = 0; k < 32; ++k) x[k] = u[static_cast<size_t>(k) * a.n];   // 32 loads in flight per thread
+  }
+  // plan constants above; the query and the workspace once the preceding grids are complete, and only
+  // then may the attention kernel start, which reads the cache
+  ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
+  if (s == 0 && tid == 0) a.ticket[bg * 16 + i] = 0;
+  if (live && tid < D) qv[tid] = __bfloat162float(a.q[(static_cast<size_t>(b) * a.n_q_heads + hq) * D + tid]);
+  __syncthreads();
+  if (live) {
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int k = 0; k < 32; ++k) acc[k & 3] = fmaf(x[k], qv[32 * dq + k], acc[k & 3]);
@@ -254,18 +261,38 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
   const int pslot0 = (a.layer * a.n_kv + g * GH) * 2;   // plan slot of slice 0, keys (values + 1)
   const size_t stream_words = static_cast<size_t>(a.n_tiles) * a.n_words * TILE;
 
-  // ---- the score A fragments (built by the query kernel) by cp.async, with the first ring chunk;
-  // the value offsets, the slice layouts and the query scales by plain loads
+  ptx::grid_launch_dependents();
+  // ---- record chunks: per tile the key words of slices 0 .. GH-1, then their value words; the first
+  // ones now (the query kernel lets this one start only when the cache is complete)
+  const int n_chunks = 2 * (tile_hi - tile_lo);
+  const int S = a.stages, cw = L.chunk_words;
+  auto issue = [&](int u) {
+    if (u < n_chunks) {
+      const int tile = tile_lo + (u >> 1), kind = u & 1;
+      uint32_t* dst = ring + (u % S) * GH * cw;
+#pragma unroll
+      for (int sl = 0; sl < GH; ++sl) {
+        const uint32_t* src = a.words + ((slot0 + sl) * 2 + kind) * stream_words + static_cast<size_t>(tile) * cw;
+        for (int p = tid * 4; p < cw; p += kGAThreads * 4) cp_async16(dst + sl * cw + p, src + p);
+      }
+    }
+    cp_async_commit();
+  };
+  for (int u = 0; u < S - 1; ++u) issue(u);
+  // ---- the value offsets and the slice layouts (plan constants) by plain loads
+  for (int j = tid; j < N; j += kGAThreads) offv[j] = a.enc[(pslot0 + 2 * (j / D) + 1) * D + j % D].off;
+  if (tid < 2 * GH) {
+    info[2 * tid] = a.lay[pslot0 + tid].n2;
+    info[2 * tid + 1] = a.lay[pslot0 + tid].n1;
+  }
+  // ---- what the query kernel wrote: the score A fragments by cp.async, the query scales
+  ptx::grid_dependency_wait();
   {
     const int fw = GH * a.ks_max * 128;
     const uint32_t* fsrc = a.qfrag + bg * 2 * fw;
     uint32_t* fdst = reinterpret_cast<uint32_t*>(qfh);   // hi table, then the lo table (contiguous)
     for (int p = tid * 4; p < 2 * fw; p += kGAThreads * 4) cp_async16(fdst + p, fsrc + p);
-  }
-  for (int j = tid; j < N; j += kGAThreads) offv[j] = a.enc[(pslot0 + 2 * (j / D) + 1) * D + j % D].off;
-  if (tid < 2 * GH) {
-    info[2 * tid] = a.lay[pslot0 + tid].n2;
-    info[2 * tid + 1] = a.lay[pslot0 + tid].n1;
+    cp_async_commit();
   }
   if (tid < 16 * GH) qsl[tid] = a.qsc[(bg * 16 * GH + tid) * 2] * 16777216.0f;
   if (tid < 16) {
@@ -308,22 +335,7 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
   }
   const uint32_t psel = (2 * (t & 1)) | 0x40u | ((2 * (t & 1) + 1) << 8) | 0x4000u;   // bytes i0, i0 + 1 -> halves
 
-  // ---- record chunks: per tile the key words of slices 0 .. GH-1, then their value words
-  const int n_chunks = 2 * (tile_hi - tile_lo);
-  const int S = a.stages, cw = L.chunk_words;
-  auto issue = [&](int u) {
-    if (u < n_chunks) {
-      const int tile = tile_lo + (u >> 1), kind = u & 1;
-      uint32_t* dst = ring + (u % S) * GH * cw;
-#pragma unroll
-      for (int sl = 0; sl < GH; ++sl) {
-        const uint32_t* src = a.words + ((slot0 + sl) * 2 + kind) * stream_words + static_cast<size_t>(tile) * cw;
-        for (int p = tid * 4; p < cw; p += kGAThreads * 4) cp_async16(dst + sl * cw + p, src + p);
-      }
-    }
-    cp_async_commit();
-  };
-  for (int u = 0; u < S - 1; ++u) issue(u);
+  cp_async_wait<0>();                             // fragments (and the chunks before them): the loop counts its own
 
   float oacc[NPW][4];
 #pragma unroll
@@ -588,9 +600,24 @@ __global__ void __launch_bounds__(kGMThreads) aatc_group_merge_kernel(const Grou
   const size_t bg = static_cast<size_t>(b) * a.n_groups + g;
   const size_t pstride = static_cast<size_t>(N) + 4;
   const float* pb = a.part + ((bg * a.nq + i) * a.n_splits) * pstride;
+  // U_V rows of the slice's part (plan constants), requested before the attention kernel's partials
+  const float* u = a.uvt + (static_cast<size_t>(a.layer) * a.n_groups + g) * static_cast<size_t>(N) * N +
+                   static_cast<size_t>(s * D + 32 * q4) * N + static_cast<size_t>(m) * D + c;
+  float uv[32];
+#pragma unroll
+  for (int k = 0; k < 32; ++k) uv[k] = u[static_cast<size_t>(k) * N];   // 32 loads in flight per thread
+  ptx::grid_dependency_wait();
+  ptx::grid_launch_dependents();
+  // the slice's partial sums of the first 4 * 24 splits, with the (m, l) pairs: one round trip
+  const float* pc = pb + s * D + c;
+  float x[24];
+#pragma unroll
+  for (int k = 0; k < 24; ++k) x[k] = q4 + 4 * k < a.n_splits ? pc[static_cast<size_t>(q4 + 4 * k) * pstride] : 0.0f;
+  const bool mine = tid < a.n_splits;
+  const float2 ml = mine ? *reinterpret_cast<const float2*>(pb + tid * pstride + N) : make_float2(-INFINITY, 0.0f);
   // M = max_s m_s (block reduction), then w_s and l = sum_s w_s l_s
-  float mloc = -INFINITY;
-  for (int s2 = tid; s2 < a.n_splits; s2 += kGMThreads) mloc = fmaxf(mloc, pb[s2 * pstride + N]);
+  float mloc = ml.x;
+  for (int s2 = tid + kGMThreads; s2 < a.n_splits; s2 += kGMThreads) mloc = fmaxf(mloc, pb[s2 * pstride + N]);
   for (int o = 16; o > 0; o >>= 1) mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, o));
   if ((tid & 31) == 0) red[tid >> 5] = mloc;
   __syncthreads();
@@ -599,10 +626,10 @@ __global__ void __launch_bounds__(kGMThreads) aatc_group_merge_kernel(const Grou
   __syncthreads();
   float lloc = 0.0f;
   for (int s2 = tid; s2 < a.n_splits; s2 += kGMThreads) {
-    const float ms = pb[s2 * pstride + N];
-    const float w = ms == -INFINITY ? 0.0f : exp2f(ms - M);
+    const float2 v = s2 == tid ? ml : *reinterpret_cast<const float2*>(pb + s2 * pstride + N);
+    const float w = v.x == -INFINITY ? 0.0f : exp2f(v.x - M);
     wsp[s2] = w;
-    lloc += w * pb[s2 * pstride + N + 1];
+    lloc += w * v.y;
   }
   for (int o = 16; o > 0; o >>= 1) lloc += __shfl_xor_sync(0xffffffffu, lloc, o);
   if ((tid & 31) == 0) red[tid >> 5] = lloc;
@@ -614,12 +641,12 @@ __global__ void __launch_bounds__(kGMThreads) aatc_group_merge_kernel(const Grou
   }
   // o_hat over the slice's channels: quarter q4 takes splits q4, q4 + 4, ...
   {
-    const float* pc = pb + s * D + c;
     float o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     for (int s0 = q4; s0 < a.n_splits; s0 += 4 * 24) {   // 24 loads in flight per thread
-      float x[24];
+      if (s0 != q4) {
 #pragma unroll
-      for (int k = 0; k < 24; ++k) x[k] = s0 + 4 * k < a.n_splits ? pc[static_cast<size_t>(s0 + 4 * k) * pstride] : 0.0f;
+        for (int k = 0; k < 24; ++k) x[k] = s0 + 4 * k < a.n_splits ? pc[static_cast<size_t>(s0 + 4 * k) * pstride] : 0.0f;
+      }
 #pragma unroll
       for (int k = 0; k < 24; ++k)
         if (s0 + 4 * k < a.n_splits) o[k & 3] = fmaf(wsp[s0 + 4 * k], x[k], o[k & 3]);
@@ -634,14 +661,9 @@ __global__ void __launch_bounds__(kGMThreads) aatc_group_merge_kernel(const Grou
   __syncthreads();
   // the slice's part of U_V[block m rows] o_hat: quarter q4 takes channels 32 q4 .. 32 q4 + 31
   {
-    const float* u = a.uvt + (static_cast<size_t>(a.layer) * a.n_groups + g) * static_cast<size_t>(N) * N +
-                     static_cast<size_t>(s * D + 32 * q4) * N + static_cast<size_t>(m) * D + c;
-    float x[32];
-#pragma unroll
-    for (int k = 0; k < 32; ++k) x[k] = u[static_cast<size_t>(k) * N];   // 32 loads in flight per thread
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int k = 0; k < 32; ++k) acc[k & 3] = fmaf(x[k], ohat[32 * q4 + k], acc[k & 3]);
+    for (int k = 0; k < 32; ++k) acc[k & 3] = fmaf(uv[k], ohat[32 * q4 + k], acc[k & 3]);
     part[q4][c] = (acc[0] + acc[1]) + (acc[2] + acc[3]);
   }
   __syncthreads();
@@ -754,28 +776,21 @@ cudaError_t launch_group_decode(const Plan& plan, int layer, const void* q, cons
   if (GroupDigitSmem(gh, a.ks_max, a.n_words, 3).total > 227 * 1024) a.stages = 2;
   const size_t smem = static_cast<size_t>(GroupDigitSmem(gh, a.ks_max, a.n_words, a.stages).total);
   if (a.nq > 16 || npw > 24 || smem > 227 * 1024) return cudaErrorNotSupported;
-  aatc_group_query_kernel<<<dim3(16, a.n_groups * gh, batch), kGQThreads, 0, st>>>(a);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(aatc_group_query_kernel, dim3(16, a.n_groups * gh, batch), dim3(kGQThreads), 0, st, a);
   if (e != cudaSuccess) return e;
   const dim3 grid(a.n_splits, a.n_groups, batch);
   // pairs per warp: 12, 16 (g_h = 4 at ~2.75 bits: up to 32 value tiles per slice) or 24
-  const void* kern = gh == 2 ? (npw <= 12 ? reinterpret_cast<const void*>(aatc_group_digit_kernel<2, 12>)
-                                          : reinterpret_cast<const void*>(aatc_group_digit_kernel<2, 24>))
-                             : (npw <= 12 ? reinterpret_cast<const void*>(aatc_group_digit_kernel<4, 12>)
-                                : npw <= 16 ? reinterpret_cast<const void*>(aatc_group_digit_kernel<4, 16>)
-                                            : reinterpret_cast<const void*>(aatc_group_digit_kernel<4, 24>));
-  e = ensure_smem_optin(kern, smem);
+  using Kernel = void (*)(const GroupDecodeArgs);
+  const Kernel kern = gh == 2 ? (npw <= 12 ? aatc_group_digit_kernel<2, 12> : aatc_group_digit_kernel<2, 24>)
+                              : (npw <= 12 ? aatc_group_digit_kernel<4, 12>
+                                 : npw <= 16 ? aatc_group_digit_kernel<4, 16>
+                                             : aatc_group_digit_kernel<4, 24>);
+  e = ensure_smem_optin(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
-  if (gh == 2 && npw <= 12) aatc_group_digit_kernel<2, 12><<<grid, kGAThreads, smem, st>>>(a);
-  else if (gh == 2) aatc_group_digit_kernel<2, 24><<<grid, kGAThreads, smem, st>>>(a);
-  else if (npw <= 12) aatc_group_digit_kernel<4, 12><<<grid, kGAThreads, smem, st>>>(a);
-  else if (npw <= 16) aatc_group_digit_kernel<4, 16><<<grid, kGAThreads, smem, st>>>(a);
-  else aatc_group_digit_kernel<4, 24><<<grid, kGAThreads, smem, st>>>(a);
-  e = cudaGetLastError();
+  e = launch_pdl(kern, grid, dim3(kGAThreads), smem, st, a);
   if (e != cudaSuccess) return e;
   const size_t msm = static_cast<size_t>(a.n_splits) * 4;
-  aatc_group_merge_kernel<<<dim3(a.nq, a.n_groups * gh, batch), kGMThreads, msm, st>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(aatc_group_merge_kernel, dim3(a.nq, a.n_groups * gh, batch), dim3(kGMThreads), msm, st, a);
 }
 
 }  // namespace aatc
