@@ -108,17 +108,22 @@ def _ptr(a) -> int:
     return a.ctypes.data
 
 
-def _stream(stream=None) -> int:
-    import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
-
-
-try:                      # the binding's device helpers compare against torch dtypes
+try:                      # the binding's device helpers use torch's dtypes, allocator and streams
     import torch as _torch
-    _F32 = _torch.float32
+    _F32, _BF16, _empty = _torch.float32, _torch.bfloat16, _torch.empty
+    # the handle of the current stream without building a torch.cuda.Stream around it (3 us a call)
+    _raw_stream = getattr(_torch._C, "_cuda_getCurrentRawStream", None)
+    _current_device = getattr(_torch._C, "_cuda_getDevice", None)
 except ImportError:       # host-only use (planner, plan files) works without torch
-    _F32 = None
+    _torch = _F32 = _BF16 = _empty = _raw_stream = _current_device = None
+
+
+def _stream(stream=None) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is None or _current_device is None or not _torch.cuda.is_initialized():
+        return _torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_current_device())
 
 
 def _arg_error(where: str, what: str):
@@ -404,12 +409,11 @@ class GroupPlan(Plan):
 def encode(plan: Plan, layer: int, K, V, cache, start: int, max_tokens: int, stream=None):
     """aatc_encode: K, V bf16 [batch][n_tokens][H_kv][128] (device); writes positions
     [start, start + n_tokens) of the packed cache."""
-    import torch
-    _dev_tensor(K, "aatc_encode", "K", torch.bfloat16, 4, (None, None, plan.dims.n_kv_heads, HEAD_DIM))
-    _dev_tensor(V, "aatc_encode", "V", torch.bfloat16, 4, tuple(K.shape))
+    _dev_tensor(K, "aatc_encode", "K", _BF16, 4, (None, None, plan.dims.n_kv_heads, HEAD_DIM))
+    _dev_tensor(V, "aatc_encode", "V", _BF16, 4, tuple(K.shape))
     batch, n_tokens = K.shape[0], K.shape[1]
     _cache_ok(plan, cache, batch, max_tokens, "aatc_encode")
-    _check(load().aatc_encode(plan.handle, layer, _ptr(K), _ptr(V), batch, start, n_tokens, _ptr(cache),
+    _check(_lib.aatc_encode(plan.handle, layer, _ptr(K), _ptr(V), batch, start, n_tokens, _ptr(cache),
                               max_tokens, _stream(stream)), "aatc_encode")
 
 
@@ -417,14 +421,13 @@ def encode_hidden(plan: Plan, layer: int, x, a_hat, cache, start: int, max_token
     """aatc_encode_hidden: x bf16 [batch][n_tokens][d_model] hidden states (device), a_hat bf16
     [L][H_kv][2][128][d_model] from hidden_operand (device); writes positions [start, start +
     n_tokens) of the packed cache with the codes of x W U (keys and values of every kv-head)."""
-    import torch
-    _dev_tensor(x, "aatc_encode_hidden", "x", torch.bfloat16, 3)
+    _dev_tensor(x, "aatc_encode_hidden", "x", _BF16, 3)
     batch, n_tokens, d_model = x.shape
-    _dev_tensor(a_hat, "aatc_encode_hidden", "a_hat", torch.bfloat16)
+    _dev_tensor(a_hat, "aatc_encode_hidden", "a_hat", _BF16)
     if a_hat.numel() != plan.dims.n_layers * plan.dims.n_kv_heads * 2 * HEAD_DIM * d_model:
         _arg_error("aatc_encode_hidden", "a_hat must be [L][H_kv][2][128][d_model] for the d_model of x")
     _cache_ok(plan, cache, batch, max_tokens, "aatc_encode_hidden")
-    _check(load().aatc_encode_hidden(plan.handle, layer, _ptr(x), d_model, _ptr(a_hat), batch, start, n_tokens,
+    _check(_lib.aatc_encode_hidden(plan.handle, layer, _ptr(x), d_model, _ptr(a_hat), batch, start, n_tokens,
                                      _ptr(cache), max_tokens, _stream(stream)), "aatc_encode_hidden")
 
 
@@ -432,21 +435,20 @@ def prefill_attention(plan: Plan, layer: int, q, q_start: int, cache, n_ctx: int
                       workspace=None, stream=None):
     """aatc_prefill_attention: q bf16 [batch][n_q][H_q][128] at positions q_start .. q_start + n_q - 1,
     causal over the packed cache tokens [0, n_ctx) -> fp32 [batch][n_q][H_q][128]."""
-    import torch
-    _dev_tensor(q, "aatc_prefill_attention", "q", torch.bfloat16, 4, (None, None, plan.dims.n_q_heads, HEAD_DIM))
+    _dev_tensor(q, "aatc_prefill_attention", "q", _BF16, 4, (None, None, plan.dims.n_q_heads, HEAD_DIM))
     batch, n_q = q.shape[0], q.shape[1]
     _cache_ok(plan, cache, batch, max_tokens, "aatc_prefill_attention")
     if out is None:
-        out = torch.empty((batch, n_q, plan.dims.n_q_heads, HEAD_DIM), dtype=torch.float32, device=q.device)
+        out = _empty((batch, n_q, plan.dims.n_q_heads, HEAD_DIM), dtype=_F32, device=q.device)
     _out_ok(out, batch * n_q * plan.dims.n_q_heads * HEAD_DIM, "aatc_prefill_attention")
-    nb = _SZ()
-    _check(load().aatc_prefill_workspace_bytes(plan.handle, batch, n_ctx, ctypes.byref(nb)),
-           "aatc_prefill_workspace_bytes")
-    if workspace is None:
-        workspace = torch.empty(max(4, (nb.value + 3) // 4), dtype=torch.float32, device=q.device)
-    _check(load().aatc_prefill_attention(plan.handle, layer, _ptr(q), q_start, n_q, _ptr(cache), batch, n_ctx,
+    if workspace is None:                 # (the library refuses one that is too small)
+        nb = _SZ()
+        _check(_lib.aatc_prefill_workspace_bytes(plan.handle, batch, n_ctx, ctypes.byref(nb)),
+               "aatc_prefill_workspace_bytes")
+        workspace = _empty(max(4, (nb.value + 3) // 4), dtype=_F32, device=q.device)
+    _check(_lib.aatc_prefill_attention(plan.handle, layer, _ptr(q), q_start, n_q, _ptr(cache), batch, n_ctx,
                                          max_tokens, _ptr(out), _ptr(workspace),
-                                         workspace.numel() * workspace.element_size(), _stream(stream)),
+                                         workspace.nbytes, _stream(stream)),
            "aatc_prefill_attention")
     return out
 
@@ -454,19 +456,17 @@ def prefill_attention(plan: Plan, layer: int, q, q_start: int, cache, n_ctx: int
 def decode_attention(plan: Plan, layer: int, q, cache, n_ctx: int, max_tokens: int, out=None, workspace=None,
                      stream=None):
     """aatc_decode_attention: q bf16 [batch][H_q][128] -> fp32 [batch][H_q][128]."""
-    import torch
-    _dev_tensor(q, "aatc_decode_attention", "q", torch.bfloat16, 3, (None, plan.dims.n_q_heads, HEAD_DIM))
+    _dev_tensor(q, "aatc_decode_attention", "q", _BF16, 3, (None, plan.dims.n_q_heads, HEAD_DIM))
     batch = q.shape[0]
     _cache_ok(plan, cache, batch, max_tokens, "aatc_decode_attention")
     if out is None:
-        out = torch.empty((batch, plan.dims.n_q_heads, HEAD_DIM), dtype=torch.float32, device=q.device)
+        out = _empty((batch, plan.dims.n_q_heads, HEAD_DIM), dtype=_F32, device=q.device)
     _out_ok(out, batch * plan.dims.n_q_heads * HEAD_DIM, "aatc_decode_attention")
-    nbytes = plan.workspace_bytes(batch, n_ctx)
-    if workspace is None:
-        workspace = torch.empty(max(1, nbytes // 4), dtype=torch.float32, device=q.device)
-    _check(load().aatc_decode_attention(plan.handle, layer, _ptr(q), _ptr(cache), batch, n_ctx, max_tokens,
-                                        _ptr(out), _ptr(workspace), workspace.numel() * workspace.element_size(),
-                                        _stream(stream)), "aatc_decode_attention")
+    if workspace is None:                 # (the library refuses one that is too small)
+        workspace = _empty(max(1, plan.workspace_bytes(batch, n_ctx) // 4), dtype=_F32, device=q.device)
+    _check(_lib.aatc_decode_attention(plan.handle, layer, _ptr(q), _ptr(cache), batch, n_ctx, max_tokens,
+                                      _ptr(out), _ptr(workspace), workspace.nbytes, _stream(stream)),
+           "aatc_decode_attention")
     return out
 
 
@@ -476,28 +476,27 @@ def decode_attention_sw(plan: Plan, layer: int, q, cache, t_first: int, t_end: i
     """aatc_decode_attention_sw: packed tokens [t_first, t_end) plus the n_full tokens at rows
     [full_row0, full_row0 + n_full) of k_full / v_full (bf16 [batch][cap][H_kv][128]; the row
     stride between sequences stays cap) in one softmax -> fp32 [batch][H_q][128]."""
-    import torch
     where = "aatc_decode_attention_sw"
-    _dev_tensor(q, where, "q", torch.bfloat16, 3, (None, plan.dims.n_q_heads, HEAD_DIM))
+    _dev_tensor(q, where, "q", _BF16, 3, (None, plan.dims.n_q_heads, HEAD_DIM))
     batch = q.shape[0]
     _cache_ok(plan, cache, batch, max_tokens, where)
     if k_full is not None or v_full is not None:
-        _dev_tensor(k_full, where, "k_full", torch.bfloat16, 4, (batch, None, plan.dims.n_kv_heads, HEAD_DIM))
-        _dev_tensor(v_full, where, "v_full", torch.bfloat16, 4, tuple(k_full.shape))
+        _dev_tensor(k_full, where, "k_full", _BF16, 4, (batch, None, plan.dims.n_kv_heads, HEAD_DIM))
+        _dev_tensor(v_full, where, "v_full", _BF16, 4, tuple(k_full.shape))
     if out is None:
-        out = torch.empty((batch, plan.dims.n_q_heads, HEAD_DIM), dtype=torch.float32, device=q.device)
+        out = _empty((batch, plan.dims.n_q_heads, HEAD_DIM), dtype=_F32, device=q.device)
     _out_ok(out, batch * plan.dims.n_q_heads * HEAD_DIM, where)
     cap = 0 if k_full is None else int(k_full.shape[1])
     if full_row0 < 0 or (k_full is not None and (not k_full.is_contiguous() or not v_full.is_contiguous()
                                                  or full_row0 + int(n_full) > cap)):
         _arg_error(where, "k_full / v_full must be contiguous and hold rows [full_row0, full_row0 + n_full)")
     if t_end > t_first and workspace is None:
-        workspace = torch.empty(max(1, plan.workspace_bytes(batch, t_end) // 4), dtype=torch.float32,
+        workspace = _empty(max(1, plan.workspace_bytes(batch, t_end) // 4), dtype=_F32,
                                 device=q.device)
     ws_ptr = None if workspace is None else _ptr(workspace)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     row_bytes = int(full_row0) * plan.dims.n_kv_heads * HEAD_DIM * 2
-    _check(load().aatc_decode_attention_sw(plan.handle, layer, _ptr(q), _ptr(cache), batch, t_first, t_end,
+    _check(_lib.aatc_decode_attention_sw(plan.handle, layer, _ptr(q), _ptr(cache), batch, t_first, t_end,
                                            max_tokens, None if k_full is None else _ptr(k_full) + row_bytes,
                                            None if v_full is None else _ptr(v_full) + row_bytes, int(n_full), cap,
                                            _ptr(out),
@@ -508,12 +507,11 @@ def decode_attention_sw(plan: Plan, layer: int, q, cache, t_first: int, t_end: i
 def decode_attention_noalloc(plan: Plan, layer: int, q, out, cache, n_ctx: int, max_tokens: int, stream=None):
     """aatc_decode_attention_noalloc: as decode_attention, but with no workspace and no allocation
     (the caller passes `out`; the library's fixed scratch holds the split partials)."""
-    import torch
     where = "aatc_decode_attention_noalloc"
-    _dev_tensor(q, where, "q", torch.bfloat16, 3, (None, plan.dims.n_q_heads, HEAD_DIM))
+    _dev_tensor(q, where, "q", _BF16, 3, (None, plan.dims.n_q_heads, HEAD_DIM))
     _cache_ok(plan, cache, q.shape[0], max_tokens, where)
     _out_ok(out, q.shape[0] * plan.dims.n_q_heads * HEAD_DIM, where)
-    _check(load().aatc_decode_attention_noalloc(plan.handle, layer, _ptr(q), _ptr(cache), q.shape[0], n_ctx,
+    _check(_lib.aatc_decode_attention_noalloc(plan.handle, layer, _ptr(q), _ptr(cache), q.shape[0], n_ctx,
                                                 max_tokens, _ptr(out), _stream(stream)),
            "aatc_decode_attention_noalloc")
     return out
@@ -521,10 +519,9 @@ def decode_attention_noalloc(plan: Plan, layer: int, q, out, cache, n_ctx: int, 
 
 def dequantize(plan: Plan, layer: int, cache, batch: int, t0: int, n: int, max_tokens: int, stream=None):
     """aatc_dequantize test hook -> fp32 [batch][n][H_kv][2][128]."""
-    import torch
     _cache_ok(plan, cache, batch, max_tokens, "aatc_dequantize")
-    out = torch.empty((batch, n, plan.dims.n_kv_heads, 2, HEAD_DIM), dtype=torch.float32, device=cache.device)
-    _check(load().aatc_dequantize(plan.handle, layer, _ptr(cache), batch, t0, n, max_tokens, _ptr(out),
+    out = _empty((batch, n, plan.dims.n_kv_heads, 2, HEAD_DIM), dtype=_F32, device=cache.device)
+    _check(_lib.aatc_dequantize(plan.handle, layer, _ptr(cache), batch, t0, n, max_tokens, _ptr(out),
                                   _stream(stream)), "aatc_dequantize")
     return out
 
@@ -538,18 +535,17 @@ def bf16_workspace_bytes(batch: int, n_kv: int, n_q: int, n_ctx: int) -> int:
 
 def bf16_decode_attention(K, V, q, n_ctx: int, out=None, workspace=None, stream=None):
     """Uncompressed reference decode: K, V bf16 [batch][max_tokens][H_kv][128]; q bf16 [batch][H_q][128]."""
-    import torch
     where = "aatc_bf16_decode_attention"
-    _dev_tensor(K, where, "K", torch.bfloat16, 4, (None, None, None, HEAD_DIM))
-    _dev_tensor(V, where, "V", torch.bfloat16, 4, tuple(K.shape))
+    _dev_tensor(K, where, "K", _BF16, 4, (None, None, None, HEAD_DIM))
+    _dev_tensor(V, where, "V", _BF16, 4, tuple(K.shape))
     batch, max_tokens, n_kv = K.shape[0], K.shape[1], K.shape[2]
-    _dev_tensor(q, where, "q", torch.bfloat16, 3, (batch, None, HEAD_DIM))
+    _dev_tensor(q, where, "q", _BF16, 3, (batch, None, HEAD_DIM))
     n_q = q.shape[1]
     if out is None:
-        out = torch.empty((batch, n_q, HEAD_DIM), dtype=torch.float32, device=q.device)
+        out = _empty((batch, n_q, HEAD_DIM), dtype=_F32, device=q.device)
     _out_ok(out, batch * n_q * HEAD_DIM, where)
     if workspace is None:
-        workspace = torch.empty(max(1, bf16_workspace_bytes(batch, n_kv, n_q, n_ctx) // 4), dtype=torch.float32,
+        workspace = _empty(max(1, bf16_workspace_bytes(batch, n_kv, n_q, n_ctx) // 4), dtype=_F32,
                                 device=q.device)
     _check(load().aatc_bf16_decode_attention(_ptr(K), _ptr(V), _ptr(q), batch, n_ctx, max_tokens, n_kv, n_q,
                                              _ptr(out), _ptr(workspace), workspace.numel() * 4, _stream(stream)),

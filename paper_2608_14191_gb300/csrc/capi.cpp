@@ -38,6 +38,17 @@ uint16_t f32_to_bf16_rne(float f) {
   return static_cast<uint16_t>((u + round) >> 16);
 }
 
+// Whether every value is finite (the exponent bits of an infinity or NaN are all ones).
+bool all_finite(const float* x, size_t n) {
+  uint32_t bad = 0;
+  for (size_t i = 0; i < n; ++i) {
+    uint32_t u;
+    std::memcpy(&u, x + i, 4);
+    bad |= (u & 0x7F800000u) == 0x7F800000u;
+  }
+  return bad == 0;
+}
+
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -226,13 +237,7 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   }
   const int n_g = D * g_h, NG = dims->n_kv_heads / g_h;
   const size_t GB = static_cast<size_t>(dims->n_layers) * NG * 2 * n_g * n_g;   // group basis elements
-  if (basis) {
-    for (size_t i = 0; i < SD * D; ++i)
-      if (!std::isfinite(basis[i])) return AATC_ERR_INVALID_ARG;
-  } else {
-    for (size_t i = 0; i < GB; ++i)
-      if (!std::isfinite(gbasis[i])) return AATC_ERR_INVALID_ARG;
-  }
+  if (!(basis ? all_finite(basis, SD * D) : all_finite(gbasis, GB))) return AATC_ERR_INVALID_ARG;
   std::vector<StreamLayout> layout(S);
   std::vector<std::vector<short>> entries(S);
   int W = 1;
@@ -306,12 +311,18 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   for (int s = 0; s < S; ++s) {
     if (basis) {
       const float* bs = basis + static_cast<size_t>(s) * D * D;   // [dim][channel]
-      for (int d = 0; d < D; ++d)
-        for (int c = 0; c < D; ++c) {
-          ubf[(static_cast<size_t>(s) * D + c) * D + d] = f32_to_bf16_rne(bs[d * D + c]);
-          u32[(static_cast<size_t>(s) * D + d) * D + c] = bs[d * D + c];
-          u32t[(static_cast<size_t>(s) * D + c) * D + d] = bs[d * D + c];
-        }
+      std::memcpy(u32 + static_cast<size_t>(s) * D * D, bs, sizeof(float) * D * D);
+      constexpr int B = 16;                                        // transposed in blocks
+      for (int c0 = 0; c0 < D; c0 += B)
+        for (int d0 = 0; d0 < D; d0 += B)
+          for (int c = c0; c < c0 + B; ++c) {
+            float* t = u32t + (static_cast<size_t>(s) * D + c) * D;
+            uint16_t* h = ubf + (static_cast<size_t>(s) * D + c) * D;
+            for (int d = d0; d < d0 + B; ++d) {
+              t[d] = bs[d * D + c];
+              h[d] = f32_to_bf16_rne(t[d]);
+            }
+          }
     }
     for (int c = 0; c < D; ++c) {
       const size_t i = static_cast<size_t>(s) * D + c;
