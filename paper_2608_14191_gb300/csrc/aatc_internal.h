@@ -56,6 +56,19 @@ constexpr int kChanEnt = 16;
 // wider than 8 bits must lie in that prefix (widths are non-increasing in storage order).
 constexpr int kMaxWideChannels = 32;
 
+// Packing operand of one stream for the encode's tensor-core packing.  A token's stored values, as the
+// digit planes (u >> 2k) & 3 of 32-channel blocks, times this matrix are its record: rows are the record's
+// half-words, columns the blocks' channels, the weight 2^(bit position in the half-word) of the digit's
+// lowest bit.  Layer k has the blocks that hold channels of width >= 2k + 1; blocks are ordered by
+// channels, then layers.  Half-words (in sixteens) and digits (four a column) share the 128
+// accumulator columns of the projection they replace, so a stream has an operand if 8 columns per block
+// and its half-words fit, its record has at most 24 words, and no channel is wider than 8 bits.
+constexpr int kPackRows = 48;       // half-words of the longest record
+constexpr int kPackAtoms = 3;       // 128-channel-digit K-atoms: at most 12 blocks
+constexpr int kPackBytes = kPackRows * 128 * kPackAtoms;   // e5m2, 128-byte swizzled K-atoms
+AATC_HD inline int pack_blocks(const StreamLayout& l, int k) { return (l.lodd[k] + 31) / 32; }
+AATC_HD inline int pack_cols(const StreamLayout& l) { return (2 * l.words + 15) / 16 * 16; }
+
 struct PlanDevice {
   const void* ubf16_t;    // bf16 [S][128 channel][128 dim]   encode basis (MMA B operand, K-major)
   const float* u32;       // fp32 [S][128 dim][128 channel]   decode query rotation
@@ -68,6 +81,7 @@ struct PlanDevice {
   const short* chan_ent;  // [S][128][kChanEnt]: entries of each channel (-1 padded)
   const short* ce8;       // [S][128][8]: the first eight of them (0 padded)
   const float* cw8;       // [S][128][8]: 2^shift of those (0: none)
+  const unsigned char* pack;  // [S][kPackBytes] packing operands
   const unsigned char* proj;  // projection operands of the prefill (per-kv-head plans)
   int* err;               // [4] sticky device flags
 };
@@ -103,6 +117,7 @@ struct Plan {
   size_t block_bytes = 0;
   alignas(64) unsigned char tmap_u[128];   // CUtensorMap over ubf16_t (2D: 128 dims x S*128 rows)
   bool tmap_ok = false;
+  std::vector<char> pack_ok;  // [n_layers] every stream of the layer has a packing operand
   int group_heads = 1;    // g_h: 1 for per-kv-head plans
   GroupDevice gdev{};
   alignas(64) unsigned char tmap_g[128];   // group plans: CUtensorMap over gdev.ubf (n dims x rows)

@@ -180,6 +180,28 @@ void build_layout(const uint8_t* bits, StreamLayout* lay, std::vector<short>& en
   entries.insert(entries.end(), d1.begin(), d1.end());
 }
 
+// The packing operand of one stream (see kPackRows) into `op` (zeroed), or false where it has none.
+bool build_pack_operand(const StreamLayout& lay, const std::vector<short>& entries, unsigned char* op) {
+  if (lay.lodd[4] > 0 || 2 * lay.words > kPackRows) return false;
+  int block[4][4], n = 0;                               // [layer][32 channels]
+  for (int c = 0; c < 4; ++c)
+    for (int k = 0; k < 4; ++k)
+      if (c < pack_blocks(lay, k)) block[k][c] = n++;
+  if (8 * n + pack_cols(lay) > D) return false;
+  auto put = [&](int c, int sh, int pos) {              // the digit at bit sh of channel c starts at record bit pos
+    // in its block, the order in which the encode's lanes hold the channels: column 4 (c / 16) + c / 2 % 4,
+    // byte 2 (c / 8 % 2) + c % 2 (c the channel of the block)
+    const int in = 4 * (4 * (c % 32 / 16) + c / 2 % 4) + 2 * (c / 8 % 2) + c % 2;
+    const int k = 32 * block[sh / 2][c / 32] + in, h = pos / 16;
+    const int at = (k >> 7) * (kPackRows * 128) + h * 128 + ((((k & 127) >> 4) ^ (h & 7)) << 4) + (k & 15);
+    op[at] = static_cast<unsigned char>((pos % 16 + 15) << 2);     // e5m2 of 2^(pos mod 16)
+  };
+  for (int e = 0; e < lay.n2; ++e) put(entries[e] & 0xFF, entries[e] >> 8, 2 * e);
+  for (int e = lay.n2; e < lay.n2 + lay.n1; ++e)        // top bits; digits moved behind them, as bit pairs
+    if ((entries[e] >> 8) % 2 == 0) put(entries[e] & 0xFF, entries[e] >> 8, 2 * lay.n2 + e - lay.n2);
+  return true;
+}
+
 }  // namespace aatc
 
 extern "C" {
@@ -267,6 +289,7 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   const size_t o_ce8 = off;  off = align_up(off + SD * 8 * sizeof(short), 256);
   const size_t o_cw8 = off;  off = align_up(off + SD * 8 * sizeof(float), 256);
   const size_t o_err = off;  off = align_up(off + 16, 256);
+  const size_t o_pck = off;  off = align_up(off + (basis ? static_cast<size_t>(S) * kPackBytes : 0), 256);
   const size_t total = off;
   std::vector<unsigned char> host;
   try {
@@ -308,8 +331,11 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
           }
         }
   }
+  std::vector<char> pack_ok(dims->n_layers, basis != nullptr);
   for (int s = 0; s < S; ++s) {
     if (basis) {
+      if (!build_pack_operand(layout[s], entries[s], host.data() + o_pck + static_cast<size_t>(s) * kPackBytes))
+        pack_ok[s / (2 * dims->n_kv_heads)] = 0;
       const float* bs = basis + static_cast<size_t>(s) * D * D;   // [dim][channel]
       std::memcpy(u32 + static_cast<size_t>(s) * D * D, bs, sizeof(float) * D * D);
       constexpr int B = 16;                                        // transposed in blocks
@@ -366,6 +392,7 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   plan->retained = retained;
   plan->nbits = nbits;
   plan->layout = layout;
+  plan->pack_ok = pack_ok;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaGetDevice(&plan->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&plan->num_sms, cudaDevAttrMultiProcessorCount, plan->device);
@@ -391,6 +418,7 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   plan->dev.ce8 = reinterpret_cast<const short*>(base + o_ce8);
   plan->dev.cw8 = reinterpret_cast<const float*>(base + o_cw8);
   plan->dev.err = reinterpret_cast<int*>(base + o_err);
+  plan->dev.pack = base + o_pck;
   plan->group_heads = g_h;
   if (basis) {
     plan->dev.proj = base + total;
