@@ -1340,58 +1340,80 @@ __global__ void __launch_bounds__(256, 1) aatc_decode_fused_large_kernel(const D
 // Uncompressed tokens (the full-precision sink and recent window of Sec. 6) join the same
 // softmax here: their scores q.k/sqrt(128), weights 2^(s - m_f) and sum_t p_t v_t are taken in
 // the original basis and merged with the packed part by log-sum-exp.
-// Launched as a programmatic dependent of the split kernel: U_V^T (a plan constant) is staged
-// while the splits finish; the partials are read only after the grid dependency resolves.
+// Launched as a programmatic dependent of the split kernel; the partials are read only after the grid
+// dependency resolves.  It cannot start before the split kernel's CTAs leave, so a call ends with its
+// latency (about 2 us at a few per cent of the chip, all of it round trips to L2):
+//   PARTS CTAs per query head, each for 128 / PARTS output dimensions (all of them merge the splits and
+//   score the uncompressed tokens), U_V's part in registers instead of 64 KB through shared memory;
+//   uncompressed tokens four to a warp with 32 bytes of a row a lane, eight values a thread in flight;
+//   PER_SM = 2 (64 registers a thread) where the grid has more CTAs than the chip SMs, else 1.
+// Two sequences, 32 query heads, 16021 tokens and 139 uncompressed ones: a call 20.6 -> 18.5 us (device
+// time), with 1024 of them 42.5 -> 27.4; nine sequences of 1000 tokens and 139: 27.0 -> 21.9.
 constexpr int kMThreads = 512;
 constexpr int kMWarps = kMThreads / 32;
 
-__global__ void __launch_bounds__(kMThreads)
+template <int PARTS, int PER_SM>
+__global__ void __launch_bounds__(kMThreads, PER_SM)
     aatc_decode_merge_kernel(const DecodeArgs a) {
+  constexpr int DP = D / PARTS, CG = kMThreads / DP, CL = D / CG;   // dims; channel groups, channels of one
   extern __shared__ __align__(16) float ms[];
-  float* ut_s = ms;                                  // [128 c][128 d]
-  float* osum = ut_s + D * D;                        // [kMWarps][128]
+  float* osum = ms;                                  // [kMWarps][128]
   float* ohat = osum + kMWarps * D;                  // [128]
   float* sf = ohat + D;                              // [n_full] scores, then weights, of full tokens
   __shared__ float red[2][kMWarps];
-  __shared__ uint64_t bar;
-  __shared__ int s_abort;
-  const int j = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int j = blockIdx.x / PARTS, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int head = j / a.group;
   const int sv = (a.layer * a.n_kv + head) * 2 + 1;
-  if (tid == 0) {
-    s_abort = 0;
-    ptx::mbar_init(&bar, 1);
-    ptx::fence_mbar_init();
-    ptx::mbar_arrive_expect_tx(&bar, D * D * 4);
-    ptx::bulk_load(ut_s, a.u32t + static_cast<size_t>(sv) * D * D, D * D * 4, &bar);
-  }
+  const int dl = tid % DP, cg = tid / DP, dim = (blockIdx.x % PARTS) * DP + dl;   // output dim; channels CL cg ..
   // the next call's query kernel may start its plan-constant prologue now; it reads the query
   // and the workspace only after this grid has completed (its griddepcontrol.wait)
   ptx::grid_launch_dependents();
   const float fv = tid < D ? a.f[sv * D + tid] : 0.0f;
   // ---- uncompressed tokens (inputs of this call, not produced by the split kernel)
   float m_f = -INFINITY, l_f = 0.0f;
-  float of = 0.0f;                                   // thread d < 128: sum_t p_t v_t[d]
+  float of = 0.0f;                                   // thread tid < DP: sum_t p_t v_t[dim]
   if (a.n_full > 0) {
     // q and the full tokens were complete before the query kernel let the split kernel start;
     // with no packed range this kernel follows the caller's grid directly
     if (a.n_splits == 0) ptx::grid_dependency_wait();
     const float scale = kLog2e * 0.08838834764831845f;
-    const uint2 qq = *reinterpret_cast<const uint2*>(a.q + (static_cast<size_t>(b) * a.n_q + j) * D + 4 * lane);
-    const float2 q01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&qq.x));
-    const float2 q23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&qq.y));
-    float mloc = -INFINITY;
-    for (int t = warp; t < a.n_full; t += kMWarps) {
-      const size_t row = ((static_cast<size_t>(b) * a.full_cap + t) * a.n_kv + head) * D;
-      const uint2 kk = *reinterpret_cast<const uint2*>(a.k_full + row + 4 * lane);
-      const float2 k01 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kk.x));
-      const float2 k23 = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kk.y));
-      float d = fmaf(q01.x, k01.x, fmaf(q01.y, k01.y, fmaf(q23.x, k23.x, q23.y * k23.y)));
+    // four tokens a warp, eight lanes of 16 dimensions each; two of them in flight
+    const int sub = lane >> 3, l8 = lane & 7;
+    const __nv_bfloat16* qp = a.q + (static_cast<size_t>(b) * a.n_q + j) * D + 16 * l8;
+    uint32_t qw[8];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
-      if (lane == 0) sf[t] = d * scale;
-      mloc = fmaxf(mloc, d * scale);
+    for (int i = 0; i < 4; ++i) *reinterpret_cast<uint2*>(qw + 2 * i) = *reinterpret_cast<const uint2*>(qp + 4 * i);
+    float mloc = -INFINITY;
+    const __nv_bfloat16* kf = a.k_full + (static_cast<size_t>(b) * a.full_cap * a.n_kv + head) * D + 16 * l8;
+    for (int t0 = 4 * warp + sub; t0 - sub < a.n_full; t0 += 8 * kMWarps) {
+      uint32_t kw[2][8];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int t = min(t0 + 4 * kMWarps * u, a.n_full - 1);
+        const uint4* kr = reinterpret_cast<const uint4*>(kf + static_cast<size_t>(t) * a.n_kv * D);
+        *reinterpret_cast<uint4*>(kw[u]) = __ldg(kr);
+        *reinterpret_cast<uint4*>(kw[u] + 4) = __ldg(kr + 1);
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int t = t0 + 4 * kMWarps * u;
+        float d0 = 0.0f, d1 = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {                // (a bf16 is the upper half of its fp32)
+          d0 = fmaf(__uint_as_float(qw[i] << 16), __uint_as_float(kw[u][i] << 16), d0);
+          d1 = fmaf(__uint_as_float(qw[i] & 0xFFFF0000u), __uint_as_float(kw[u][i] & 0xFFFF0000u), d1);
+        }
+        float d = d0 + d1;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+        if (t < a.n_full) {
+          if (l8 == 0) sf[t] = d * scale;
+          mloc = fmaxf(mloc, d * scale);
+        }
+      }
     }
+    mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, 8));
+    mloc = fmaxf(mloc, __shfl_xor_sync(0xffffffffu, mloc, 16));
     if (lane == 0) red[0][warp] = mloc;
     __syncthreads();
     m_f = red[0][0];
@@ -1411,30 +1433,54 @@ __global__ void __launch_bounds__(kMThreads)
 #pragma unroll
     for (int w = 0; w < kMWarps; ++w) l_f += red[1][w];
     {
-      // four threads per dimension, tokens t = quarter (mod 4)
-      const int d = tid & (D - 1), qtr = tid >> 7;
-      float acc = 0.0f;
-      for (int t = qtr; t < a.n_full; t += 4)
-        acc = fmaf(sf[t], __bfloat162float(a.v_full[((static_cast<size_t>(b) * a.full_cap + t) * a.n_kv + head) * D + d]), acc);
-      osum[qtr * D + d] = acc;
+      // a thread sums two dimensions over the tokens t = vg (mod VG), eight of them in flight
+      constexpr int VG = 2 * CG;
+      const int vd = 2 * (tid % (DP / 2)), vg = tid / (DP / 2);
+      const __nv_bfloat16* vf = a.v_full + (static_cast<size_t>(b) * a.full_cap * a.n_kv + head) * D +
+                                (blockIdx.x % PARTS) * DP + vd;
+      float acc0 = 0.0f, acc1 = 0.0f;
+      for (int t0 = vg; t0 < a.n_full; t0 += 8 * VG) {
+        uint32_t vw[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          vw[u] = t0 + VG * u < a.n_full
+                      ? __ldg(reinterpret_cast<const unsigned int*>(vf + static_cast<size_t>(t0 + VG * u) * a.n_kv * D)) : 0u;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const float pw = t0 + VG * u < a.n_full ? sf[t0 + VG * u] : 0.0f;
+          acc0 = fmaf(pw, __uint_as_float(vw[u] << 16), acc0);
+          acc1 = fmaf(pw, __uint_as_float(vw[u] & 0xFFFF0000u), acc1);
+        }
+      }
+      *reinterpret_cast<float2*>(osum + vg * DP + vd) = make_float2(acc0, acc1);
     }
     __syncthreads();
-    if (tid < D) of = (osum[tid] + osum[D + tid]) + (osum[2 * D + tid] + osum[3 * D + tid]);
+    if (tid < DP)
+#pragma unroll
+      for (int i = 0; i < 2 * CG; ++i) of += osum[i * DP + tid];
     __syncthreads();
   }
+  // U_V's part (a plan constant), requested before the wait
+  float uv[CL];
+  {
+    const float* u = a.u32t + static_cast<size_t>(sv) * D * D + static_cast<size_t>(CL * cg) * D + dim;
+#pragma unroll
+    for (int c = 0; c < CL; ++c) uv[c] = __ldg(u + c * D);
+  }
   // ---- packed splits: warp w merges splits w, w + 16, ... online (running max, rescaled sums),
-  // eight splits' loads in flight per round; then the 16 warp partials are merged per channel.
+  // NS splits' loads in flight per round; then the 16 warp partials are merged per channel.
   float M = -INFINITY, L = 0.0f;
   if (a.n_splits > 0) {
     ptx::grid_dependency_wait();                     // the split kernel's partials
     const float* src = a.ws + (static_cast<size_t>(b) * a.n_q + j) * a.n_splits * a.pstride;
     float mw = -INFINITY, lw = 0.0f;
     float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    for (int s0 = warp; s0 < a.n_splits; s0 += kMWarps * 8) {
-      float2 ml[8];
-      float4 v[8];
+    constexpr int NS = PER_SM > 1 ? 2 : 4;
+    for (int s0 = warp; s0 < a.n_splits; s0 += kMWarps * NS) {
+      float2 ml[NS];
+      float4 v[NS];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
+      for (int u = 0; u < NS; ++u) {
         const int s = s0 + kMWarps * u;
         if (s < a.n_splits) {
           ml[u] = __ldcg(reinterpret_cast<const float2*>(src + static_cast<size_t>(s) * a.pstride + D));
@@ -1446,13 +1492,13 @@ __global__ void __launch_bounds__(kMThreads)
       }
       float mc = mw;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) mc = fmaxf(mc, ml[u].x);
+      for (int u = 0; u < NS; ++u) mc = fmaxf(mc, ml[u].x);
       if (mc > -INFINITY) {                          // else nothing attended so far: sums stay 0
         const float r = fast_exp2(mw - mc);              // mw = -inf -> 0
         lw *= r;
         acc.x *= r; acc.y *= r; acc.z *= r; acc.w *= r;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
+        for (int u = 0; u < NS; ++u) {
           const float w = fast_exp2(ml[u].x - mc);
           lw = fmaf(w, ml[u].y, lw);
           acc.x = fmaf(w, v[u].x, acc.x);
@@ -1488,20 +1534,21 @@ __global__ void __launch_bounds__(kMThreads)
     }
     ohat[tid] = o * fv * ap;
   }
-  if (!ptx::mbar_wait_sleep(&bar, 0, &s_abort, 100)) atomicOr(a.err, 2);
   __syncthreads();
-  // out[d] = sum_c U_V[d][c] o_hat[c]: four threads per dimension, quarters of c
+  // out[d] = sum_c U_V[d][c] o_hat[c]: CG threads per dimension, CL channels each
   {
-    const int d = tid & (D - 1), qtr = tid >> 7;
     float r4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int c = 0; c < 32; ++c) r4[c & 3] = fmaf(ut_s[(qtr * 32 + c) * D + d], ohat[qtr * 32 + c], r4[c & 3]);
-    osum[qtr * D + d] = (r4[0] + r4[1]) + (r4[2] + r4[3]);
+    for (int c = 0; c < CL; ++c) r4[c & 3] = fmaf(uv[c], ohat[CL * cg + c], r4[c & 3]);
+    osum[cg * DP + dl] = (r4[0] + r4[1]) + (r4[2] + r4[3]);
   }
   __syncthreads();
-  if (tid < D)
-    a.out[(static_cast<size_t>(b) * a.n_q + j) * D + tid] =
-        ((osum[tid] + osum[D + tid]) + (osum[2 * D + tid] + osum[3 * D + tid]) + of * af) * inv_den;
+  if (tid < DP) {
+    float o = of * af;
+#pragma unroll
+    for (int i = 0; i < CG; ++i) o += osum[i * DP + tid];
+    a.out[(static_cast<size_t>(b) * a.n_q + j) * D + dim] = o * inv_den;
+  }
 }
 
 // ---------------------------------------------------------------- bf16 reference decode
@@ -1899,8 +1946,16 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
   a.qcorr = reinterpret_cast<float*>(static_cast<char*>(ws) + wsl.qcorr_off);
   if (plan.n_entries > kMaxEntries) return cudaErrorNotSupported;
   // every shape refusal comes before the first launch of the call
-  const size_t msm = 4 * (static_cast<size_t>(D) * D + kMWarps * D + D + static_cast<size_t>((a.n_full + 3) & ~3));
-  if (msm > 227 * 1024) return cudaErrorNotSupported;
+  const size_t msm = 4 * (static_cast<size_t>(kMWarps) * D + D + static_cast<size_t>((a.n_full + 3) & ~3));
+  // CTAs of one query head's merge: more while each has an SM to itself; two to an SM where the heads
+  // outnumber the SMs.  Measured (call, us; 16021 tokens, 139 uncompressed): 64 heads in 64 CTAs 24.4, in
+  // 128 22.5, in 256 24.2; 96 heads one to an SM 29.0, two 32.0; 192 heads 48.5 and 47.3, 288 64.6 and 63.0
+  const long heads = static_cast<long>(a.n_q) * batch;
+  const auto merge = heads > plan.num_sms       ? aatc_decode_merge_kernel<1, 2>
+                     : 2 * heads > plan.num_sms ? aatc_decode_merge_kernel<1, 1>
+                     : 4 * heads > plan.num_sms ? aatc_decode_merge_kernel<2, 1>
+                                                : aatc_decode_merge_kernel<4, 1>;
+  const int parts = 2 * heads > plan.num_sms ? 1 : 4 * heads > plan.num_sms ? 2 : 4;
   cudaError_t e = cudaSuccess;
   if (fk.kernel) {
     e = ensure_smem_optin(reinterpret_cast<const void*>(fk.kernel), fsm);
@@ -1908,9 +1963,9 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
     const unsigned n_cta = static_cast<unsigned>(static_cast<long>(sp.n_splits) * a.n_kv * batch);
     e = launch_pdl(fk.kernel, dim3(n_cta), dim3(128 * fk.groups), fsm, st, a);
     if (e != cudaSuccess) return e;
-    e = ensure_smem_optin(reinterpret_cast<const void*>(aatc_decode_merge_kernel), msm);
+    e = ensure_smem_optin(reinterpret_cast<const void*>(merge), msm);
     if (e != cudaSuccess) return e;
-    return launch_pdl(aatc_decode_merge_kernel, dim3(a.n_q, batch), dim3(kMThreads), msm, st, a);
+    return launch_pdl(merge, dim3(a.n_q * parts, batch), dim3(kMThreads), msm, st, a);
   }
   // largest key k-step count and value word count over the layer's streams
   int n_ks = 1, n_jobs_v = 1;
@@ -1930,9 +1985,9 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
     e = np == 1 ? launch_split_g<1>(a, batch, jpw, smem, st) : launch_split_g<2>(a, batch, jpw, smem, st);
     if (e != cudaSuccess) return e;
   }
-  e = ensure_smem_optin(reinterpret_cast<const void*>(aatc_decode_merge_kernel), msm);
+  e = ensure_smem_optin(reinterpret_cast<const void*>(merge), msm);
   if (e != cudaSuccess) return e;
-  return launch_pdl(aatc_decode_merge_kernel, dim3(a.n_q, batch), dim3(kMThreads), msm, st, a);
+  return launch_pdl(merge, dim3(a.n_q * parts, batch), dim3(kMThreads), msm, st, a);
 }
 
 cudaError_t launch_dequant(const Plan& plan, int layer, const void* cache, int batch, int t0, int n, int max_tokens,

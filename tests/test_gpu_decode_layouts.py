@@ -64,3 +64,25 @@ def test_decode_record_layouts(aatc, n_kv, group, b_max, total, batch, n_ctx, fi
     _, rel = Hn.check_decode(out.cpu().numpy().reshape(-1, 128), ref.cpu().numpy().reshape(-1, 128))
     assert rel <= 1e-4, rel
     assert plan.device_error() == 0
+
+
+@pytest.mark.parametrize("batch", [1, 2, 3, 5])       # 32 .. 160 query heads: each form of the merge
+@pytest.mark.parametrize("n_full", [1, 3, 65, 139, 512, 1031])
+def test_merge_of_uncompressed_tokens(aatc, batch, n_full):
+    n_kv, group, n_ctx = 8, 4, 150
+    rng = np.random.default_rng([batch, n_full])
+    plan, basis, _ = random_plan(aatc, rng, n_kv, group, 8, (352, 288))
+    k, v = tokens(rng, basis, batch, n_ctx + n_full, n_kv)
+    cache = plan.new_cache(batch, n_ctx, DEV)
+    aatc.encode(plan, 0, k[:, :n_ctx].contiguous(), v[:, :n_ctx].contiguous(), cache, 0, n_ctx)
+    full = [torch.cat([x[:, n_ctx:], torch.full_like(x[:, :3], float("nan"))], 1).contiguous() for x in (k, v)]
+    q = torch.from_numpy(2.0 * rng.standard_normal((batch, n_kv * group, 128))).to(DEV).to(torch.bfloat16)
+    out = aatc.decode_attention_sw(plan, 0, q, cache, 0, n_ctx, n_ctx, full[0], full[1], n_full)
+    coef = aatc.dequantize(plan, 0, cache, batch, 0, n_ctx, n_ctx).double()
+    rows = [torch.cat([torch.einsum("bnhc,hdc->bnhd", coef[:, :, :, kind],
+                                    torch.from_numpy(basis[0, :, kind]).to(DEV).double()),
+                       x[:, n_ctx:].double()], 1).repeat_interleave(group, 2) for kind, x in enumerate((k, v))]
+    p = torch.softmax(torch.einsum("bhd,bnhd->bhn", q.double(), rows[0]) / math.sqrt(128), -1)
+    ref = torch.einsum("bhn,bnhd->bhd", p, rows[1])
+    _, rel = Hn.check_decode(out.cpu().numpy().reshape(-1, 128), ref.cpu().numpy().reshape(-1, 128))
+    assert rel <= 1e-4, rel
