@@ -12,7 +12,7 @@
 //   query  per (query row < 16, slice, group, sequence): q'' = (U_K^T q~) f log2(e) / sqrt(128)
 //          over the slice's 128 channels, the slice's scale and part of the offset correction, and
 //          the row's words of the slice's score A fragments (entry order of its key records)
-//   attn   per (split, group, sequence), 8 warps: the slices' record words are the operands of
+//   attn   per (split, group, sequence), 16 warps: the slices' record words are the operands of
 //          mma.sync m16n8k16 f16 (a digit or bit masked into a 16-bit half is the subnormal
 //          digit 2^-24), rows = the group's <= 16 query heads: scores summed over every slice
 //          and corrected by the stored-value offsets, online softmax with the exponent of
@@ -33,7 +33,8 @@ namespace aatc {
 namespace {
 
 constexpr float kGLog2e = 1.4426950408889634f;
-constexpr int kGAThreads = 256;                  // 8 warps; each also runs the softmax of 16 tokens
+constexpr int kGAWarps = 16;                     // of the digit kernel; each runs the softmax of 8 tokens
+constexpr int kGAThreads = 32 * kGAWarps;
 
 struct GroupDecodeArgs {
   const float* alpha;        // cache alpha region [b][n_kv][K|V][n_tiles * 128]
@@ -49,6 +50,8 @@ struct GroupDecodeArgs {
   float* out;                // [b][H_q][128]
   const uint32_t* words;     // cache word region (the digit kernel reads the records directly)
   const short* entry;        // plan: [slot][n_entries] (channel | shift << 8), -1 padded
+  const short* ce8;          // plan: [slot][128][8] a channel's entries (0 padded)
+  const float* cw8;          // plan: [slot][128][8] 2^shift of those (0: none)
   const ChanEnc* enc;        // plan: [slot][128] (offset 2^(b-1) of each stored value)
   const StreamLayout* lay;   // plan: [slot]
   int layer, n_kv, gh, n_groups, group, nq, n, n_q_heads, n_ctx, n_ctx_pad, n_tiles, n_splits;
@@ -194,16 +197,20 @@ __global__ void __launch_bounds__(kGQThreads) aatc_group_query_kernel(const Grou
 // digit (or a single bit) masked into a 16-bit half is the subnormal f16 value d 2^(p - 24), p its
 // bit position in the half; the power 2^p is folded into the other operand's scale.
 //   chunks: per tile, the key words of all g_h slices, then their value words (cp.async ring)
-//   scores: warp (slice sl, part) over its slice's k-steps and 8 (g_h = 4) or 4 (g_h = 2)
+//   scores: warp (slice sl, part) over its slice's k-steps and 4 (g_h = 4) or 2 (g_h = 2)
 //           token n-tiles: A = q''_c 2^shift per entry (rows = queries, hi / lo, lane t's columns
 //           scaled by 2^-2t for D2 words, 2^-t for D1 words), B = the tokens' fields masked in
 //           place; the slice partials meet in shared memory and are summed per token, then
 //           raw = sum q'' u, s = alpha^K (raw - C) with C = sum_c q''_c 2^(b_c - 1)
-//   values: warp (slice sl, part) owns the 8-entry tiles part, part + 8 / g_h, ... of slice sl:
+//   values: warp (slice sl, part) owns the 8-entry tiles part, part + 16 / g_h, ... of slice sl:
 //           A = P' (queries x 16 tokens, hi / lo, loaded once per k-step), B = the entries'
 //           fields of those tokens from the quad-interleaved value slots (byte permute + mask);
 //           the entry sums become channel sums o_c = sum_e 2^(shift - p) O_e - 2^(b_c - 1) S'
-//           (S' = the represented sum of P') through shared-memory adds at the end of the split.
+//           (S' = the represented sum of P') at the end of the split, gathered by channel.
+// Bound by the MMAs of a CTA's one or two tiles in series: of some 6.7 us a tile, 2.7 scores, 1.1 softmax
+// and 2.9 values, of which the mma.sync rate is 3.6.  16384 tokens in two groups of four, a whole call
+// (device time): 38.3 us with eight warps and the channel sums by shared-memory adds, 34.2 with sixteen
+// warps (half of the tokens and value tiles a warp, the softmax over all of them), 29.0 with the gather.
 constexpr int kGRS = TILE + 8;                   // padded row stride of the per-slice score partials
 
 struct GroupDigitSmem {
@@ -211,24 +218,23 @@ struct GroupDigitSmem {
   __host__ __device__ GroupDigitSmem(int gh, int ks_max, int n_words, int stages) {
     chunk_words = n_words * TILE;                 // one slice, one kind, one tile
     const int qf = gh * ks_max * 32 * 16, pf = (TILE / 16) * 32 * 16;
-    const int rw = stages * gh * chunk_words * 4, qc = 16 * D * gh * 4;
     int o = 0;
     qfh = o;   o += qf;                           // [slice][k-step][lane] uint4, hi parts
     qfl = o;   o += qf;                           //   lo parts
     pfh = o;   o += pf;                           // [k-step][lane] uint4, hi parts of P'
     pfl = o;   o += pf;
-    ring = o;  o += rw > qc ? rw : qc;            // record chunks; channel sums at the end
+    ring = o;  o += stages * gh * chunk_words * 4;   // record chunks
     red = o;   o += gh * 16 * kGRS * 4;           // [slice][query][token] score partials
     offs = o;  o += D * gh * 4;                   // stored-value offsets 2^(b-1) of the values
     info = o;  o += 16 * gh;                      // [slice][K|V] (n2, n1)
-    misc = o;  o += 16 * 4 * (gh + 5) + 3 * 8 * 16 * 4;
+    misc = o;  o += 16 * 4 * (gh + 6) + kGAWarps * 16 * 4;
     total = o;
   }
 };
 
 template <int GH, int NPW>
 __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const GroupDecodeArgs a) {
-  constexpr int N = D * GH, WPS = 8 / GH, NTK = TILE / (8 * WPS);   // warps per slice, key n-tiles per warp
+  constexpr int N = D * GH, WPS = kGAWarps / GH, NTK = TILE / (8 * WPS);   // warps per slice, key n-tiles per warp
   extern __shared__ __align__(128) unsigned char smb[];
   const GroupDigitSmem L(GH, a.ks_max, a.n_words, a.stages);
   uint4* qfh = reinterpret_cast<uint4*>(smb + L.qfh);
@@ -240,14 +246,14 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
   float* offv = reinterpret_cast<float*>(smb + L.offs);
   int* info = reinterpret_cast<int*>(smb + L.info);
   float* qsl = reinterpret_cast<float*>(smb + L.misc);   // [16][g_h] slice scales x 2^24
-  float* mrow = qsl + 16 * GH;
-  float* lrow = mrow + 16;
+  float* mrow = qsl + 16 * GH;                    // [2][16] running maximum, by tile parity
+  float* lrow = mrow + 32;
   float* srow = lrow + 16;                        // S' of each query
   float* rscale = srow + 16;
   float* corr = rscale + 16;                      // C of each query
-  float* redm = corr + 16;                        // [8][16]
-  float* reds = redm + 8 * 16;                    // [8][16]
-  float* redp = reds + 8 * 16;                    // [8][16]
+  float* redm = corr + 16;                        // [kGAWarps][16]
+  float* reds = red;                              // [kGAWarps][16], once the score partials are read
+  float* redp = reds + kGAWarps * 16;             // [kGAWarps][16]
   const int split = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gq = lane >> 2, t = lane & 3;
   const int ws = warp / WPS, wsub = warp % WPS;   // this warp's slice and its part of the slice
@@ -300,7 +306,7 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
 #pragma unroll
     for (int sl = 0; sl < GH; ++sl) cs += a.qsc[((bg * 16 + tid) * GH + sl) * 2 + 1];
     corr[tid] = cs;
-    mrow[tid] = -INFINITY;
+    mrow[tid] = -INFINITY;                        // (the first tile's)
     lrow[tid] = 0.0f;
     srow[tid] = 0.0f;
   }
@@ -344,7 +350,7 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
     for (int r = 0; r < 4; ++r) oacc[j][r] = 0.0f;
   const int n2k = info[4 * ws], n2wk = n2k >> 4, n1wk = (info[4 * ws + 1] + 31) >> 5;
   const uint32_t M2 = 0x00030003u << (2 * t), M1 = 0x00010001u << t;
-  const int tb = wsub * 8 * NTK, tw = 16 * warp;
+  const int tb = wsub * 8 * NTK, tw = 8 * warp;
 
   for (int u = 0; u < n_chunks; ++u) {
     issue(u + S - 1);
@@ -354,6 +360,9 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
     const int tile = tile_lo + (u >> 1);
     const uint32_t* cs = ring + (u % S) * GH * cw + ws * cw;   // this warp's slice
     if ((u & 1) == 0) {
+      // the scales of the lane's two tokens (the cache region holds whole tiles; masked below)
+      const int tok0 = tile * TILE + tw + 2 * t;
+      const float2 ak2 = *reinterpret_cast<const float2*>(kalpha + tok0), av2 = *reinterpret_cast<const float2*>(valpha + tok0);
       // ---- slice partial scores of tokens tb .. tb + 8 NTK
       float sacc[NTK][4];
 #pragma unroll
@@ -393,15 +402,13 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
         *reinterpret_cast<float2*>(&rs[(gq + 8) * kGRS + col]) = make_float2(sacc[nt][2], sacc[nt][3]);
       }
       __syncthreads();
-      // ---- online softmax of the tile (warp w < 8: tokens 16 w ..), raw = sum_s acc_s 2^24 scale_s - C.
-      // Lane (gq, t) holds rows gq, gq + 8 and tokens tw + 8 nt + 2t + {0, 1}; e = s + floor(log2 alpha^V)
+      // ---- online softmax of the tile (warp w: tokens 8 w ..), raw = sum_s acc_s 2^24 scale_s - C.
+      // Lane (gq, t) holds rows gq, gq + 8 and tokens tw + 2t + {0, 1}; e = s + floor(log2 alpha^V)
       // keeps P' = 2^(e - m) mant(alpha^V) < 2.
-      float e[2][4], mant[2][4], lav[2][4];
-      if (warp < 8) {
-      float sc[2][4];
-#pragma unroll
-      for (int nt = 0; nt < 2; ++nt) {
-        const int col = tw + 8 * nt + 2 * t;
+      float e[4], mant[4], lav[4];
+      float mx0 = -INFINITY, mx1 = -INFINITY;
+      {
+        const int col = tw + 2 * t;
         float2 s0 = make_float2(0.0f, 0.0f), s1 = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int sl = 0; sl < GH; ++sl) {
@@ -411,34 +418,28 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
           s0.x = fmaf(v0.x, w0, s0.x); s0.y = fmaf(v0.y, w0, s0.y);
           s1.x = fmaf(v1.x, w1, s1.x); s1.y = fmaf(v1.y, w1, s1.y);
         }
-        sc[nt][0] = s0.x; sc[nt][1] = s0.y; sc[nt][2] = s1.x; sc[nt][3] = s1.y;
-      }
-      float mx0 = -INFINITY, mx1 = -INFINITY;
-      const float c0 = corr[gq], c1 = corr[gq + 8];
+        const float sc[4] = {s0.x, s0.y, s1.x, s1.y};
+        const float c0 = corr[gq], c1 = corr[gq + 8];
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
+        for (int k = 0; k < 2; ++k) {
+          const float ak = k ? ak2.y : ak2.x, avv = k ? av2.y : av2.x;
+          int ex = 0;
+          const float fr = frexpf(avv, &ex);
+          const float lv = avv > 0.0f ? static_cast<float>(max(ex - 1, -64)) : -64.0f;
+          float mv = avv > 0.0f ? fr * 2.0f : 0.0f;
+          if (avv > 0.0f && ex - 1 < -64) mv = avv * 18446744073709551616.0f;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const int tok = tile * TILE + tw + 8 * nt + 2 * t + (r & 1);
-          const int row = r < 2 ? gq : gq + 8;
-          const bool ok = tok < a.n_ctx && row < a.nq;
-          float ev = -INFINITY, mv = 0.0f, lv = 0.0f;
-          if (ok) {
-            const float ak = kalpha[tok], avv = valpha[tok];
-            const float sv = (sc[nt][r] - (r < 2 ? c0 : c1)) * ak;
-            int ex = 0;
-            const float fr = frexpf(avv, &ex);
-            lv = avv > 0.0f ? static_cast<float>(max(ex - 1, -64)) : -64.0f;
-            mv = avv > 0.0f ? fr * 2.0f : 0.0f;
-            if (avv > 0.0f && ex - 1 < -64) mv = avv * 18446744073709551616.0f;
-            ev = sv + lv;
+          for (int h = 0; h < 2; ++h) {
+            const int r = 2 * h + k, row = gq + 8 * h;
+            const bool ok = tok0 + k < a.n_ctx && row < a.nq;
+            e[r] = ok ? (sc[r] - (h ? c1 : c0)) * ak + lv : -INFINITY;
+            mant[r] = ok ? mv : 0.0f;
+            lav[r] = ok ? lv : 0.0f;
           }
-          e[nt][r] = ev;
-          mant[nt][r] = mv;
-          lav[nt][r] = lv;
-          if (r < 2) mx0 = fmaxf(mx0, ev);
-          else mx1 = fmaxf(mx1, ev);
         }
+        mx0 = fmaxf(e[0], e[1]);
+        mx1 = fmaxf(e[2], e[3]);
+      }
       mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 1));
       mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, 2));
       mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, 1));
@@ -447,48 +448,53 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
         redm[warp * 16 + gq] = mx0;
         redm[warp * 16 + gq + 8] = mx1;
       }
-      }
       __syncthreads();
-      if (tid < 16) {
-        float mt = -INFINITY;
+      // every lane quad finds its two rows' maxima over the warps; warp 0 keeps them for the next tile
+      const float* mold = mrow + 16 * ((u >> 1) & 1);
+      float* mnew = mrow + 16 * (((u >> 1) & 1) ^ 1);
+      float m0 = -INFINITY, m1r = -INFINITY;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) mt = fmaxf(mt, redm[w * 16 + tid]);
-        const float mo = mrow[tid], mn = fmaxf(mo, mt);
-        rscale[tid] = mo == -INFINITY ? 0.0f : fexp2(mo - mn);
-        mrow[tid] = mn;
+      for (int w = 0; w < kGAWarps / 4; ++w) {
+        m0 = fmaxf(m0, redm[(4 * w + t) * 16 + gq]);
+        m1r = fmaxf(m1r, redm[(4 * w + t) * 16 + gq + 8]);
       }
-      __syncthreads();
-      if (warp < 8) {
-      const float m0 = mrow[gq], m1r = mrow[gq + 8];
+      m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 1));
+      m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, 2));
+      m1r = fmaxf(m1r, __shfl_xor_sync(0xffffffffu, m1r, 1));
+      m1r = fmaxf(m1r, __shfl_xor_sync(0xffffffffu, m1r, 2));
+      const float mo0 = mold[gq], mo1 = mold[gq + 8];
+      m0 = fmaxf(mo0, m0);
+      m1r = fmaxf(mo1, m1r);
+      const float r0 = mo0 == -INFINITY ? 0.0f : fexp2(mo0 - m0), r1 = mo1 == -INFINITY ? 0.0f : fexp2(mo1 - m1r);
+      if (warp == 0 && t == 0) {
+        mnew[gq] = m0;
+        mnew[gq + 8] = m1r;
+        rscale[gq] = r0;
+        rscale[gq + 8] = r1;
+      }
       float ls0 = 0.0f, ls1 = 0.0f, ps0 = 0.0f, ps1 = 0.0f;
-      float p[2][4];
+      float p[4];
 #pragma unroll
-      for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const float mm = r < 2 ? m0 : m1r;
-          const float x = e[nt][r] == -INFINITY ? 0.0f : fexp2(e[nt][r] - mm);
-          p[nt][r] = x * mant[nt][r];
-          const float l = e[nt][r] == -INFINITY ? 0.0f : x * exp2f(-lav[nt][r]);
-          if (r < 2) ls0 += l;
-          else ls1 += l;
-        }
-      uint4 ph, pl;
-      split2(p[0][0], p[0][1], ph.x, pl.x);
-      split2(p[0][2], p[0][3], ph.y, pl.y);
-      split2(p[1][0], p[1][1], ph.z, pl.z);
-      split2(p[1][2], p[1][3], ph.w, pl.w);
-      pfh[warp * 32 + lane] = ph;
-      pfl[warp * 32 + lane] = pl;
+      for (int r = 0; r < 4; ++r) {
+        const float x = e[r] == -INFINITY ? 0.0f : fexp2(e[r] - (r < 2 ? m0 : m1r));
+        p[r] = x * mant[r];
+        const float l = e[r] == -INFINITY ? 0.0f : x * exp2f(-lav[r]);
+        if (r < 2) ls0 += l;
+        else ls1 += l;
+      }
+      uint2 ph, pl;
+      split2(p[0], p[1], ph.x, pl.x);
+      split2(p[2], p[3], ph.y, pl.y);
+      // (half of the k-step warp / 2: its first or second eight tokens)
+      reinterpret_cast<uint2*>(pfh + (warp >> 1) * 32 + lane)[warp & 1] = ph;
+      reinterpret_cast<uint2*>(pfl + (warp >> 1) * 32 + lane)[warp & 1] = pl;
       // S': the represented P' (hi + lo) that the value MMAs add
       {
         const __half2* hh = reinterpret_cast<const __half2*>(&ph);
         const __half2* ll = reinterpret_cast<const __half2*>(&pl);
         float2 v;
         v = __half22float2(hh[0]); ps0 += v.x + v.y; v = __half22float2(ll[0]); ps0 += v.x + v.y;
-        v = __half22float2(hh[2]); ps0 += v.x + v.y; v = __half22float2(ll[2]); ps0 += v.x + v.y;
         v = __half22float2(hh[1]); ps1 += v.x + v.y; v = __half22float2(ll[1]); ps1 += v.x + v.y;
-        v = __half22float2(hh[3]); ps1 += v.x + v.y; v = __half22float2(ll[3]); ps1 += v.x + v.y;
       }
       ls0 += __shfl_xor_sync(0xffffffffu, ls0, 1);
       ls0 += __shfl_xor_sync(0xffffffffu, ls0, 2);
@@ -504,9 +510,7 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
         redp[warp * 16 + gq] = ps0;
         redp[warp * 16 + gq + 8] = ps1;
       }
-      }
       // value accumulators: rows of D are the queries (c0, c1: row gq; c2, c3: row gq + 8)
-      const float r0 = rscale[gq], r1 = rscale[gq + 8];
 #pragma unroll
       for (int j = 0; j < NPW; ++j) {
         oacc[j][0] *= r0;
@@ -518,7 +522,7 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
       if (tid < 16) {
         float lt = 0.0f, pt = 0.0f;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) {
+        for (int w = 0; w < kGAWarps; ++w) {
           lt += reds[w * 16 + tid];
           pt += redp[w * 16 + tid];
         }
@@ -540,44 +544,53 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
           }
         }
       }
+      __syncthreads();                            // (the keys' words were last read before the score barrier)
     }
-    __syncthreads();
   }
   cp_async_wait<0>();
   __syncthreads();
 
-  // ---- entry sums -> channel sums (shared-memory adds), then the split's partials
-  float* oc = reinterpret_cast<float*>(ring);     // [16][N]
-  for (int i = tid; i < 16 * N; i += kGAThreads) oc[i] = 0.0f;
-  __syncthreads();
+  // ---- entry sums into shared memory, [slice][query][EP] over the score fragments (the table needs no
+  // more than theirs and P' s), then per channel o_c = sum_e 2^shift E_e - 2^(b_c - 1) S' and the split's
+  // partials: thread = channel, its entries and weights (plan constants) read once for all queries
+  float* es = reinterpret_cast<float*>(smb);
+  const int EP = 16 * a.ks_max + (a.ks_max & 1 ? 24 : 8);   // 8 mod 32: a warp's pairs hit every bank once
+  constexpr int PQ = kGAThreads / N;                        // queries i = tid / N (mod PQ)
+  const int j = tid & (N - 1);
+  const size_t sv = static_cast<size_t>(pslot0 + 2 * (j >> 7) + 1) * D + (j & (D - 1));
+  const uint4 cev = *reinterpret_cast<const uint4*>(a.ce8 + sv * 8);
+  const float4 wa = *reinterpret_cast<const float4*>(a.cw8 + sv * 8), wb = *reinterpret_cast<const float4*>(a.cw8 + sv * 8 + 4);
   {
-    const short* et = a.entry + static_cast<size_t>(pslot0 + 2 * ws + 1) * a.n_entries;
+    float* e0 = es + (ws * 16 + gq) * EP + 2 * t;
+    if (nev == 0 && wsub == 0) e0[0] = e0[8 * EP] = 0.0f;   // an empty slice: its channels all point at entry 0
 #pragma unroll
-    for (int j = 0; j < NPW; ++j) {
-      if (j >= npv) break;
-#pragma unroll
-      for (int k = 0; k < 2; ++k) {
-        const int e = 8 * (wsub + WPS * j) + 2 * t + k;   // D column 2t + k
-        const int ce = e < nev ? et[e] : -1;
-        if (ce < 0) continue;
-        const int p = e < n2v ? 2 * (e & 3) : (e - n2v) & 7;   // the field's bit position in its byte
-        const float w2 = ldexpf(1.0f, ((ce >> 8) & 15) + 24 - p);   // fields entered as d 2^(p - 24)
-        const int jj = ws * D + (ce & 0xFF);
-        if (gq < a.nq) atomicAdd(&oc[gq * N + jj], w2 * oacc[j][k]);
-        if (gq + 8 < a.nq) atomicAdd(&oc[(gq + 8) * N + jj], w2 * oacc[j][2 + k]);
-      }
+    for (int jj = 0; jj < NPW; ++jj) {
+      if (jj >= npv) break;
+      const int e = 8 * (wsub + WPS * jj);                  // fields entered as d 2^(p - 24), p their bit position
+      const float k0 = e < n2v ? (t & 1 ? 1048576.0f : 16777216.0f) : __uint_as_float((127 + 24 - 2 * t) << 23);
+      const float k1 = e < n2v ? 0.25f * k0 : 0.5f * k0;
+      *reinterpret_cast<float2*>(e0 + e) = make_float2(oacc[jj][0] * k0, oacc[jj][1] * k1);
+      *reinterpret_cast<float2*>(e0 + 8 * EP + e) = make_float2(oacc[jj][2] * k0, oacc[jj][3] * k1);
     }
   }
   __syncthreads();
   const size_t pstride = static_cast<size_t>(N) + 4;
   float* pb = a.part + ((static_cast<size_t>(b) * a.n_groups + g) * a.nq) * a.n_splits * pstride;
-  for (int idx = tid; idx < a.nq * N; idx += kGAThreads) {
-    const int i = idx / N, j = idx % N;
-    pb[(static_cast<size_t>(i) * a.n_splits + split) * pstride + j] = oc[i * N + j] - offv[j] * srow[i];
+  {
+    const uint32_t cw4[4] = {cev.x, cev.y, cev.z, cev.w};
+    const float w8[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+    const float off = offv[j];
+    for (int i = tid / N; i < a.nq; i += PQ) {
+      const float* er = es + ((j >> 7) * 16 + i) * EP;
+      float o = -off * srow[i];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) o = fmaf(w8[k], er[(cw4[k >> 1] >> (16 * (k & 1))) & 0xFFFF], o);
+      pb[(static_cast<size_t>(i) * a.n_splits + split) * pstride + j] = o;
+    }
   }
   if (tid < a.nq) {
     float* d = pb + (static_cast<size_t>(tid) * a.n_splits + split) * pstride + N;
-    d[0] = mrow[tid];
+    d[0] = mrow[16 * ((tile_hi - tile_lo) & 1) + tid];
     d[1] = lrow[tid];
   }
 }
@@ -760,31 +773,33 @@ cudaError_t launch_group_decode(const Plan& plan, int layer, const void* q, cons
   a.n_splits = group_splits(plan, batch, n_ctx);
   a.words = static_cast<const uint32_t*>(cache);
   a.entry = plan.dev.entry;
+  a.ce8 = plan.dev.ce8;
+  a.cw8 = plan.dev.cw8;
   a.enc = plan.dev.enc;
   a.lay = plan.dev.lay;
   a.n_words = plan.n_words;
   a.n_entries = plan.n_entries;
   a.ks_max = group_ks_max(plan, layer);
-  // value pairs per warp: 8-entry tiles of the widest value slice over the 8 / g_h warps of a slice
+  // value pairs per warp: 8-entry tiles of the widest value slice over the 16 / g_h warps of a slice
   int ntp = 1;
   for (int h = 0; h < a.n_kv; ++h) {
     const StreamLayout& ly = plan.layout[(layer * a.n_kv + h) * 2 + 1];
     ntp = std::max(ntp, (ly.n2 + ly.n1 + 7) / 8);
   }
-  const int npw = (ntp + 8 / gh - 1) / (8 / gh);
+  const int npw = (ntp + kGAWarps / gh - 1) / (kGAWarps / gh);
   a.stages = 3;
   if (GroupDigitSmem(gh, a.ks_max, a.n_words, 3).total > 227 * 1024) a.stages = 2;
   const size_t smem = static_cast<size_t>(GroupDigitSmem(gh, a.ks_max, a.n_words, a.stages).total);
-  if (a.nq > 16 || npw > 24 || smem > 227 * 1024) return cudaErrorNotSupported;
+  if (a.nq > 16 || npw > 12 || smem > 227 * 1024) return cudaErrorNotSupported;
   cudaError_t e = launch_pdl(aatc_group_query_kernel, dim3(16, a.n_groups * gh, batch), dim3(kGQThreads), 0, st, a);
   if (e != cudaSuccess) return e;
   const dim3 grid(a.n_splits, a.n_groups, batch);
-  // pairs per warp: 12, 16 (g_h = 4 at ~2.75 bits: up to 32 value tiles per slice) or 24
+  // pairs per warp: 6, 8 (g_h = 4 at ~2.75 bits: up to 32 value tiles per slice) or 12
   using Kernel = void (*)(const GroupDecodeArgs);
-  const Kernel kern = gh == 2 ? (npw <= 12 ? aatc_group_digit_kernel<2, 12> : aatc_group_digit_kernel<2, 24>)
-                              : (npw <= 12 ? aatc_group_digit_kernel<4, 12>
-                                 : npw <= 16 ? aatc_group_digit_kernel<4, 16>
-                                             : aatc_group_digit_kernel<4, 24>);
+  const Kernel kern = gh == 2 ? (npw <= 6 ? aatc_group_digit_kernel<2, 6> : aatc_group_digit_kernel<2, 12>)
+                              : (npw <= 6 ? aatc_group_digit_kernel<4, 6>
+                                 : npw <= 8 ? aatc_group_digit_kernel<4, 8>
+                                            : aatc_group_digit_kernel<4, 12>);
   e = ensure_smem_optin(reinterpret_cast<const void*>(kern), smem);
   if (e != cudaSuccess) return e;
   e = launch_pdl(kern, grid, dim3(kGAThreads), smem, st, a);
