@@ -60,65 +60,68 @@ __device__ __forceinline__ uint32_t spread_digits(uint32_t x) {
 __device__ __forceinline__ uint32_t spread_bits(uint32_t x) { return (x * 0x00204081u) & 0x01010101u; }
 __device__ __forceinline__ uint32_t low_mask(int n) { return n >= 32 ? 0xFFFFFFFFu : (1u << n) - 1u; }
 
-// One CTA per (128-token tile, kv-head x K|V, sequence), thread = token: the packed record -> the
+// One CTA per (128-token tile, kv-head x K|V, sequence), thread = (token, 64 channels): the packed record -> the
 // signed codes as one 32 KB tensor-core operand, written as a whole by a bulk copy.
 // The record is read as the bit stream that the encode wrote (digit layers in channel order, then
 // the odd widths' top bits, then the digits moved out of the last D2 word): 16 digits or up to 32
-// bits per step, spread into the byte lanes of 32 registers (stored value u_c of channel c = byte
-// c & 3 of U[c >> 2]; kWide: UH holds the high bytes of the first 32 channels), which the run
-// bounds, uniform over the CTA, guard.  code = u - 2^(b-1) as f16: below 9 bits the byte is put
+// bits per step, spread into the byte lanes of 16 registers (stored value u_c of the thread's channel c =
+// byte c & 3 of U[c >> 2]; kWide: UH holds the high bytes of the first 32 channels), which the run
+// bounds, uniform over the warp, guard.  code = u - 2^(b-1) as f16: below 9 bits the byte is put
 // into the mantissa of 1024 + u, and (1024 + u) - (1024 + 2^(b-1)) is exact.
-// Bound by issue next to the write of 256 B per token and stream: 8 heads x 30011 tokens at 2.75
-// bits take 45 us (2.7 TB/s written), a single tile 6 us.  Reading each channel's entries through
-// the plan's entry lists, one field at a time in dependent loads, took 280 us and 60 us.
+// Bound by the latency of a thread's steps next to the write of 256 B per token and stream: 8 heads x
+// 30011 tokens at 2.75 bits take 38 us (3.3 TB/s written), a single tile 4.8 us.  With all 128 channels
+// of a token in one thread 46 us and 6 us, with 32 in each of four 41 us and 4.3 us; reading each
+// channel's entries through the plan's entry lists, one field at a time in dependent loads, 280 and 60 us.
+constexpr int kCodesThreads = 2 * TILE;
 template <bool kWide>
-__global__ void __launch_bounds__(TILE) aatc_prefill_codes_kernel(const PrefillArgs a) {
+__global__ void __launch_bounds__(kCodesThreads) aatc_prefill_codes_kernel(const PrefillArgs a) {
   extern __shared__ __align__(128) unsigned char smc[];
   unsigned char* op = smc;                                        // the operand, swizzled
   uint32_t* rec = reinterpret_cast<uint32_t*>(smc + kTOp);        // [n_words + 1][128], token-planar
   __shared__ __align__(16) uint32_t off2[D / 2];                  // f16 pairs 1024 + 2^(b-1) of channels 2i, 2i + 1
   __shared__ float offw[32];                                      // 2^(b-1) of the first 32 channels (kWide)
   __shared__ StreamLayout ly;
-  const int tile = blockIdx.x, hk = blockIdx.y, b = blockIdx.z, t = threadIdx.x;
+  const int tile = blockIdx.x, hk = blockIdx.y, b = blockIdx.z, tid = threadIdx.x;
+  const int t = tid & (TILE - 1), half = ptx::warp_uniform(tid >> 7), ch0 = 64 * half;   // token; the thread's first channel
   const int head = hk >> 1, kind = hk & 1;
   const size_t cs = (static_cast<size_t>(b) * a.n_kv + head) * 2 + kind;
   const int s = (a.layer * a.n_kv + head) * 2 + kind;
   const int nw = a.lay[s].words;
   const uint32_t* tw = a.words + (cs * a.n_tiles + tile) * static_cast<size_t>(a.n_words) * TILE;
-  if (t < D / 2) {
-    const __half2 o = __floats2half2_rn(1024.0f + a.enc[s * D + 2 * t].off, 1024.0f + a.enc[s * D + 2 * t + 1].off);
-    off2[t] = *reinterpret_cast<const uint32_t*>(&o);
+  if (tid < D / 2) {
+    const __half2 o = __floats2half2_rn(1024.0f + a.enc[s * D + 2 * tid].off, 1024.0f + a.enc[s * D + 2 * tid + 1].off);
+    off2[tid] = *reinterpret_cast<const uint32_t*>(&o);
   }
-  if (kWide && t < 32) offw[t] = a.enc[s * D + t].off;
-  if (t < static_cast<int>(sizeof(StreamLayout) / 4))
-    reinterpret_cast<int*>(&ly)[t] = reinterpret_cast<const int*>(a.lay + s)[t];
-  for (int w0 = 0; w0 < nw; w0 += 8) {
+  if (kWide && tid < 32) offw[tid] = a.enc[s * D + tid].off;
+  if (tid < static_cast<int>(sizeof(StreamLayout) / 4))
+    reinterpret_cast<int*>(&ly)[tid] = reinterpret_cast<const int*>(a.lay + s)[tid];
+  for (int w0 = half; w0 < nw; w0 += 16) {     // every other word of the record
     uint32_t x[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) x[i] = w0 + i < nw ? tw[(w0 + i) * TILE + t] : 0u;
+    for (int i = 0; i < 8; ++i) x[i] = w0 + 2 * i < nw ? tw[(w0 + 2 * i) * TILE + t] : 0u;
 #pragma unroll
     for (int i = 0; i < 8; ++i)
-      if (w0 + i < nw) rec[(w0 + i) * TILE + t] = x[i];
+      if (w0 + 2 * i < nw) rec[(w0 + 2 * i) * TILE + t] = x[i];
   }
   rec[nw * TILE + t] = 0u;                     // read (and masked) past the last word
   if (kind == 1) {
     // quad-interleaved: byte t & 3 of slots 4Q + (0, 2, 1, 3)[r] is quarter r of this token's word
     const uint32_t lo = (t & 3) | ((4 + (t & 3)) << 4);
-    for (int w = 0; w < nw; ++w) {
+    for (int w = half; w < nw; w += 2) {
       __syncwarp();
       const uint4 q = *reinterpret_cast<const uint4*>(rec + w * TILE + (t & ~3));
       __syncwarp();
       rec[w * TILE + t] = __byte_perm(__byte_perm(q.x, q.z, lo), __byte_perm(q.y, q.w, lo), 0x5410);
     }
   }
-  __syncthreads();                             // off2, offw, ly
+  __syncthreads();                             // the other half's words; off2, offw, ly
   auto get = [&](int p) {                      // the 32 record bits from bit p on (own column)
     const uint32_t* r = rec + (p >> 5) * TILE + t;
     return __funnelshift_r(r[0], r[TILE], p & 31);
   };
-  uint32_t U[32], UH[8];
+  uint32_t U[16], UH[8];
 #pragma unroll
-  for (int i = 0; i < 32; ++i) U[i] = 0u;
+  for (int i = 0; i < 16; ++i) U[i] = 0u;
 #pragma unroll
   for (int i = 0; i < 8; ++i) UH[i] = 0u;
   constexpr int kLayers = kWide ? 8 : 4;
@@ -131,20 +134,20 @@ __global__ void __launch_bounds__(TILE) aatc_prefill_codes_kernel(const PrefillA
     const int ca = ly.l2all[k], cb = ly.lodd[k];
     if (ca >= cb) continue;
     const int sh = 2 * (k & 3);
-    auto put = [&](int i, uint32_t (&dst)[8]) {            // 32 channels from 32 i
-      const int lo = max(ca - 32 * i, 0), n = min(cb - 32 * i, 32) - lo;
-      const uint32_t v = (get(pos) & low_mask(n)) << lo;
-      pos += n;
+    auto put = [&](int c32, uint32_t (&dst)[8]) {          // 32 channels
+      const int lo = max(ca - c32, 0), n = min(cb - c32, 32) - lo;
+      const uint32_t v = (get(pos + c32 + lo - ca) & low_mask(n)) << lo;
 #pragma unroll
       for (int j = 0; j < 8; ++j) dst[j] |= spread_bits((v >> (4 * j)) & 15u) << sh;
     };
     if (kWide && k >= 4) {
-      put(0, UH);
-      continue;
-    }
+      if (half == 0) put(0, UH);
+    } else {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (ca < 32 * i + 32 && cb > 32 * i) put(i, *reinterpret_cast<uint32_t(*)[8]>(&U[8 * i]));
+      for (int i = 0; i < 2; ++i)
+        if (ca < ch0 + 32 * i + 32 && cb > ch0 + 32 * i) put(ch0 + 32 * i, *reinterpret_cast<uint32_t(*)[8]>(&U[8 * i]));
+    }
+    pos += cb - ca;
   }
   // digit layers: layer k has the digits of channels [0, l2all[k]), the first l2[k] of them in D2
   pos = 0;
@@ -153,37 +156,37 @@ __global__ void __launch_bounds__(TILE) aatc_prefill_codes_kernel(const PrefillA
     const int lk = ly.l2[k], la = ly.l2all[k];
     if (la == 0) break;
     const int sh = 2 * (k & 3);
-    auto put = [&](int c, uint32_t (&dst)[4]) {            // 16 channels from 16 c
-      const int nd = min(max(lk - 16 * c, 0), 16), nm = min(la - 16 * c, 16) - nd;
-      uint32_t v = nd > 0 ? get(pos + 32 * c) & low_mask(2 * nd) : 0u;
-      if (nm > 0) {                                        // at most 15 digits move in all
-        v |= (get(mpos) & low_mask(2 * nm)) << (2 * nd);
-        mpos += 2 * nm;
-      }
+    auto put = [&](int c16, uint32_t (&dst)[4]) {          // 16 channels
+      const int nd = min(max(lk - c16, 0), 16), nm = min(la - c16, 16) - nd;
+      uint32_t v = nd > 0 ? get(pos + 2 * c16) & low_mask(2 * nd) : 0u;
+      if (nm > 0)                                          // at most 15 digits move in all
+        v |= (get(mpos + 2 * (c16 + nd - lk)) & low_mask(2 * nm)) << (2 * nd);
 #pragma unroll
       for (int j = 0; j < 4; ++j) dst[j] |= spread_digits((v >> (8 * j)) & 0xFFu) << sh;
     };
     if (kWide && k >= 4) {
 #pragma unroll
       for (int c = 0; c < 2; ++c)
-        if (16 * c < la) put(c, *reinterpret_cast<uint32_t(*)[4]>(&UH[4 * c]));
+        if (half == 0 && 16 * c < la) put(16 * c, *reinterpret_cast<uint32_t(*)[4]>(&UH[4 * c]));
     } else {
 #pragma unroll
-      for (int c = 0; c < 8; ++c)
-        if (16 * c < la) put(c, *reinterpret_cast<uint32_t(*)[4]>(&U[4 * c]));
+      for (int c = 0; c < 4; ++c)
+        if (ch0 + 16 * c < la) put(ch0 + 16 * c, *reinterpret_cast<uint32_t(*)[4]>(&U[4 * c]));
     }
     pos += 2 * lk;
+    mpos += 2 * (la - lk);
   }
   // f16 codes into the operand: keys K = channel, row = token; values K = token, row = channel
 #pragma unroll
-  for (int g8 = 0; g8 < 16; ++g8) {                        // eight channels
-    const uint4 o4 = *reinterpret_cast<const uint4*>(off2 + 4 * g8);
+  for (int g8 = 0; g8 < 8; ++g8) {                         // eight channels, from c8
+    const int c8 = ch0 + 8 * g8;
+    const uint4 o4 = *reinterpret_cast<const uint4*>(off2 + c8 / 2);
     const uint32_t ov[4] = {o4.x, o4.y, o4.z, o4.w};
     uint32_t h[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const uint32_t u = U[2 * g8 + (j >> 1)];
-      if (kWide && g8 < 4) {
+      if (kWide && g8 < 4 && half == 0) {
         const uint32_t uh = UH[2 * g8 + (j >> 1)], i0 = 16 * (j & 1);
         const float u0 = static_cast<float>(((u >> i0) & 0xFFu) | (((uh >> i0) & 0xFFu) << 8));
         const float u1 = static_cast<float>(((u >> (i0 + 8)) & 0xFFu) | (((uh >> (i0 + 8)) & 0xFFu) << 8));
@@ -196,18 +199,18 @@ __global__ void __launch_bounds__(TILE) aatc_prefill_codes_kernel(const PrefillA
       }
     }
     if (kind == 0) {
-      *reinterpret_cast<uint4*>(op + sw128_off(t, 8 * g8)) = make_uint4(h[0], h[1], h[2], h[3]);
+      *reinterpret_cast<uint4*>(op + sw128_off(t, c8)) = make_uint4(h[0], h[1], h[2], h[3]);
     } else {
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        *reinterpret_cast<uint16_t*>(op + sw128_off(8 * g8 + 2 * j, t)) = static_cast<uint16_t>(h[j]);
-        *reinterpret_cast<uint16_t*>(op + sw128_off(8 * g8 + 2 * j + 1, t)) = static_cast<uint16_t>(h[j] >> 16);
+        *reinterpret_cast<uint16_t*>(op + sw128_off(c8 + 2 * j, t)) = static_cast<uint16_t>(h[j]);
+        *reinterpret_cast<uint16_t*>(op + sw128_off(c8 + 2 * j + 1, t)) = static_cast<uint16_t>(h[j] >> 16);
       }
     }
   }
   ptx::fence_proxy_async_smem();
   __syncthreads();
-  if (t == 0) {
+  if (tid == 0) {
     ptx::bulk_store(a.codes + (cs * (a.n_ctx_pad / TILE) + tile) * static_cast<size_t>(TILE * D), op, kTOp);
     ptx::bulk_store_drain();
   }
@@ -825,7 +828,7 @@ cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_sta
   const size_t csm = kTOp + static_cast<size_t>(plan.n_words + 1) * TILE * 4;
   cudaError_t e = ensure_smem_optin(reinterpret_cast<const void*>(codes), csm);
   if (e != cudaSuccess) return e;
-  codes<<<dim3(a.n_ctx_pad / TILE, a.n_kv * 2, batch), TILE, csm, st>>>(a);
+  codes<<<dim3(a.n_ctx_pad / TILE, a.n_kv * 2, batch), kCodesThreads, csm, st>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t smem = sizeof(PrefillTcSmem) + 1024;
