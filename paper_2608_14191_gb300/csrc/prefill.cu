@@ -87,6 +87,7 @@ __global__ void __launch_bounds__(kCodesThreads) aatc_prefill_codes_kernel(const
   const size_t cs = (static_cast<size_t>(b) * a.n_kv + head) * 2 + kind;
   const int s = (a.layer * a.n_kv + head) * 2 + kind;
   const int nw = a.lay[s].words;
+  ptx::grid_launch_dependents();               // the attention kernel waits for this grid before its first codes
   const uint32_t* tw = a.words + (cs * a.n_tiles + tile) * static_cast<size_t>(a.n_words) * TILE;
   if (tid < D / 2) {
     const __half2 o = __floats2half2_rn(1024.0f + a.enc[s * D + 2 * tid].off, 1024.0f + a.enc[s * D + 2 * tid + 1].off);
@@ -470,6 +471,7 @@ __global__ void __launch_bounds__(kTThreads, 1)
       ptx::bulk_load(dst + st * kTOp, src + static_cast<size_t>(t) * TILE * D, kTOp, bar + st);
       return true;
     };
+    ptx::grid_dependency_wait();                          // the codes (the only thread that reads them)
     const __half* ck = a.codes + (csk * a.n_ctx_pad + tok0) * D;    // tiles of this head's keys, values: 32 KB
     const __half* cv = a.codes + (csv * a.n_ctx_pad + tok0) * D;
     int nk = 0, nv = 0;                                   // tiles requested
@@ -843,8 +845,17 @@ cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_sta
   const size_t rows = static_cast<size_t>(a.n_split) * batch * a.n_kv * n_rows;
   a.part = reinterpret_cast<float*>(static_cast<char*>(ws) + codes_bytes);
   a.part_ml = reinterpret_cast<float2*>(a.part + rows * D);
-  aatc_prefill_tc_kernel<<<dim3(blocks * a.n_split, a.n_kv, batch), kTThreads, smem, st>>>(a);
-  e = cudaGetLastError();
+  // Up to a CTA per SM a programmatic dependent of the codes kernel: its prologue (5 us) needs only q and
+  // plan constants, which were complete when that one started.  Two tokens of two sequences, a call:
+  // 17.2 -> 13.8 us.  Larger grids gain nothing by it (a chunk of 176 CTAs 258 us both ways) or lose (16
+  // rounds of CTAs 2414 -> 2477 us).
+  const dim3 grid(blocks * a.n_split, a.n_kv, batch);
+  if (static_cast<long>(grid.x) * grid.y * grid.z <= plan.num_sms) {
+    e = launch_pdl(aatc_prefill_tc_kernel, grid, dim3(kTThreads), smem, st, a);
+  } else {
+    aatc_prefill_tc_kernel<<<grid, kTThreads, smem, st>>>(a);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess || a.n_split == 1) return e;
   const long all = static_cast<long>(batch) * a.n_kv * n_rows;
   aatc_prefill_merge_kernel<<<static_cast<unsigned>((all + kPMergeRows - 1) / kPMergeRows), 32 * kPMergeRows, 0, st>>>(
