@@ -100,7 +100,10 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t& hi, uint32_t&
 // (p = 2t for base-4 words, t for bit words: the position at which the digit kernel leaves the
 // lane's fields), hi and lo parts.
 constexpr int kGQThreads = 512;
-__global__ void __launch_bounds__(kGQThreads) aatc_group_query_kernel(const GroupDecodeArgs a) {
+// kAhead: the slice's part of U_K is requested before the wait, at 64 registers (two CTAs an SM); else
+// three share an SM (see launch_group_decode).
+template <bool kAhead>
+__global__ void __launch_bounds__(kGQThreads, kAhead ? 2 : 3) aatc_group_query_kernel(const GroupDecodeArgs a) {
   __shared__ float qv[D];
   __shared__ float part[4][D];
   __shared__ float qsm[D];
@@ -113,12 +116,13 @@ __global__ void __launch_bounds__(kGQThreads) aatc_group_query_kernel(const Grou
   const size_t bg = static_cast<size_t>(b) * a.n_groups + g;
   const int pslot = (a.layer * a.n_kv + g * a.gh + s) * 2;   // plan slot of the slice's keys
   float x[32];
-  if (live) {
+  auto load_u = [&]() {
     const float* u = a.uk + (static_cast<size_t>(a.layer) * a.n_groups + g) * a.n * a.n +
                      static_cast<size_t>(m * D + 32 * dq) * a.n + s * D + c;
 #pragma unroll
     for (int k = 0; k < 32; ++k) x[k] = u[static_cast<size_t>(k) * a.n];   // 32 loads in flight per thread
-  }
+  };
+  if (kAhead && live) load_u();
   // plan constants above; the query and the workspace once the preceding grids are complete, and only
   // then may the attention kernel start, which reads the cache
   ptx::grid_dependency_wait();
@@ -127,6 +131,7 @@ __global__ void __launch_bounds__(kGQThreads) aatc_group_query_kernel(const Grou
   if (live && tid < D) qv[tid] = __bfloat162float(a.q[(static_cast<size_t>(b) * a.n_q_heads + hq) * D + tid]);
   __syncthreads();
   if (live) {
+    if (!kAhead) load_u();
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int k = 0; k < 32; ++k) acc[k & 3] = fmaf(x[k], qv[32 * dq + k], acc[k & 3]);
@@ -601,7 +606,10 @@ __global__ void __launch_bounds__(kGAThreads, 1) aatc_group_digit_kernel(const G
 // channels).  The CTA that arrives last for (i, group, sequence) adds the g_h parts in slice order
 // and divides by l, so the result does not depend on the arrival order.
 constexpr int kGMThreads = 512;
-__global__ void __launch_bounds__(kGMThreads) aatc_group_merge_kernel(const GroupDecodeArgs a) {
+// kAhead: U_V's part and the first partial sums are requested at once, at 98 registers; else three CTAs
+// share an SM.
+template <bool kAhead>
+__global__ void __launch_bounds__(kGMThreads, kAhead ? 1 : 3) aatc_group_merge_kernel(const GroupDecodeArgs a) {
   extern __shared__ float wsp[];                  // w [n_splits]
   __shared__ float red[kGMThreads / 32];
   __shared__ float part[4][D];
@@ -617,15 +625,21 @@ __global__ void __launch_bounds__(kGMThreads) aatc_group_merge_kernel(const Grou
   const float* u = a.uvt + (static_cast<size_t>(a.layer) * a.n_groups + g) * static_cast<size_t>(N) * N +
                    static_cast<size_t>(s * D + 32 * q4) * N + static_cast<size_t>(m) * D + c;
   float uv[32];
+  auto load_u = [&]() {
 #pragma unroll
-  for (int k = 0; k < 32; ++k) uv[k] = u[static_cast<size_t>(k) * N];   // 32 loads in flight per thread
+    for (int k = 0; k < 32; ++k) uv[k] = u[static_cast<size_t>(k) * N];   // 32 loads in flight per thread
+  };
+  if (kAhead) load_u();
   ptx::grid_dependency_wait();
   ptx::grid_launch_dependents();
   // the slice's partial sums of the first 4 * 24 splits, with the (m, l) pairs: one round trip
   const float* pc = pb + s * D + c;
   float x[24];
+  auto load_x = [&](int s0) {                     // 24 loads in flight per thread
 #pragma unroll
-  for (int k = 0; k < 24; ++k) x[k] = q4 + 4 * k < a.n_splits ? pc[static_cast<size_t>(q4 + 4 * k) * pstride] : 0.0f;
+    for (int k = 0; k < 24; ++k) x[k] = s0 + 4 * k < a.n_splits ? pc[static_cast<size_t>(s0 + 4 * k) * pstride] : 0.0f;
+  };
+  if (kAhead) load_x(q4);
   const bool mine = tid < a.n_splits;
   const float2 ml = mine ? *reinterpret_cast<const float2*>(pb + tid * pstride + N) : make_float2(-INFINITY, 0.0f);
   // M = max_s m_s (block reduction), then w_s and l = sum_s w_s l_s
@@ -655,11 +669,8 @@ __global__ void __launch_bounds__(kGMThreads) aatc_group_merge_kernel(const Grou
   // o_hat over the slice's channels: quarter q4 takes splits q4, q4 + 4, ...
   {
     float o[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    for (int s0 = q4; s0 < a.n_splits; s0 += 4 * 24) {   // 24 loads in flight per thread
-      if (s0 != q4) {
-#pragma unroll
-        for (int k = 0; k < 24; ++k) x[k] = s0 + 4 * k < a.n_splits ? pc[static_cast<size_t>(s0 + 4 * k) * pstride] : 0.0f;
-      }
+    for (int s0 = q4; s0 < a.n_splits; s0 += 4 * 24) {
+      if (!kAhead || s0 != q4) load_x(s0);
 #pragma unroll
       for (int k = 0; k < 24; ++k)
         if (s0 + 4 * k < a.n_splits) o[k & 3] = fmaf(wsp[s0 + 4 * k], x[k], o[k & 3]);
@@ -674,6 +685,7 @@ __global__ void __launch_bounds__(kGMThreads) aatc_group_merge_kernel(const Grou
   __syncthreads();
   // the slice's part of U_V[block m rows] o_hat: quarter q4 takes channels 32 q4 .. 32 q4 + 31
   {
+    if (!kAhead) load_u();
     float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
     for (int k = 0; k < 32; ++k) acc[k & 3] = fmaf(uv[k], ohat[32 * q4 + k], acc[k & 3]);
@@ -791,7 +803,11 @@ cudaError_t launch_group_decode(const Plan& plan, int layer, const void* q, cons
   if (GroupDigitSmem(gh, a.ks_max, a.n_words, 3).total > 227 * 1024) a.stages = 2;
   const size_t smem = static_cast<size_t>(GroupDigitSmem(gh, a.ks_max, a.n_words, a.stages).total);
   if (a.nq > 16 || npw > 12 || smem > 227 * 1024) return cudaErrorNotSupported;
-  cudaError_t e = launch_pdl(aatc_group_query_kernel, dim3(16, a.n_groups * gh, batch), dim3(kGQThreads), 0, st, a);
+  // the query and merge CTAs (16 and nq a slice) request their matrices ahead while each has an SM to
+  // itself; beyond that the kernels are bound by those reads, and three to an SM are faster (25 sequences
+  // of 933 tokens, two groups of four: a call 98 us, 140 with the reads ahead)
+  const bool ahead = 16L * a.n_groups * gh * batch <= plan.num_sms;
+  cudaError_t e = launch_pdl(ahead ? aatc_group_query_kernel<true> : aatc_group_query_kernel<false>, dim3(16, a.n_groups * gh, batch), dim3(kGQThreads), 0, st, a);
   if (e != cudaSuccess) return e;
   const dim3 grid(a.n_splits, a.n_groups, batch);
   // pairs per warp: 6, 8 (g_h = 4 at ~2.75 bits: up to 32 value tiles per slice) or 12
@@ -805,7 +821,7 @@ cudaError_t launch_group_decode(const Plan& plan, int layer, const void* q, cons
   e = launch_pdl(kern, grid, dim3(kGAThreads), smem, st, a);
   if (e != cudaSuccess) return e;
   const size_t msm = static_cast<size_t>(a.n_splits) * 4;
-  return launch_pdl(aatc_group_merge_kernel, dim3(a.nq, a.n_groups * gh, batch), dim3(kGMThreads), msm, st, a);
+  return launch_pdl(ahead ? aatc_group_merge_kernel<true> : aatc_group_merge_kernel<false>, dim3(a.nq, a.n_groups * gh, batch), dim3(kGMThreads), msm, st, a);
 }
 
 }  // namespace aatc
