@@ -1344,7 +1344,7 @@ __global__ void __launch_bounds__(256, 1) aatc_decode_fused_large_kernel(const D
 // dependency resolves.  It cannot start before the split kernel's CTAs leave, so a call ends with its
 // latency (about 2 us at a few per cent of the chip, all of it round trips to L2):
 //   PARTS CTAs per query head, each for 128 / PARTS output dimensions (all of them merge the splits and
-//   score the uncompressed tokens), U_V's part in registers instead of 64 KB through shared memory;
+//   score the uncompressed tokens), with U_V's part in registers (PARTS > 1);
 //   uncompressed tokens four to a warp with 32 bytes of a row a lane, eight values a thread in flight;
 //   PER_SM = 2 (64 registers a thread) where the grid has more CTAs than the chip SMs, else 1.
 // Two sequences, 32 query heads, 16021 tokens and 139 uncompressed ones: a call 20.6 -> 18.5 us (device
@@ -1359,12 +1359,32 @@ __global__ void __launch_bounds__(kMThreads, PER_SM)
   extern __shared__ __align__(16) float ms[];
   float* osum = ms;                                  // [kMWarps][128]
   float* ohat = osum + kMWarps * D;                  // [128]
-  float* sf = ohat + D;                              // [n_full] scores, then weights, of full tokens
+  float* ut_s = ohat + D;                            // one CTA a head: U_V^T [128 c][128 d]
+  float* sf = ut_s + (PARTS == 1 ? D * D : 0);       // [n_full] scores, then weights, of full tokens
   __shared__ float red[2][kMWarps];
+  __shared__ uint64_t bar;
+  __shared__ int s_abort;
   const int j = blockIdx.x / PARTS, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int head = j / a.group;
   const int sv = (a.layer * a.n_kv + head) * 2 + 1;
   const int dl = tid % DP, cg = tid / DP, dim = (blockIdx.x % PARTS) * DP + dl;   // output dim; channels CL cg ..
+  // U_V's part (a plan constant), before the wait: to registers, or whole by a bulk copy that holds
+  // nothing up (as 64 KB of loads per CTA would the partials': 18 sequences of 5 tokens, 8 query heads, a
+  // call 15.9 us against 13.6)
+  float uv[PARTS > 1 ? CL : 1];
+  if (PARTS == 1) {
+    if (tid == 0) {
+      s_abort = 0;
+      ptx::mbar_init(&bar, 1);
+      ptx::fence_mbar_init();
+      ptx::mbar_arrive_expect_tx(&bar, D * D * 4);
+      ptx::bulk_load(ut_s, a.u32t + static_cast<size_t>(sv) * D * D, D * D * 4, &bar);
+    }
+  } else {
+    const float* u = a.u32t + static_cast<size_t>(sv) * D * D + static_cast<size_t>(CL * cg) * D + dim;
+#pragma unroll
+    for (int c = 0; c < (PARTS > 1 ? CL : 1); ++c) uv[c] = __ldg(u + c * D);
+  }
   // the next call's query kernel may start its plan-constant prologue now; it reads the query
   // and the workspace only after this grid has completed (its griddepcontrol.wait)
   ptx::grid_launch_dependents();
@@ -1460,13 +1480,6 @@ __global__ void __launch_bounds__(kMThreads, PER_SM)
       for (int i = 0; i < 2 * CG; ++i) of += osum[i * DP + tid];
     __syncthreads();
   }
-  // U_V's part (a plan constant), requested before the wait
-  float uv[CL];
-  {
-    const float* u = a.u32t + static_cast<size_t>(sv) * D * D + static_cast<size_t>(CL * cg) * D + dim;
-#pragma unroll
-    for (int c = 0; c < CL; ++c) uv[c] = __ldg(u + c * D);
-  }
   // ---- packed splits: warp w merges splits w, w + 16, ... online (running max, rescaled sums),
   // NS splits' loads in flight per round; then the 16 warp partials are merged per channel.
   float M = -INFINITY, L = 0.0f;
@@ -1475,7 +1488,7 @@ __global__ void __launch_bounds__(kMThreads, PER_SM)
     const float* src = a.ws + (static_cast<size_t>(b) * a.n_q + j) * a.n_splits * a.pstride;
     float mw = -INFINITY, lw = 0.0f;
     float4 acc = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    constexpr int NS = PER_SM > 1 ? 2 : 4;
+    constexpr int NS = PER_SM > 1 ? 2 : 4;           // (eight at once take registers that let fewer CTAs wait early)
     for (int s0 = warp; s0 < a.n_splits; s0 += kMWarps * NS) {
       float2 ml[NS];
       float4 v[NS];
@@ -1535,11 +1548,13 @@ __global__ void __launch_bounds__(kMThreads, PER_SM)
     ohat[tid] = o * fv * ap;
   }
   __syncthreads();
+  if (PARTS == 1 && !ptx::mbar_wait_sleep(&bar, 0, &s_abort, 100)) atomicOr(a.err, 2);
   // out[d] = sum_c U_V[d][c] o_hat[c]: CG threads per dimension, CL channels each
   {
     float r4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
-    for (int c = 0; c < CL; ++c) r4[c & 3] = fmaf(uv[c], ohat[CL * cg + c], r4[c & 3]);
+    for (int c = 0; c < CL; ++c)
+      r4[c & 3] = fmaf(PARTS == 1 ? ut_s[(CL * cg + c) * D + dim] : uv[PARTS > 1 ? c : 0], ohat[CL * cg + c], r4[c & 3]);
     osum[cg * DP + dl] = (r4[0] + r4[1]) + (r4[2] + r4[3]);
   }
   __syncthreads();
@@ -1860,10 +1875,13 @@ struct FusedChoice {
 // some four tiles (`tiles` = 128-token tiles of all sequences and kv-heads): its CTAs each rotate the
 // queries and choose their code, which a few tiles do not pay for (two layers of 152 tiles: 22.0 us
 // against 19.9 of the three launches; 960 tiles: 19.9 against 24.7; 1256 tiles, four kv-head widths
-// apart: 22.0 against 26.7 a layer).  Records beyond the last (more than 32 + 2 x 5 value tiles, or
-// kAccTiles with more than four query heads per kv-head): the query / split / merge launches.
+// apart: 22.0 against 26.7 a layer), and once its CTAs, one an SM, fill four fifths of the SMs they take
+// turns on: the three launches balance many sequences better (80 CTAs of 95 tiles: 153 us a layer
+// against 115; 160 CTAs of 38 tiles: 75.5 against 69.8; 112 of 132: 65.0 against 63.3).  Records beyond the last
+// (more than 32 + 2 x 5 value tiles, or kAccTiles with more than four query heads per kv-head): the query /
+// split / merge launches.
 template <int NP>
-static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, int num_sms) {
+static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, long units, int num_sms) {
   constexpr int WG = NP == 1 ? 4 : 2;
   if (sh.same) {
     if (sh.n2v == 9 && sh.n1v == 2) return {aatc_decode_fused_kernel<9, 2, NP, WG>, WG};
@@ -1871,7 +1889,8 @@ static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, int num_sm
     if (sh.n2v == 5 && sh.n1v == 3) return {aatc_decode_fused_kernel<5, 3, NP, WG>, WG};
     if (sh.n2v == 13 && sh.n1v == 3) return {aatc_decode_fused_kernel<13, 3, NP, WG>, WG};
   }
-  if (tiles < 4L * num_sms) return {};
+  const long ctas = units * std::max(1L, std::min(num_sms / units, tiles / units));
+  if (tiles < 4L * num_sms || 5 * ctas < 4 * ((ctas + num_sms - 1) / num_sms * num_sms)) return {};
   if (sh.mixed) return {aatc_decode_fused_mixed_kernel<NP, WG>, WG};
   if (NP == 1 && sh.n2v <= 32 && sh.n1v <= 5) return {aatc_decode_fused_large_kernel, 2};
   return {};
@@ -1918,7 +1937,8 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
   if (extra.t_first < n_ctx && plan.max_bits <= 14) {
     const LayerShape sh = layer_shape(plan, layer);
     const long tiles = static_cast<long>(batch) * a.n_kv * ((n_ctx + TILE - 1) / TILE - extra.t_first / TILE);
-    fk = np == 1 ? fused_kernel_for<1>(sh, tiles, plan.num_sms) : fused_kernel_for<2>(sh, tiles, plan.num_sms);
+    const long units = static_cast<long>(batch) * a.n_kv;
+    fk = np == 1 ? fused_kernel_for<1>(sh, tiles, units, plan.num_sms) : fused_kernel_for<2>(sh, tiles, units, plan.num_sms);
     a.stage_bytes = sh.stage;
     a.nks_max = sh.nks;
     if (fk.kernel) {
@@ -1946,7 +1966,6 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
   a.qcorr = reinterpret_cast<float*>(static_cast<char*>(ws) + wsl.qcorr_off);
   if (plan.n_entries > kMaxEntries) return cudaErrorNotSupported;
   // every shape refusal comes before the first launch of the call
-  const size_t msm = 4 * (static_cast<size_t>(kMWarps) * D + D + static_cast<size_t>((a.n_full + 3) & ~3));
   // CTAs of one query head's merge: more while each has an SM to itself; two to an SM where the heads
   // outnumber the SMs.  Measured (call, us; 16021 tokens, 139 uncompressed): 64 heads in 64 CTAs 24.4, in
   // 128 22.5, in 256 24.2; 96 heads one to an SM 29.0, two 32.0; 192 heads 48.5 and 47.3, 288 64.6 and 63.0
@@ -1956,6 +1975,8 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
                      : 4 * heads > plan.num_sms ? aatc_decode_merge_kernel<2, 1>
                                                 : aatc_decode_merge_kernel<4, 1>;
   const int parts = 2 * heads > plan.num_sms ? 1 : 4 * heads > plan.num_sms ? 2 : 4;
+  const size_t msm = 4 * (static_cast<size_t>(kMWarps) * D + D + (parts == 1 ? D * D : 0) +
+                          static_cast<size_t>((a.n_full + 3) & ~3));
   cudaError_t e = cudaSuccess;
   if (fk.kernel) {
     e = ensure_smem_optin(reinterpret_cast<const void*>(fk.kernel), fsm);
