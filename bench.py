@@ -938,7 +938,7 @@ def run_ours(args):
                             "peak": peak, "unit": "GB/s",
                             "frac": round(enc_in_bytes / (enc_mean * 1e-3) / 1e9 / peak, 4),
                             "traffic": _traffic("encode_layer"), "algorithmic_bytes": enc_in_bytes,
-                            "kernel": "aatc_encode_kernel (one encode of the layer: bf16 K/V input bytes)",
+                            "kernel": "aatc_encode_tc_kernel (one encode of the layer: bf16 K/V input bytes)",
                             "peak_source": f"{peak_kind} hbm_gbs (MEASURED_PEAKS.json)"},
         "e2e": {"value": round(ws_ * steps_dec * dbytes / (e2e_ms * 1e-3) / 1e9, 2), "unit": "GB/s",
                 "h2d_bytes_per_step": int(h2d), "d2h_bytes_per_step": int(d2h),

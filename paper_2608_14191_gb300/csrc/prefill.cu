@@ -68,7 +68,7 @@ __device__ __forceinline__ uint32_t low_mask(int n) { return n >= 32 ? 0xFFFFFFF
 // byte c & 3 of U[c >> 2]; kWide: UH holds the high bytes of the first 32 channels), which the run
 // bounds, uniform over the warp, guard.  code = u - 2^(b-1) as f16: below 9 bits the byte is put
 // into the mantissa of 1024 + u, and (1024 + u) - (1024 + 2^(b-1)) is exact.
-// Bound by the latency of a thread's steps next to the write of 256 B per token and stream: 8 heads x
+// Bound by the ALU pipe (72 % active, issue 75 %) next to the write of 256 B per token and stream: 8 heads x
 // 30011 tokens at 2.75 bits take 38 us (3.3 TB/s written), a single tile 4.8 us.  With all 128 channels
 // of a token in one thread 46 us and 6 us, with 32 in each of four 41 us and 4.3 us; reading each
 // channel's entries through the plan's entry lists, one field at a time in dependent loads, 280 and 60 us.
@@ -847,7 +847,7 @@ cudaError_t launch_prefill(const Plan& plan, int layer, const void* q, int q_sta
   a.part_ml = reinterpret_cast<float2*>(a.part + rows * D);
   // Up to a CTA per SM a programmatic dependent of the codes kernel: its prologue (5 us) needs only q and
   // plan constants, which were complete when that one started.  Two tokens of two sequences, a call:
-  // 17.2 -> 13.8 us.  Larger grids gain nothing by it (a chunk of 176 CTAs 258 us both ways) or lose (16
+  // 17.2 -> 13.8 us.  Larger grids gain nothing by it (a chunk of 440 CTAs 258 us both ways) or lose (16
   // rounds of CTAs 2414 -> 2477 us).
   const dim3 grid(blocks * a.n_split, a.n_kv, batch);
   if (static_cast<long>(grid.x) * grid.y * grid.z <= plan.num_sms) {
