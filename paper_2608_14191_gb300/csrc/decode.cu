@@ -5,8 +5,8 @@
 // Two launch plans, each a chain of programmatic dependents.  Two launches per call for nearly every
 // layer: aatc_decode_fused_kernel (see there) rotates the queries and streams each split's tiles
 // through per-warp-group rings, then the merge kernel below.  Layers whose records are too large for
-// it (fused_kernel_for), or have channels wider than 14 bits, take three launches (flash-decoding
-// split over the context):
+// it or differ while its CTAs would have little to do or leave SMs idle (fused_kernel_for), or have
+// channels wider than 14 bits, take three launches (flash-decoding split over the context):
 //   query    per (sequence, kv-head, query slot): q' = (U_K^T q) f^K log2(e)/sqrt(128) for the
 //            G query heads of the GQA group, the offset corrections C_g = sum_c q'_c 2^(b_c-1),
 //            and q' per record entry as f16 hi/lo tensor-core fragments (mma.sync m16n8k16);
@@ -16,7 +16,7 @@
 //            p = 2^(s - m_g), P' = p alpha^V_t as f16 hi/lo, value entry sums
 //            sum_t P'_{g,t} digit_{t,e} by the same MMA; entry sums folded into channel sums with
 //            the offset correction; (o, m, l) per split;
-//   merge    per (sequence, query head): log-sum-exp merge of the splits, f^V / l, out = U_V o_hat.
+//   merge    per (sequence, query head, part of the dimensions): log-sum-exp merge of the splits, f^V / l, out = U_V o_hat.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
