@@ -395,6 +395,13 @@ aatc_status_t aatc_dequantize(aatc_plan_t plan, int32_t layer, const void* cache
  */
 aatc_status_t aatc_selftest_bounded_wait(int32_t limit_us, int32_t* dev_flags, void* stream);
 
+/*
+ * Test hook (host only): the most record entries of one channel in a stream of the given widths,
+ * bits [128], non-increasing, 0..AATC_MAX_BITS.  It decides which decode kernels may take a layer.
+ * Errors: AATC_ERR_INVALID_ARG, AATC_ERR_NOMEM.
+ */
+aatc_status_t aatc_selftest_channel_entries(const uint8_t* bits, int32_t* most);
+
 /* Sticky device error flags of the plan (bit 0: non-finite token scale seen by encode;
  * bit 1: a bounded wait inside a kernel timed out).  Synchronizes; clear != 0 resets them. */
 aatc_status_t aatc_get_device_error(aatc_plan_t plan, int32_t* flags, int32_t clear);

@@ -49,6 +49,7 @@ SIGNATURES = {
     "aatc_calibrate": (_I32, [ctypes.POINTER(Dims), _P, _P, _I32, _P, _I32, _F64, _F64, _I32, _P, _P, _P, _P, _P, _I32]),
     "aatc_calibrate_head_group": (_I32, [_I32, _I32, _P, _I32, _P, _I32, _F64, _I32, _I32, _P, _P, _P, _P, _P]),
     "aatc_selftest_bounded_wait": (_I32, [_I32, _P, _P]),
+    "aatc_selftest_channel_entries": (_I32, [_P, ctypes.POINTER(_I32)]),
     "aatc_plan_save": (_I32, [ctypes.c_char_p, _P, _P, _P, _P]),
     "aatc_plan_file_dims": (_I32, [ctypes.c_char_p, _P]),
     "aatc_plan_load": (_I32, [ctypes.c_char_p, _P, _P, _P, _P]),
@@ -261,6 +262,16 @@ def selftest_bounded_wait(limit_us: int, flags, stream=None):
     bit 1 of the device int32 `flags` (a torch tensor) and returns."""
     _check(load().aatc_selftest_bounded_wait(int(limit_us), _ptr(flags), _stream(stream)),
            "aatc_selftest_bounded_wait")
+
+
+def selftest_channel_entries(bits: np.ndarray) -> int:
+    """aatc_selftest_channel_entries: the most record entries of one channel of a stream, bits uint8 [128]."""
+    bits = np.ascontiguousarray(bits, np.uint8)
+    if bits.shape != (HEAD_DIM,):
+        _arg_error("aatc_selftest_channel_entries", "bits must be [128]")
+    most = _I32()
+    _check(load().aatc_selftest_channel_entries(_ptr(bits), ctypes.byref(most)), "aatc_selftest_channel_entries")
+    return most.value
 
 
 def allocate_global(dm: Dims, sigma2: np.ndarray, weights: np.ndarray, avg_bits_k: float,

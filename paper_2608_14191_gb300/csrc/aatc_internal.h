@@ -44,14 +44,18 @@ struct StreamLayout {
   int n1;                 // D1 entries
   int words;              // record words this stream uses
   int nret;               // retained channels R
+  int most;               // most entries of one channel
   int l2[8];              // D2 digit-layer lengths (digits kept in D2)
   int l2all[8];           // channels with b >= 2k + 2 (digit k exists; those past l2[k] moved to D1)
   int lodd[8];            // channels with b >= 2k + 1 (width 2k + 1 channels: [l2all[k], lodd[k]))
 };
 
-// Record entries of one channel: at most 8 digits, or 7 with one moved to D1 as two bits plus an
-// odd top bit, so 9 at 16 bits; the per-channel entry table keeps kChanEnt slots.
+// Record entries of one channel, at most: every digit is one entry, or two if it moved to D1, and the
+// moved digits come off the highest layers, so they may all belong to one channel: b entries for b bits
+// (8 up to 8 bits).  The per-channel entry table keeps kChanEnt slots.
 constexpr int kChanEnt = 16;
+static_assert(kChanEnt >= AATC_MAX_BITS, "a channel's entries");
+constexpr int kFusedChanEnt = 8;    // slots that the fused decode and the head-group decode read of it
 // The register-resident encode keeps the high bytes of the first 32 stored values: channels
 // wider than 8 bits must lie in that prefix (widths are non-increasing in storage order).
 constexpr int kMaxWideChannels = 32;
@@ -79,7 +83,7 @@ struct PlanDevice {
   const StreamLayout* lay;  // [S]
   const short* entry;     // [S][n_entries]
   const short* chan_ent;  // [S][128][kChanEnt]: entries of each channel (-1 padded)
-  const short* ce8;       // [S][128][8]: the first eight of them (0 padded)
+  const short* ce8;       // [S][128][8]: the first kFusedChanEnt of them (0 padded)
   const float* cw8;       // [S][128][8]: 2^shift of those (0: none)
   const unsigned char* pack;  // [S][kPackBytes] packing operands
   const unsigned char* proj;  // projection operands of the prefill (per-kv-head plans)

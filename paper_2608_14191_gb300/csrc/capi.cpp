@@ -178,6 +178,9 @@ void build_layout(const uint8_t* bits, StreamLayout* lay, std::vector<short>& en
   lay->words = lay->n2 / 16 + (lay->n1 + 31) / 32;
   entries = d2;
   entries.insert(entries.end(), d1.begin(), d1.end());
+  int count[D] = {0};
+  lay->most = 0;
+  for (const short e : entries) lay->most = std::max(lay->most, ++count[e & 0xFF]);
 }
 
 // The packing operand of one stream (see kPackRows) into `op` (zeroed), or false where it has none.
@@ -223,6 +226,21 @@ const char* aatc_status_string(aatc_status_t s) {
 }
 
 int32_t aatc_last_cuda_error(void) { return g_last_cuda_error; }
+
+aatc_status_t aatc_selftest_channel_entries(const uint8_t* bits, int32_t* most) {
+  if (!bits || !most) return AATC_ERR_INVALID_ARG;
+  for (int c = 0; c < aatc::D; ++c)
+    if (bits[c] > AATC_MAX_BITS || (c > 0 && bits[c] > bits[c - 1])) return AATC_ERR_INVALID_ARG;
+  try {
+    aatc::StreamLayout lay{};
+    std::vector<short> entries;
+    aatc::build_layout(bits, &lay, entries);
+    *most = lay.most;
+  } catch (const std::bad_alloc&) {
+    return AATC_ERR_NOMEM;
+  }
+  return AATC_OK;
+}
 
 int32_t aatc_version(void) { return 200; }   // 0.2.0: plan files, AATC_ERR_IO, planner widths to 16
 
@@ -286,8 +304,8 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
   const size_t o_lay = off;  off = align_up(off + static_cast<size_t>(S) * sizeof(StreamLayout), 256);
   const size_t o_ent = off;  off = align_up(off + static_cast<size_t>(S) * E * sizeof(short), 256);
   const size_t o_che = off;  off = align_up(off + SD * kChanEnt * sizeof(short), 256);
-  const size_t o_ce8 = off;  off = align_up(off + SD * 8 * sizeof(short), 256);
-  const size_t o_cw8 = off;  off = align_up(off + SD * 8 * sizeof(float), 256);
+  const size_t o_ce8 = off;  off = align_up(off + SD * kFusedChanEnt * sizeof(short), 256);
+  const size_t o_cw8 = off;  off = align_up(off + SD * kFusedChanEnt * sizeof(float), 256);
   const size_t o_err = off;  off = align_up(off + 16, 256);
   const size_t o_pck = off;  off = align_up(off + (basis ? static_cast<size_t>(S) * kPackBytes : 0), 256);
   const size_t total = off;
@@ -373,8 +391,8 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
     int fill[D] = {0};
     for (int e = 0; e < static_cast<int>(entries[s].size()); ++e) {
       const int c = entries[s][e] & 0xFF;
-      if (fill[c] < 8) {
-        const size_t i = (static_cast<size_t>(s) * D + c) * 8 + fill[c];
+      if (fill[c] < kFusedChanEnt) {
+        const size_t i = (static_cast<size_t>(s) * D + c) * kFusedChanEnt + fill[c];
         ce8[i] = static_cast<short>(e);
         cw8[i] = std::ldexp(1.0f, entries[s][e] >> 8);
       }

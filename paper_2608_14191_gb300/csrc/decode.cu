@@ -5,8 +5,9 @@
 // Two launch plans, each a chain of programmatic dependents.  Two launches per call for nearly every
 // layer: aatc_decode_fused_kernel (see there) rotates the queries and streams each split's tiles
 // through per-warp-group rings, then the merge kernel below.  Layers whose records are too large for
-// it or differ while its CTAs would have little to do or leave SMs idle (fused_kernel_for), or have
-// channels wider than 14 bits, take three launches (flash-decoding split over the context):
+// it or differ while its CTAs would have little to do or leave SMs idle (fused_kernel_for), or that have
+// value channels of more than eight record entries or a plan with channels wider than 14 bits, take
+// three launches (flash-decoding split over the context):
 //   query    per (sequence, kv-head, query slot): q' = (U_K^T q) f^K log2(e)/sqrt(128) for the
 //            G query heads of the GQA group, the offset corrections C_g = sum_c q'_c 2^(b_c-1),
 //            and q' per record entry as f16 hi/lo tensor-core fragments (mma.sync m16n8k16);
@@ -833,9 +834,9 @@ __device__ __forceinline__ void decode_fused(const DecodeArgs& a, FusedShared& f
     s_abort = 0;
     s_never = 0;
   }
-  // plan constants (never written by a kernel): the value stream's entries per channel (the first 8:
-  // all of them for widths up to 14, the only plans this kernel is launched for), the key stream's
-  // entry table; key channel constants
+  // plan constants (never written by a kernel): the value stream's entries per channel (eight slots: the
+  // layers this kernel is launched for have no channel with more), the key stream's entry table; key
+  // channel constants
   if (tid == 0) {
     ptx::mbar_init(&s_tab, 1);
     ptx::fence_mbar_init();
@@ -1839,6 +1840,7 @@ struct LayerShape {
   bool same = true;               // every key and value stream has the shape (n2v, n1v)
   bool mixed = true;              // every value stream fits the mixed kernel's accumulators
   int n2v = 0, n1v = 0;           // largest over the value streams
+  int most = 0;                   // most record entries of a value channel
   int nks = 0;                    // most score k-steps of a key stream
   int stage = 0;                  // bytes of the largest tile stage (keys, values, alpha)
 };
@@ -1854,6 +1856,7 @@ static LayerShape layer_shape(const Plan& plan, int layer) {
     }
     r.same = r.same && n2k == r.n2v && n1k == r.n1v && n2v == r.n2v && n1v == r.n1v;
     r.mixed = r.mixed && n2v + 2 * std::max(n1v, 2) <= kAccTiles && n1v <= 5;
+    r.most = std::max(r.most, l[2 * h + 1].most);
     r.n2v = std::max(r.n2v, n2v);
     r.n1v = std::max(r.n1v, n1v);
     r.nks = std::max(r.nks, n2k + 2 * n1k);
@@ -1883,6 +1886,7 @@ struct FusedChoice {
 template <int NP>
 static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, long units, int num_sms) {
   constexpr int WG = NP == 1 ? 4 : 2;
+  if (sh.most > kFusedChanEnt) return {};     // (possible from 9 bits on: nine entries, say, of 10 + 63 x 2 bits)
   if (sh.same) {
     if (sh.n2v == 9 && sh.n1v == 2) return {aatc_decode_fused_kernel<9, 2, NP, WG>, WG};
     if (sh.n2v == 3 && sh.n1v == 3) return {aatc_decode_fused_kernel<3, 3, NP, WG>, WG};
@@ -1929,9 +1933,8 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
   a.n_full = extra.n_full;
   a.full_cap = extra.full_cap;
   const int np = (a.group + 3) / 4;
-  // the fused kernel: a packed range, records it holds (widths up to 14: at most 8 entries a channel)
-  // and at least two ring stages in one SM's shared memory (uncompressed tokens, if any, join in the
-  // merge kernel)
+  // the fused kernel: a packed range, a plan of at most 14 bits a channel, records it holds and at least
+  // two ring stages in one SM's shared memory (uncompressed tokens, if any, join in the merge kernel)
   FusedChoice fk;
   size_t fsm = 0;
   if (extra.t_first < n_ctx && plan.max_bits <= 14) {

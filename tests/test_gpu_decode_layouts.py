@@ -10,9 +10,9 @@ import pytest
 import torch
 
 import harness as Hn
+from oracle import aatc_oracle as O
 from test_gpu_prefill_layouts import random_plan, tokens
 
-pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
@@ -39,6 +39,7 @@ CASES = [
 ]
 
 
+@pytest.mark.gpu
 @pytest.mark.parametrize("many", [False, True])
 @pytest.mark.parametrize("n_kv,group,b_max,total,batch,n_ctx,first", CASES)
 def test_decode_record_layouts(aatc, n_kv, group, b_max, total, batch, n_ctx, first, many):
@@ -66,6 +67,74 @@ def test_decode_record_layouts(aatc, n_kv, group, b_max, total, batch, n_ctx, fi
     assert plan.device_error() == 0
 
 
+def widths(*runs):
+    """Widths of a stream from (width, channels) runs, zeros behind them."""
+    w = np.concatenate([np.full(n, b) for b, n in runs])
+    return np.concatenate([w, np.zeros(128 - len(w))]).astype(np.uint8)
+
+
+# Value widths whose moved digits (each two entries) belong to one channel, with that channel's entries;
+# the last is of a record shape (9 + 2 words) that the fused kernel has an exact form for.
+MANY_ENTRIES = [
+    (widths((10, 1), (2, 63)), 9),
+    (widths((12, 1), (3, 127)), 11),
+    (widths((13, 1), (4, 10), (2, 117)), 12),
+    (widths((14, 1), (2, 127)), 13),
+    (widths((9, 3)), 9),
+    (widths((14, 1), (4, 15), (3, 30), (2, 82)), 12),
+]
+
+
+def entries_of_widest(bits):
+    d2, d1 = O.record_entries(bits.astype(np.int64))
+    return max(np.bincount([c for c, _ in d2 + d1], minlength=128)) if bits.any() else 0
+
+
+def test_channel_entries(aatc):
+    """The entry count that decides which decode kernels may take a layer, against the oracle's layout over
+    random widths up to 16 and at the widths above (host only)."""
+    for bits, most in MANY_ENTRIES:
+        assert aatc.selftest_channel_entries(bits) == entries_of_widest(bits) == most
+    rng = np.random.default_rng(9)
+    seen = set()
+    for _ in range(2000):
+        n = int(np.exp(rng.uniform(0, np.log(128.9))))
+        wide = int(np.exp(rng.uniform(0, np.log(min(n, 32) + 0.9))))
+        b = np.concatenate([rng.integers(1, 17, wide), rng.integers(1, 9, n - wide)])
+        bits = np.zeros(128, np.uint8)
+        bits[:n] = np.sort(np.minimum(b, rng.integers(1, 17)))[::-1]
+        most = aatc.selftest_channel_entries(bits)
+        assert most == entries_of_widest(bits)
+        assert most <= max(bits.max(), 1)              # one entry a bit: every width up to 8 fits eight slots
+        seen.add(most)
+    assert max(seen) > 8
+    with pytest.raises(aatc.AatcError):
+        aatc.selftest_channel_entries(np.full(128, 17, np.uint8))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n_ctx", [300, 39000])       # under four tiles an SM; 76 CTAs a head of eight or nine tiles
+@pytest.mark.parametrize("bits,most", MANY_ENTRIES)
+def test_decode_channels_of_many_entries(aatc, bits, most, n_ctx):
+    """Value channels of more record entries than the fused kernels' eight slots."""
+    rng = np.random.default_rng([n_ctx, most])
+    n_kv, group = 2, 4
+    basis = np.stack([np.linalg.qr(rng.standard_normal((128, 128)))[0] for _ in range(2 * n_kv)])
+    basis = basis.reshape(1, n_kv, 2, 128, 128).astype(np.float32)
+    scales = (2.6 * np.arange(1, 129) ** -0.7 * np.ones((1, n_kv, 2, 1))).astype(np.float32)
+    plan = aatc.Plan(aatc.dims(1, n_kv, n_kv * group, b_max=14), basis, np.tile(bits, (1, n_kv, 2, 1)), scales)
+    k, v = tokens(rng, basis, 1, n_ctx, n_kv)
+    cache = plan.new_cache(1, n_ctx, DEV)
+    aatc.encode(plan, 0, k, v, cache, 0, n_ctx)
+    q = torch.from_numpy(rng.standard_normal((1, n_kv * group, 128))).to(DEV).to(torch.bfloat16)
+    out = aatc.decode_attention(plan, 0, q, cache, n_ctx, n_ctx)
+    ref = attention(aatc.dequantize(plan, 0, cache, 1, 0, n_ctx, n_ctx), basis, q, group)
+    _, rel = Hn.check_decode(out.cpu().numpy().reshape(-1, 128), ref.cpu().numpy().reshape(-1, 128))
+    assert rel <= 1e-4, rel
+    assert plan.device_error() == 0
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("batch", [1, 2, 3, 5])       # 32 .. 160 query heads: each form of the merge
 @pytest.mark.parametrize("n_full", [1, 3, 65, 139, 512, 1031])
 def test_merge_of_uncompressed_tokens(aatc, batch, n_full):
