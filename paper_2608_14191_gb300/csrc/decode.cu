@@ -1810,8 +1810,19 @@ __global__ void aatc_dequant_kernel(const uint32_t* words, const float* alpha, c
   }
 }
 
+// The CTAs of one SM are held to an even share of the grid (two at least), by its shared memory: launched as
+// a dependent, the grid starts while the query kernel's CTAs still leave, and what fits (up to five a SM)
+// goes to the SMs that are free first.  Two layers of 360 CTAs (three sequences of 1825 tokens, 32 heads),
+// replayed as a graph: 28.3 us with four fitting an SM (104 registers), 31.6 with five (96), 25.7 with the
+// three of an even share; 520 CTAs 14.4 -> 13.4, 24 sequences of 981 tokens over three layers 50.9 -> 39.3.
+// One each is no faster where that is the share: the merge kernel, which may wait beside them, then has
+// fewer free SMs (four sequences with 266 uncompressed tokens 14.3 us, 11.9 with two).
+constexpr size_t kSmemPerSm = 228 * 1024, kSmemPerCta = 1024 + 128;   // of an SM; a CTA's besides the dynamic part
 template <int JPW, int NP>
 cudaError_t launch_split_t(const DecodeArgs& a, int batch, size_t smem, cudaStream_t st) {
+  const long ctas = static_cast<long>(a.n_splits) * a.n_kv * batch;
+  const long share = std::max(2L, (ctas + a.num_sms - 1) / std::max(1, a.num_sms));
+  if (share < 8) smem = std::max(smem, kSmemPerSm / (share + 1) - kSmemPerCta + 256);   // one more does not fit
   cudaError_t e = ensure_smem_optin(reinterpret_cast<const void*>(aatc_decode_split_kernel<JPW, NP>), smem);
   if (e != cudaSuccess) return e;
   return launch_pdl(aatc_decode_split_kernel<JPW, NP>, dim3(a.n_splits, a.n_kv, batch), dim3(kThreads), smem, st, a);
