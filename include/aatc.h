@@ -402,6 +402,15 @@ aatc_status_t aatc_selftest_bounded_wait(int32_t limit_us, int32_t* dev_flags, v
  */
 aatc_status_t aatc_selftest_channel_entries(const uint8_t* bits, int32_t* most);
 
+/*
+ * Test hook (host only): the kernels that a decode of packed tokens [t_first, t_end) of `batch` sequences
+ * takes, as *form: 0 query / split / merge; fused / merge with 1 one record shape, 2 records that differ,
+ * 3 large records; and *n_splits, the splits of each (sequence, kv-head).
+ * Errors: AATC_ERR_INVALID_ARG (also head-group plans and more than 8 query heads per kv-head).
+ */
+aatc_status_t aatc_selftest_decode_form(aatc_plan_t plan, int32_t layer, int32_t batch, int32_t t_first,
+                                        int32_t t_end, int32_t* form, int32_t* n_splits);
+
 /* Sticky device error flags of the plan (bit 0: non-finite token scale seen by encode;
  * bit 1: a bounded wait inside a kernel timed out).  Synchronizes; clear != 0 resets them. */
 aatc_status_t aatc_get_device_error(aatc_plan_t plan, int32_t* flags, int32_t clear);

@@ -50,6 +50,7 @@ SIGNATURES = {
     "aatc_calibrate_head_group": (_I32, [_I32, _I32, _P, _I32, _P, _I32, _F64, _I32, _I32, _P, _P, _P, _P, _P]),
     "aatc_selftest_bounded_wait": (_I32, [_I32, _P, _P]),
     "aatc_selftest_channel_entries": (_I32, [_P, ctypes.POINTER(_I32)]),
+    "aatc_selftest_decode_form": (_I32, [_P, _I32, _I32, _I32, _I32, ctypes.POINTER(_I32), ctypes.POINTER(_I32)]),
     "aatc_plan_save": (_I32, [ctypes.c_char_p, _P, _P, _P, _P]),
     "aatc_plan_file_dims": (_I32, [ctypes.c_char_p, _P]),
     "aatc_plan_load": (_I32, [ctypes.c_char_p, _P, _P, _P, _P]),
@@ -272,6 +273,15 @@ def selftest_channel_entries(bits: np.ndarray) -> int:
     most = _I32()
     _check(load().aatc_selftest_channel_entries(_ptr(bits), ctypes.byref(most)), "aatc_selftest_channel_entries")
     return most.value
+
+
+def selftest_decode_form(plan: Plan, layer: int, batch: int, t_first: int, t_end: int) -> tuple[int, int]:
+    """aatc_selftest_decode_form: (form, splits) of a decode: form 0 query / split / merge, else fused / merge
+    with 1 one record shape, 2 records that differ, 3 large records."""
+    form, splits = _I32(), _I32()
+    _check(load().aatc_selftest_decode_form(plan.handle, layer, batch, t_first, t_end, ctypes.byref(form),
+                                            ctypes.byref(splits)), "aatc_selftest_decode_form")
+    return form.value, splits.value
 
 
 def allocate_global(dm: Dims, sigma2: np.ndarray, weights: np.ndarray, avg_bits_k: float,

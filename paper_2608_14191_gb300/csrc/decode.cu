@@ -1882,13 +1882,15 @@ using FusedKernel = void (*)(const DecodeArgs);
 struct FusedChoice {
   FusedKernel kernel = nullptr;
   int groups = 0;                 // warp groups per CTA
+  int form = 0;                   // 1: one shape, 2: mixed, 3: large (0: none of them)
 };
 
 // The fused kernel for a layer.  Warp groups per CTA (one CTA per SM): four for up to four query heads
 // per kv-head (16 warps, at most 128 registers), two for five to eight (twice the value accumulators)
 // and for records past kAccTiles value tiles.  The exact shapes are those of the per-stream plans at
 // 1.5, 2, 2.75 and 4 bits per channel.  Streams that differ take the mixed kernel once every SM has
-// some four tiles (`tiles` = 128-token tiles of all sequences and kv-heads): its CTAs each rotate the
+// some four tiles (`tiles` = 128-token tiles of all sequences and kv-heads, `ctas` = the fused kernel's grid
+// for them): its CTAs each rotate the
 // queries and choose their code, which a few tiles do not pay for (two layers of 152 tiles: 22.0 us
 // against 19.9 of the three launches; 960 tiles: 19.9 against 24.7; 1256 tiles, four kv-head widths
 // apart: 22.0 against 26.7 a layer), and once its CTAs, one an SM, fill four fifths of the SMs they take
@@ -1897,20 +1899,54 @@ struct FusedChoice {
 // (more than 32 + 2 x 5 value tiles, or kAccTiles with more than four query heads per kv-head): the query /
 // split / merge launches.
 template <int NP>
-static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, long units, int num_sms) {
+static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, long ctas, int num_sms) {
   constexpr int WG = NP == 1 ? 4 : 2;
   if (sh.most > kFusedChanEnt) return {};     // (possible from 9 bits on: nine entries, say, of 10 + 63 x 2 bits)
   if (sh.same) {
-    if (sh.n2v == 9 && sh.n1v == 2) return {aatc_decode_fused_kernel<9, 2, NP, WG>, WG};
-    if (sh.n2v == 3 && sh.n1v == 3) return {aatc_decode_fused_kernel<3, 3, NP, WG>, WG};
-    if (sh.n2v == 5 && sh.n1v == 3) return {aatc_decode_fused_kernel<5, 3, NP, WG>, WG};
-    if (sh.n2v == 13 && sh.n1v == 3) return {aatc_decode_fused_kernel<13, 3, NP, WG>, WG};
+    if (sh.n2v == 9 && sh.n1v == 2) return {aatc_decode_fused_kernel<9, 2, NP, WG>, WG, 1};
+    if (sh.n2v == 3 && sh.n1v == 3) return {aatc_decode_fused_kernel<3, 3, NP, WG>, WG, 1};
+    if (sh.n2v == 5 && sh.n1v == 3) return {aatc_decode_fused_kernel<5, 3, NP, WG>, WG, 1};
+    if (sh.n2v == 13 && sh.n1v == 3) return {aatc_decode_fused_kernel<13, 3, NP, WG>, WG, 1};
   }
-  const long ctas = units * std::max(1L, std::min(num_sms / units, tiles / units));
-  if (tiles < 4L * num_sms || 5 * ctas < 4 * ((ctas + num_sms - 1) / num_sms * num_sms)) return {};
-  if (sh.mixed) return {aatc_decode_fused_mixed_kernel<NP, WG>, WG};
-  if (NP == 1 && sh.n2v <= 32 && sh.n1v <= 5) return {aatc_decode_fused_large_kernel, 2};
+  const long turn = static_cast<long>(FUSED_CTAS_PER_SM) * num_sms;      // CTAs that run at once
+  if (tiles < 4L * num_sms || 5 * ctas < 4 * ((ctas + turn - 1) / turn * turn)) return {};
+  if (sh.mixed) return {aatc_decode_fused_mixed_kernel<NP, WG>, WG, 2};
+  if (NP == 1 && sh.n2v <= 32 && sh.n1v <= 5) return {aatc_decode_fused_large_kernel, 2, 3};
   return {};
+}
+
+// The kernels that a decode of tokens [t_first, n_ctx) takes, and its splits: the fused kernel for a packed
+// range, a plan of at most 14 bits a channel, records it holds and at least two ring stages in one SM's
+// shared memory, else the three launches (uncompressed tokens, if any, join in the merge kernel).
+struct DecodeRoute {
+  FusedChoice fused;
+  LayerShape shape;               // (where `fused` has a kernel)
+  DecodeSplit split;
+  int n_stages = 0;               // fused kernel: ring stages per warp group, and its shared memory
+  size_t smem = 0;
+};
+static DecodeRoute decode_route(const Plan& plan, int layer, int batch, int n_ctx, int t_first) {
+  DecodeRoute r;
+  const int hk = plan.dims.n_kv_heads, np = (plan.dims.n_q_heads / hk + 3) / 4, sms = std::max(1, plan.num_sms);
+  const int range = n_ctx - (t_first / TILE) * TILE;
+  if (t_first < n_ctx && plan.max_bits <= 14) {
+    r.shape = layer_shape(plan, layer);
+    r.split = decode_split_for(batch, hk, range, sms, true);
+    const long units = static_cast<long>(batch) * hk;
+    const long tiles = units * ((n_ctx + TILE - 1) / TILE - t_first / TILE), ctas = units * r.split.n_splits;
+    r.fused = np == 1 ? fused_kernel_for<1>(r.shape, tiles, ctas, sms) : fused_kernel_for<2>(r.shape, tiles, ctas, sms);
+    if (r.fused.kernel) {
+      // the deepest ring (up to 3 stages per warp group) that fits
+      for (r.n_stages = 3; r.n_stages >= 2; --r.n_stages) {
+        r.smem = static_cast<size_t>(
+            FusedSmem(r.shape.stage, r.shape.nks, np, r.fused.groups, plan.n_entries, r.n_stages).total);
+        if (r.smem <= 227 * 1024) return r;
+      }
+    }
+  }
+  r.fused = {};
+  r.split = decode_split_for(batch, hk, range, sms, false);
+  return r;
 }
 
 cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void* cache, int batch, int n_ctx,
@@ -1946,28 +1982,12 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
   a.n_full = extra.n_full;
   a.full_cap = extra.full_cap;
   const int np = (a.group + 3) / 4;
-  // the fused kernel: a packed range, a plan of at most 14 bits a channel, records it holds and at least
-  // two ring stages in one SM's shared memory (uncompressed tokens, if any, join in the merge kernel)
-  FusedChoice fk;
-  size_t fsm = 0;
-  if (extra.t_first < n_ctx && plan.max_bits <= 14) {
-    const LayerShape sh = layer_shape(plan, layer);
-    const long tiles = static_cast<long>(batch) * a.n_kv * ((n_ctx + TILE - 1) / TILE - extra.t_first / TILE);
-    const long units = static_cast<long>(batch) * a.n_kv;
-    fk = np == 1 ? fused_kernel_for<1>(sh, tiles, units, plan.num_sms) : fused_kernel_for<2>(sh, tiles, units, plan.num_sms);
-    a.stage_bytes = sh.stage;
-    a.nks_max = sh.nks;
-    if (fk.kernel) {
-      // the deepest ring (up to 3 stages per warp group) that fits
-      for (a.n_stages = 3; a.n_stages >= 2; --a.n_stages) {
-        fsm = static_cast<size_t>(FusedSmem(sh.stage, sh.nks, np, fk.groups, plan.n_entries, a.n_stages).total);
-        if (fsm <= 227 * 1024) break;
-      }
-      if (a.n_stages < 2) fk.kernel = nullptr;
-    }
-  }
-  const int range = n_ctx - (extra.t_first / TILE) * TILE;
-  const DecodeSplit sp = decode_split_for(batch, a.n_kv, range, plan.num_sms, fk.kernel != nullptr);
+  const DecodeRoute route = decode_route(plan, layer, batch, n_ctx, extra.t_first);
+  const FusedChoice& fk = route.fused;
+  const DecodeSplit& sp = route.split;
+  a.stage_bytes = route.shape.stage;
+  a.nks_max = route.shape.nks;
+  a.n_stages = route.n_stages;
   a.n_splits = extra.t_first < n_ctx ? sp.n_splits : 0;     // no packed range: merge kernel only
   a.split_len = sp.split_len;
   {
@@ -1995,10 +2015,10 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
                           static_cast<size_t>((a.n_full + 3) & ~3));
   cudaError_t e = cudaSuccess;
   if (fk.kernel) {
-    e = ensure_smem_optin(reinterpret_cast<const void*>(fk.kernel), fsm);
+    e = ensure_smem_optin(reinterpret_cast<const void*>(fk.kernel), route.smem);
     if (e != cudaSuccess) return e;
     const unsigned n_cta = static_cast<unsigned>(static_cast<long>(sp.n_splits) * a.n_kv * batch);
-    e = launch_pdl(fk.kernel, dim3(n_cta), dim3(128 * fk.groups), fsm, st, a);
+    e = launch_pdl(fk.kernel, dim3(n_cta), dim3(128 * fk.groups), route.smem, st, a);
     if (e != cudaSuccess) return e;
     e = ensure_smem_optin(reinterpret_cast<const void*>(merge), msm);
     if (e != cudaSuccess) return e;
@@ -2083,6 +2103,19 @@ std::mutex g_noalloc_mutex;
 void* g_noalloc_address[kMaxDevices] = {};
 
 }  // namespace
+
+extern "C" aatc_status_t aatc_selftest_decode_form(aatc_plan_t p, int32_t layer, int32_t batch, int32_t t_first,
+                                                   int32_t t_end, int32_t* form, int32_t* n_splits) {
+  using namespace aatc;
+  Plan* plan = plan_from_handle(p);
+  if (!plan || !form || !n_splits || layer < 0 || layer >= plan->dims.n_layers || batch < 1 || t_first < 0 ||
+      t_end <= t_first || plan->group_heads > 1 || plan->dims.n_q_heads / plan->dims.n_kv_heads > MAX_GROUP)
+    return AATC_ERR_INVALID_ARG;
+  const DecodeRoute r = decode_route(*plan, layer, batch, t_end, t_first);
+  *form = r.fused.form;
+  *n_splits = r.split.n_splits;
+  return AATC_OK;
+}
 
 extern "C" aatc_status_t aatc_decode_attention_noalloc(aatc_plan_t p, int32_t layer, const void* q,
                                                        const void* cache, int32_t batch, int32_t n_ctx,
