@@ -26,27 +26,38 @@ def attention(coef, basis, q, group, first=0):
 
 
 CASES = [
-    # n_kv, group, b_max, bit totals of the heads, batch, n_ctx, first
-    (2, 4, 8, (0, 352), 1, 1, 0),                    # one token; a head whose streams hold no bits
-    (8, 4, 8, (352, 200, 97, 288), 1, 127, 0),       # differing streams, value records up to 8 + 3 words
-    (3, 3, 8, (352, 420, 131), 2, 129, 5),           # up to 13 + 4 words; the range starts inside a tile
-    (2, 1, 8, (900, 611), 1, 1000, 0),               # past 13 + 4 words
-    (1, 8, 8, (352,), 3, 4097, 130),                 # eight query heads
-    (2, 7, 8, (420, 255), 1, 700, 0),                # seven, differing streams
-    (2, 6, 8, (900, 700), 1, 300, 0),                # more than four query heads and large records
-    (4, 4, 12, (352, 449, 300), 1, 515, 0),          # channels above 8 bits
-    (1, 4, 16, (500,), 2, 260, 0),                   # channels above 14 bits
+    # n_kv, group, b_max, bit totals of the heads, batch, n_ctx, first; the kernels that many sequences take
+    (2, 4, 8, (0, 352), 1, 1, 0, 2),                 # one token; a head whose streams hold no bits
+    (8, 4, 8, (352, 200, 97, 288), 1, 127, 0, 2),    # differing streams, value records up to 8 + 3 words
+    (3, 3, 8, (352, 420, 131), 2, 129, 5, 2),        # up to 10 + 3 words; the range starts inside a tile
+    (2, 1, 8, (900, 611), 1, 1000, 0, 0),            # up to 21 + 3: no room for sixteen warps' entry sums
+    (1, 8, 8, (352,), 3, 4097, 130, 2),              # eight query heads, key and value records that differ
+    (2, 7, 8, (420, 255), 1, 700, 0, 2),             # seven, differing streams
+    (2, 6, 8, (900, 700), 1, 300, 0, 2),             # six, value records up to 13 + 2 words
+    (4, 4, 12, (352, 449, 300), 1, 515, 0, 2),       # channels above 8 bits
+    (1, 4, 16, (500,), 2, 260, 0, 0),                # channels above 14 bits
 ]
+
+
+def sequences_for(aatc, plan, first, n_ctx, form):
+    """The fewest sequences whose decode takes the kernels `form` (aatc_selftest_decode_form)."""
+    for batch in range(1, 1300):
+        got, splits = aatc.selftest_decode_form(plan, 0, batch, first, n_ctx)
+        assert splits >= 1
+        if got == form:
+            return batch
+    raise AssertionError(f"no number of sequences takes form {form}")
 
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("many", [False, True])
-@pytest.mark.parametrize("n_kv,group,b_max,total,batch,n_ctx,first", CASES)
-def test_decode_record_layouts(aatc, n_kv, group, b_max, total, batch, n_ctx, first, many):
-    if many:                                          # sequences enough for four tiles per SM (and a few more)
-        batch = 620 // (n_kv * ((n_ctx + 127) // 128)) + 1
+@pytest.mark.parametrize("n_kv,group,b_max,total,batch,n_ctx,first,form", CASES)
+def test_decode_record_layouts(aatc, n_kv, group, b_max, total, batch, n_ctx, first, form, many):
     rng = np.random.default_rng([n_ctx, n_kv, b_max])
     plan, basis, bits = random_plan(aatc, rng, n_kv, group, b_max, total)
+    if many:
+        batch = sequences_for(aatc, plan, first, n_ctx, form) if form else 160
+    assert aatc.selftest_decode_form(plan, 0, batch, first, n_ctx)[0] == (form if many else 0)
     k, v = tokens(rng, basis, batch, n_ctx, n_kv)
     cap = n_ctx + 70
     cache = plan.new_cache(batch, cap, DEV)
@@ -71,6 +82,62 @@ def widths(*runs):
     """Widths of a stream from (width, channels) runs, zeros behind them."""
     w = np.concatenate([np.full(n, b) for b, n in runs])
     return np.concatenate([w, np.zeros(128 - len(w))]).astype(np.uint8)
+
+
+def record_words(bits):
+    """(D2, D1) words of the stream's records, by the oracle's layout."""
+    d2, d1 = O.record_entries(bits.astype(np.int64))
+    return len(d2) // 16, -(-len(d1) // 32)
+
+
+# Value widths of the largest record that each bound of the mixed kernel holds, then of records beyond them.
+BOUNDS = {
+    (8, 3): widths((3, 80), (2, 48)),
+    (17, 2): widths((7, 16), (5, 40), (4, 72)),
+    (15, 3): widths((7, 10), (5, 70), (4, 22), (2, 26)),
+    (13, 4): widths((5, 90), (3, 28)),
+    (11, 5): widths((5, 52), (3, 76)),
+    (24, 5): widths((8, 4), (7, 124)),
+    (32, 0): widths((8, 128)),
+    (32, 1): widths((9, 32), (8, 96)),
+}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("values,group,n_ctx,form", [
+    (((8, 3), (17, 2)), 4, 640, 2),
+    (((15, 3), (13, 4)), 3, 641, 2),                 # a last tile of one token
+    (((11, 5), (15, 3)), 1, 24600, 2),               # several tiles of each warp group
+    (((8, 3), (17, 2)), 7, 896, 2),                  # five to eight query heads: their instantiations
+    (((15, 3), (13, 4)), 5, 897, 2),
+    (((11, 5), (17, 2)), 8, 24600, 2),
+    (((24, 5), (32, 0)), 4, 640, 3),
+    (((32, 1), (8, 3)), 2, 24601, 3),
+    (((24, 5), (32, 0)), 5, 24600, 0),               # large records, more than four query heads
+])
+def test_decode_record_bounds(aatc, values, group, n_ctx, form):
+    """Value records of each bound of the mixed kernel, and those of the large one."""
+    rng = np.random.default_rng([n_ctx, group])
+    value_bits = [BOUNDS[v] for v in values]
+    assert [record_words(b) for b in value_bits] == list(values)
+    bits = np.stack([np.stack([value_bits[1 - h], value_bits[h]]) for h in (0, 1)])[None]   # each other's as keys
+    basis = np.stack([np.linalg.qr(rng.standard_normal((128, 128)))[0] for _ in range(4)])
+    basis = basis.reshape(1, 2, 2, 128, 128).astype(np.float32)
+    scales = (2.6 * np.arange(1, 129) ** -0.7 * np.ones((1, 2, 2, 1))).astype(np.float32)
+    plan = aatc.Plan(aatc.dims(1, 2, 2 * group, b_max=int(bits.max())), basis, bits, scales)
+    batch = sequences_for(aatc, plan, 0, n_ctx, form)
+    k, v = tokens(rng, basis, batch, n_ctx, 2)
+    cache = plan.new_cache(batch, n_ctx, DEV)
+    cache.fill_(-1)                                   # whatever the cache held before
+    aatc.encode(plan, 0, k, v, cache, 0, n_ctx)
+    q = torch.from_numpy(rng.standard_normal((batch, 2 * group, 128))).to(DEV).to(torch.bfloat16)
+    out = aatc.decode_attention(plan, 0, q, cache, n_ctx, n_ctx)
+    coef = aatc.dequantize(plan, 0, cache, batch, 0, n_ctx, n_ctx)
+    for b in range(batch):                            # (one at a time: 64-bit keys and values)
+        ref = attention(coef[b:b + 1], basis, q[b:b + 1], group)
+        _, rel = Hn.check_decode(out[b].cpu().numpy(), ref[0].cpu().numpy())
+        assert rel <= 1e-4, (b, rel)
+    assert plan.device_error() == 0
 
 
 # Value widths whose moved digits (each two entries) belong to one channel, with that channel's entries;
@@ -126,6 +193,7 @@ def test_decode_channels_of_many_entries(aatc, bits, most, n_ctx):
     k, v = tokens(rng, basis, 1, n_ctx, n_kv)
     cache = plan.new_cache(1, n_ctx, DEV)
     aatc.encode(plan, 0, k, v, cache, 0, n_ctx)
+    assert aatc.selftest_decode_form(plan, 0, 1, 0, n_ctx)[0] == 0
     q = torch.from_numpy(rng.standard_normal((1, n_kv * group, 128))).to(DEV).to(torch.bfloat16)
     out = aatc.decode_attention(plan, 0, q, cache, n_ctx, n_ctx)
     ref = attention(aatc.dequantize(plan, 0, cache, 1, 0, n_ctx, n_ctx), basis, q, group)
