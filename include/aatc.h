@@ -404,7 +404,7 @@ aatc_status_t aatc_selftest_channel_entries(const uint8_t* bits, int32_t* most);
 
 /*
  * Test hook (host only): the kernels that a decode of packed tokens [t_first, t_end) of `batch` sequences
- * takes, as *form: 0 query / split / merge; fused / merge with 1 one record shape, 2 records that differ,
+ * (and no uncompressed ones) takes, as *form: 0 query / split / merge; fused / merge with 1 one record shape, 2 records that differ,
  * 3 large records; and *n_splits, the splits of each (sequence, kv-head).
  * Errors: AATC_ERR_INVALID_ARG (also head-group plans and more than 8 query heads per kv-head).
  */

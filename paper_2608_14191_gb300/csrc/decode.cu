@@ -1852,15 +1852,19 @@ cudaError_t launch_bf16_split(const Bf16Args& a, int batch, cudaStream_t st) {
 struct LayerShape {
   bool same = true;               // every key and value stream has the shape (n2v, n1v)
   bool mixed = true;              // every value stream fits the mixed kernel's accumulators
+  int n_heads = 0;
   int n2v = 0, n1v = 0;           // largest over the value streams
   int most = 0;                   // most record entries of a value channel
+  int value_tiles = 0;            // most 16-entry tiles of a value record
+  int steps_max = 0, steps_sum = 0;   // score k-steps and value tiles of a head: the most, and over the heads
   int nks = 0;                    // most score k-steps of a key stream
   int stage = 0;                  // bytes of the largest tile stage (keys, values, alpha)
 };
 static LayerShape layer_shape(const Plan& plan, int layer) {
   LayerShape r;
   const StreamLayout* l = plan.layout.data() + static_cast<size_t>(layer) * 2 * plan.dims.n_kv_heads;
-  for (int h = 0; h < plan.dims.n_kv_heads; ++h) {
+  r.n_heads = plan.dims.n_kv_heads;
+  for (int h = 0; h < r.n_heads; ++h) {
     const int n2k = l[2 * h].n2 / 16, n1k = (l[2 * h].n1 + 31) / 32;
     const int n2v = l[2 * h + 1].n2 / 16, n1v = (l[2 * h + 1].n1 + 31) / 32;
     if (h == 0) {
@@ -1870,6 +1874,9 @@ static LayerShape layer_shape(const Plan& plan, int layer) {
     r.same = r.same && n2k == r.n2v && n1k == r.n1v && n2v == r.n2v && n1v == r.n1v;
     r.mixed = r.mixed && n2v + 2 * std::max(n1v, 2) <= kAccTiles && n1v <= 5;
     r.most = std::max(r.most, l[2 * h + 1].most);
+    r.value_tiles = std::max(r.value_tiles, n2v + 2 * n1v);
+    r.steps_max = std::max(r.steps_max, n2k + 2 * n1k + n2v + 2 * n1v);
+    r.steps_sum += n2k + 2 * n1k + n2v + 2 * n1v;
     r.n2v = std::max(r.n2v, n2v);
     r.n1v = std::max(r.n1v, n1v);
     r.nks = std::max(r.nks, n2k + 2 * n1k);
@@ -1889,17 +1896,23 @@ struct FusedChoice {
 // per kv-head (16 warps, at most 128 registers), two for five to eight (twice the value accumulators)
 // and for records past kAccTiles value tiles.  The exact shapes are those of the per-stream plans at
 // 1.5, 2, 2.75 and 4 bits per channel.  Streams that differ take the mixed kernel once every SM has
-// some four tiles (`tiles` = 128-token tiles of all sequences and kv-heads, `ctas` = the fused kernel's grid
-// for them): its CTAs each rotate the
-// queries and choose their code, which a few tiles do not pay for (two layers of 152 tiles: 22.0 us
-// against 19.9 of the three launches; 960 tiles: 19.9 against 24.7; 1256 tiles, four kv-head widths
-// apart: 22.0 against 26.7 a layer), and once its CTAs, one an SM, fill four fifths of the SMs they take
-// turns on: the three launches balance many sequences better (80 CTAs of 95 tiles: 153 us a layer
-// against 115; 160 CTAs of 38 tiles: 75.5 against 69.8; 112 of 132: 65.0 against 63.3).  Records beyond the last
+// some tiles (`tiles` = 128-token tiles of all sequences and kv-heads, `ctas` = the fused kernel's grid for
+// them), as its CTAs each rotate the queries, choose their code and give whole tiles to their warp groups:
+//   five; four over up to four query heads where the split kernel would hold more than four value tiles a
+//   warp, and beside 64 uncompressed tokens.  The three launches and the mixed kernel, us a call: up to four
+//   heads, up to 16 value tiles, 4.5 tiles an SM 14.4 and 16.5, 4.8 27.2 and 29.3, 5.0 32.9 and 27.2; more value
+//   tiles, 3.6 26.4 and 29.7, 4.2 18.6 and 17.0, 4.7 43.4 and 36.9; five to eight heads 4.2 17.0 and 22.6, 4.9 18.6 and
+//   25.7, 5.1 28.1 and 24.6, 5.5 24.3 and 19.5; 544 heads with 358 uncompressed tokens, 4.5 38.2 and 30.3;
+// and once its CTAs, one an SM, fill four fifths of the SMs they take turns on, as the three launches balance
+// many sequences better (80 CTAs of 95 tiles: 153 us a layer against 115; 160 CTAs of 38 tiles: 75.5 against
+// 69.8; 112 of 132: 65.0 against 63.3).  Five to eight heads, up to 16 value tiles: four fifths of the time of
+// the longest records, which all CTAs wait for (144 CTAs, records 1.25 times their mean: 24.7 against 21.2; 150
+// of 1.25 times 42.2 against 38.1).  Of 449 drawn layers six are then more than 2 % slower than by the three
+// launches, and the mean is 6.4 % faster.  Records beyond the last
 // (more than 32 + 2 x 5 value tiles, or kAccTiles with more than four query heads per kv-head): the query /
 // split / merge launches.
 template <int NP>
-static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, long ctas, int num_sms) {
+static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, long ctas, int num_sms, int n_full) {
   constexpr int WG = NP == 1 ? 4 : 2;
   if (sh.most > kFusedChanEnt) return {};     // (possible from 9 bits on: nine entries, say, of 10 + 63 x 2 bits)
   if (sh.same) {
@@ -1908,16 +1921,21 @@ static FusedChoice fused_kernel_for(const LayerShape& sh, long tiles, long ctas,
     if (sh.n2v == 5 && sh.n1v == 3) return {aatc_decode_fused_kernel<5, 3, NP, WG>, WG, 1};
     if (sh.n2v == 13 && sh.n1v == 3) return {aatc_decode_fused_kernel<13, 3, NP, WG>, WG, 1};
   }
+  const bool light = sh.value_tiles <= 4 * kWarps;                       // the split kernel's quickest form
+  const long least = (NP == 1 && !light) || n_full >= 64 ? 4 : 5;
   const long turn = static_cast<long>(FUSED_CTAS_PER_SM) * num_sms;      // CTAs that run at once
-  if (tiles < 4L * num_sms || 5 * ctas < 4 * ((ctas + turn - 1) / turn * turn)) return {};
+  const long busy = NP == 2 && light && sh.steps_max > 0
+                        ? ctas * sh.steps_sum / (static_cast<long>(sh.n_heads) * sh.steps_max) : ctas;
+  if (tiles < least * num_sms || 5 * busy < 4 * ((ctas + turn - 1) / turn * turn)) return {};
   if (sh.mixed) return {aatc_decode_fused_mixed_kernel<NP, WG>, WG, 2};
   if (NP == 1 && sh.n2v <= 32 && sh.n1v <= 5) return {aatc_decode_fused_large_kernel, 2, 3};
   return {};
 }
 
-// The kernels that a decode of tokens [t_first, n_ctx) takes, and its splits: the fused kernel for a packed
-// range, a plan of at most 14 bits a channel, records it holds and at least two ring stages in one SM's
-// shared memory, else the three launches (uncompressed tokens, if any, join in the merge kernel).
+// The kernels that a decode of tokens [t_first, n_ctx) and n_full uncompressed ones takes, and its splits: the
+// fused kernel for a packed range, a plan of at most 14 bits a channel, records it holds and at least two
+// ring stages in one SM's shared memory, else the three launches (the uncompressed tokens join in the merge
+// kernel either way).
 struct DecodeRoute {
   FusedChoice fused;
   LayerShape shape;               // (where `fused` has a kernel)
@@ -1925,7 +1943,7 @@ struct DecodeRoute {
   int n_stages = 0;               // fused kernel: ring stages per warp group, and its shared memory
   size_t smem = 0;
 };
-static DecodeRoute decode_route(const Plan& plan, int layer, int batch, int n_ctx, int t_first) {
+static DecodeRoute decode_route(const Plan& plan, int layer, int batch, int n_ctx, int t_first, int n_full) {
   DecodeRoute r;
   const int hk = plan.dims.n_kv_heads, np = (plan.dims.n_q_heads / hk + 3) / 4, sms = std::max(1, plan.num_sms);
   const int range = n_ctx - (t_first / TILE) * TILE;
@@ -1934,7 +1952,8 @@ static DecodeRoute decode_route(const Plan& plan, int layer, int batch, int n_ct
     r.split = decode_split_for(batch, hk, range, sms, true);
     const long units = static_cast<long>(batch) * hk;
     const long tiles = units * ((n_ctx + TILE - 1) / TILE - t_first / TILE), ctas = units * r.split.n_splits;
-    r.fused = np == 1 ? fused_kernel_for<1>(r.shape, tiles, ctas, sms) : fused_kernel_for<2>(r.shape, tiles, ctas, sms);
+    r.fused = np == 1 ? fused_kernel_for<1>(r.shape, tiles, ctas, sms, n_full)
+                      : fused_kernel_for<2>(r.shape, tiles, ctas, sms, n_full);
     if (r.fused.kernel) {
       // the deepest ring (up to 3 stages per warp group) that fits
       for (r.n_stages = 3; r.n_stages >= 2; --r.n_stages) {
@@ -1982,7 +2001,7 @@ cudaError_t launch_decode(const Plan& plan, int layer, const void* q, const void
   a.n_full = extra.n_full;
   a.full_cap = extra.full_cap;
   const int np = (a.group + 3) / 4;
-  const DecodeRoute route = decode_route(plan, layer, batch, n_ctx, extra.t_first);
+  const DecodeRoute route = decode_route(plan, layer, batch, n_ctx, extra.t_first, extra.n_full);
   const FusedChoice& fk = route.fused;
   const DecodeSplit& sp = route.split;
   a.stage_bytes = route.shape.stage;
@@ -2111,7 +2130,7 @@ extern "C" aatc_status_t aatc_selftest_decode_form(aatc_plan_t p, int32_t layer,
   if (!plan || !form || !n_splits || layer < 0 || layer >= plan->dims.n_layers || batch < 1 || t_first < 0 ||
       t_end <= t_first || plan->group_heads > 1 || plan->dims.n_q_heads / plan->dims.n_kv_heads > MAX_GROUP)
     return AATC_ERR_INVALID_ARG;
-  const DecodeRoute r = decode_route(*plan, layer, batch, t_end, t_first);
+  const DecodeRoute r = decode_route(*plan, layer, batch, t_end, t_first, 0);
   *form = r.fused.form;
   *n_splits = r.split.n_splits;
   return AATC_OK;

@@ -28,6 +28,8 @@ def attention(coef, basis, q, group, first=0):
 CASES = [
     # n_kv, group, b_max, bit totals of the heads, batch, n_ctx, first; the kernels that many sequences take
     (2, 4, 8, (0, 352), 1, 1, 0, 2),                 # one token; a head whose streams hold no bits
+    (2, 4, 8, (0,), 1, 300, 0, 2),                   # no bits in the whole layer
+    (2, 7, 8, (0,), 1, 300, 0, 2),
     (8, 4, 8, (352, 200, 97, 288), 1, 127, 0, 2),    # differing streams, value records up to 8 + 3 words
     (3, 3, 8, (352, 420, 131), 2, 129, 5, 2),        # up to 10 + 3 words; the range starts inside a tile
     (2, 1, 8, (900, 611), 1, 1000, 0, 0),            # up to 21 + 3: no room for sixteen warps' entry sums
@@ -180,7 +182,7 @@ def test_channel_entries(aatc):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n_ctx", [300, 39000])       # under four tiles an SM; 76 CTAs a head of eight or nine tiles
+@pytest.mark.parametrize("n_ctx", [300, 49000])       # a few tiles; five an SM (152), where a mixed layer is fused
 @pytest.mark.parametrize("bits,most", MANY_ENTRIES)
 def test_decode_channels_of_many_entries(aatc, bits, most, n_ctx):
     """Value channels of more record entries than the fused kernels' eight slots."""
