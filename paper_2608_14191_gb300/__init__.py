@@ -435,7 +435,7 @@ def encode(plan: Plan, layer: int, K, V, cache, start: int, max_tokens: int, str
     batch, n_tokens = K.shape[0], K.shape[1]
     _cache_ok(plan, cache, batch, max_tokens, "aatc_encode")
     _check(_lib.aatc_encode(plan.handle, layer, _ptr(K), _ptr(V), batch, start, n_tokens, _ptr(cache),
-                              max_tokens, _stream(stream)), "aatc_encode")
+                            max_tokens, _stream(stream)), "aatc_encode")
 
 
 def encode_hidden(plan: Plan, layer: int, x, a_hat, cache, start: int, max_tokens: int, stream=None):
@@ -449,7 +449,7 @@ def encode_hidden(plan: Plan, layer: int, x, a_hat, cache, start: int, max_token
         _arg_error("aatc_encode_hidden", "a_hat must be [L][H_kv][2][128][d_model] for the d_model of x")
     _cache_ok(plan, cache, batch, max_tokens, "aatc_encode_hidden")
     _check(_lib.aatc_encode_hidden(plan.handle, layer, _ptr(x), d_model, _ptr(a_hat), batch, start, n_tokens,
-                                     _ptr(cache), max_tokens, _stream(stream)), "aatc_encode_hidden")
+                                   _ptr(cache), max_tokens, _stream(stream)), "aatc_encode_hidden")
 
 
 def prefill_attention(plan: Plan, layer: int, q, q_start: int, cache, n_ctx: int, max_tokens: int, out=None,
@@ -468,8 +468,8 @@ def prefill_attention(plan: Plan, layer: int, q, q_start: int, cache, n_ctx: int
                "aatc_prefill_workspace_bytes")
         workspace = _empty(max(4, (nb.value + 3) // 4), dtype=_F32, device=q.device)
     _check(_lib.aatc_prefill_attention(plan.handle, layer, _ptr(q), q_start, n_q, _ptr(cache), batch, n_ctx,
-                                         max_tokens, _ptr(out), _ptr(workspace),
-                                         workspace.nbytes, _stream(stream)),
+                                       max_tokens, _ptr(out), _ptr(workspace),
+                                       workspace.nbytes, _stream(stream)),
            "aatc_prefill_attention")
     return out
 
@@ -512,16 +512,15 @@ def decode_attention_sw(plan: Plan, layer: int, q, cache, t_first: int, t_end: i
                                                  or full_row0 + int(n_full) > cap)):
         _arg_error(where, "k_full / v_full must be contiguous and hold rows [full_row0, full_row0 + n_full)")
     if t_end > t_first and workspace is None:
-        workspace = _empty(max(1, plan.workspace_bytes(batch, t_end) // 4), dtype=_F32,
-                                device=q.device)
+        workspace = _empty(max(1, plan.workspace_bytes(batch, t_end) // 4), dtype=_F32, device=q.device)
     ws_ptr = None if workspace is None else _ptr(workspace)
     ws_bytes = 0 if workspace is None else workspace.numel() * workspace.element_size()
     row_bytes = int(full_row0) * plan.dims.n_kv_heads * HEAD_DIM * 2
     _check(_lib.aatc_decode_attention_sw(plan.handle, layer, _ptr(q), _ptr(cache), batch, t_first, t_end,
-                                           max_tokens, None if k_full is None else _ptr(k_full) + row_bytes,
-                                           None if v_full is None else _ptr(v_full) + row_bytes, int(n_full), cap,
-                                           _ptr(out),
-                                           ws_ptr, ws_bytes, _stream(stream)), "aatc_decode_attention_sw")
+                                         max_tokens, None if k_full is None else _ptr(k_full) + row_bytes,
+                                         None if v_full is None else _ptr(v_full) + row_bytes, int(n_full), cap,
+                                         _ptr(out),
+                                         ws_ptr, ws_bytes, _stream(stream)), "aatc_decode_attention_sw")
     return out
 
 
@@ -533,7 +532,7 @@ def decode_attention_noalloc(plan: Plan, layer: int, q, out, cache, n_ctx: int, 
     _cache_ok(plan, cache, q.shape[0], max_tokens, where)
     _out_ok(out, q.shape[0] * plan.dims.n_q_heads * HEAD_DIM, where)
     _check(_lib.aatc_decode_attention_noalloc(plan.handle, layer, _ptr(q), _ptr(cache), q.shape[0], n_ctx,
-                                                max_tokens, _ptr(out), _stream(stream)),
+                                              max_tokens, _ptr(out), _stream(stream)),
            "aatc_decode_attention_noalloc")
     return out
 
@@ -543,7 +542,7 @@ def dequantize(plan: Plan, layer: int, cache, batch: int, t0: int, n: int, max_t
     _cache_ok(plan, cache, batch, max_tokens, "aatc_dequantize")
     out = _empty((batch, n, plan.dims.n_kv_heads, 2, HEAD_DIM), dtype=_F32, device=cache.device)
     _check(_lib.aatc_dequantize(plan.handle, layer, _ptr(cache), batch, t0, n, max_tokens, _ptr(out),
-                                  _stream(stream)), "aatc_dequantize")
+                                _stream(stream)), "aatc_dequantize")
     return out
 
 
@@ -566,8 +565,7 @@ def bf16_decode_attention(K, V, q, n_ctx: int, out=None, workspace=None, stream=
         out = _empty((batch, n_q, HEAD_DIM), dtype=_F32, device=q.device)
     _out_ok(out, batch * n_q * HEAD_DIM, where)
     if workspace is None:
-        workspace = _empty(max(1, bf16_workspace_bytes(batch, n_kv, n_q, n_ctx) // 4), dtype=_F32,
-                                device=q.device)
+        workspace = _empty(max(1, bf16_workspace_bytes(batch, n_kv, n_q, n_ctx) // 4), dtype=_F32, device=q.device)
     _check(load().aatc_bf16_decode_attention(_ptr(K), _ptr(V), _ptr(q), batch, n_ctx, max_tokens, n_kv, n_q,
                                              _ptr(out), _ptr(workspace), workspace.numel() * 4, _stream(stream)),
            "aatc_bf16_decode_attention")

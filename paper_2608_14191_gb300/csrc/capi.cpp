@@ -450,7 +450,7 @@ aatc_status_t create_plan(const aatc_dims_t* dims, const float* basis, const uin
     plan->gdev.uvt = reinterpret_cast<const float*>(base + o_guvt);
     // rows of n_g dims, one per (layer, group, kind, slice-major channel); box 64 dims x 256 rows
     if (e == cudaSuccess)
-      e = make_tensor_map_2d(plan->tmap_g, false, plan->gdev.ubf, static_cast<uint64_t>(n_g), GB / n_g,
+      e = make_tensor_map_2d(plan->tmap_g, plan->gdev.ubf, static_cast<uint64_t>(n_g), GB / n_g,
                              static_cast<uint64_t>(n_g) * 2, 64, 256);
   }
   const cudaError_t es = cudaStreamSynchronize(st);         // also on an error: the copy reads `host`

@@ -54,7 +54,7 @@ struct GroupDecodeArgs {
   const float* cw8;          // plan: [slot][128][8] 2^shift of those (0: none)
   const ChanEnc* enc;        // plan: [slot][128] (offset 2^(b-1) of each stored value)
   const StreamLayout* lay;   // plan: [slot]
-  int layer, n_kv, gh, n_groups, group, nq, n, n_q_heads, n_ctx, n_ctx_pad, n_tiles, n_splits;
+  int layer, n_kv, gh, n_groups, group, nq, n, n_q_heads, n_ctx, n_tiles, n_splits;
   int n_words, n_entries, ks_max, stages;    // ks_max: k-steps of the widest slice; stages: ring depth
 };
 
@@ -780,7 +780,6 @@ cudaError_t launch_group_decode(const Plan& plan, int layer, const void* q, cons
   a.n = D * gh;
   a.n_q_heads = plan.dims.n_q_heads;
   a.n_ctx = n_ctx;
-  a.n_ctx_pad = (n_ctx + TILE - 1) / TILE * TILE;
   a.n_tiles = g.n_tiles;
   a.n_splits = group_splits(plan, batch, n_ctx);
   a.words = static_cast<const uint32_t*>(cache);
