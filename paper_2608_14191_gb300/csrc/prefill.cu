@@ -791,11 +791,12 @@ size_t prefill_codes_bytes(int batch, int n_kv, int n_ctx) {
   const size_t pad = (static_cast<size_t>(n_ctx) + TILE - 1) / TILE * TILE;
   return static_cast<size_t>(batch) * n_kv * 2 * pad * D * sizeof(__half);
 }
-// The codes, then room for the partial rows of up to four rounds of split CTAs (none for contexts
-// that are never split).
+// The codes, then room for the partial rows of up to four rounds of split CTAs (none for contexts that are
+// never split: too short, or of so many sequences that two splits of a row block each are past that).
 size_t prefill_workspace(const Plan& plan, int batch, int n_ctx) {
   const int most = std::min(kPMaxSplits, (n_ctx + TILE - 1) / TILE / 4);
-  const size_t rows = most < 2 ? 0 : static_cast<size_t>(std::min(4, most)) * plan.num_sms * kTRows;
+  const long ctas = most < 2 ? 0 : std::min(4L, static_cast<long>(most)) * plan.num_sms;
+  const size_t rows = 2L * batch * plan.dims.n_kv_heads <= ctas ? static_cast<size_t>(ctas) * kTRows : 0;
   return prefill_codes_bytes(batch, plan.dims.n_kv_heads, n_ctx) + rows * kPRowBytes;
 }
 

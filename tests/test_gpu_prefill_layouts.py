@@ -1,6 +1,7 @@
 """Prefill attention over record layouts and sizes at the edges of its kernels, against 64-bit
 attention over the dequantized coefficients (aatc_dequantize, itself checked bit for bit against
 the oracle).  Tolerances: the acceptance bounds of harness.py (max-abs 1e-2, relative L2 1e-3)."""
+import ctypes
 import math
 
 import numpy as np
@@ -88,6 +89,24 @@ SPLITS = [
     (2, 3, 2, 1500, 700),                            # causal ranges that end in different splits
     (1, 2, 1, 4200, 2500),                           # rows that end before the later splits begin
 ]
+
+
+def test_prefill_workspace_room(aatc):
+    """The workspace has room for partial rows only where a context of that many sequences can be split."""
+    n_kv = 2
+    plan, _, _ = random_plan(aatc, np.random.default_rng(3), n_kv, 1, 8, (352,))
+    sms = torch.cuda.get_device_properties(DEV).multi_processor_count
+
+    def extra(batch, n_ctx):
+        n = ctypes.c_size_t()
+        assert aatc.load().aatc_prefill_workspace_bytes(plan.handle, batch, n_ctx, ctypes.byref(n)) == 0
+        return n.value - batch * n_kv * 2 * ((n_ctx + 127) // 128) * 128 * 128 * 2
+
+    assert extra(1, 896) == 0                        # seven tiles: at most one split
+    assert extra(1, 897) == 2 * sms * 128 * 130 * 4  # eight tiles: two splits
+    assert extra(1, 8192) == 4 * sms * 128 * 130 * 4
+    assert extra(sms, 8192) == 4 * sms * 128 * 130 * 4   # 2 sms row blocks at least, two splits: four rounds
+    assert extra(sms + 1, 8192) == 0
 
 
 @pytest.mark.parametrize("room", ["full", "codes only"])
