@@ -1907,8 +1907,8 @@ struct FusedChoice {
 // many sequences better (80 CTAs of 95 tiles: 153 us a layer against 115; 160 CTAs of 38 tiles: 75.5 against
 // 69.8; 112 of 132: 65.0 against 63.3).  Five to eight heads, up to 16 value tiles: four fifths of the time of
 // the longest records, which all CTAs wait for (144 CTAs, records 1.25 times their mean: 24.7 against 21.2; 150
-// of 1.25 times 42.2 against 38.1).  Of 449 drawn layers six are then more than 2 % slower than by the three
-// launches, and the mean is 6.4 % faster.  Records beyond the last
+// of 1.25 times 42.2 against 38.1).  Of 475 drawn calls on both sides of the lines seven are then more than 2 %
+// slower than by the three launches, and the mean is 6.5 % faster.  Records beyond the last
 // (more than 32 + 2 x 5 value tiles, or kAccTiles with more than four query heads per kv-head): the query /
 // split / merge launches.
 template <int NP>

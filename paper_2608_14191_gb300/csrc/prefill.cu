@@ -247,8 +247,8 @@ __device__ __forceinline__ uint32_t pack_h2(float lo, float hi) {
 //             of O += P' . code_V^T.  S(t + 2), which reuses the buffer, is issued behind PV(t) and
 //             the MMAs run in issue order.
 //   epilogue  out = (f^V O / l) U_V^T on the tensor cores, both operands split hi / lo in bf16.
-// Bound by the softmax's latency: the tensor pipe needs ~1600 cycles a tile (24 MMAs of 64 and
-// more), a tile takes ~2600 (4 x 8192 x 28 heads: 2.5 ms, 3.2 ms before this split of the roles).
+// Bound by the softmax's latency: the tensor pipe needs ~1730 cycles a tile (24 MMAs of ~72), a tile
+// takes ~2700 (4 x 8192 x 28 heads, a call: 2.42 ms, 3.35 before this split of the roles).
 // Sixteen warps, four a scheduler, hide more of it than eight; halving the MMAs, dropping the
 // exponentials or the copies changes nothing, dropping the reads of alpha saves a sixth (a column's
 // alpha is one shared-memory word for every row).
@@ -759,8 +759,8 @@ __global__ void __launch_bounds__(32 * kPMergeRows) aatc_prefill_merge_kernel(co
 // fewest rounds of one CTA per SM over (tiles of a split + the ~8 tiles' worth of time a CTA spends
 // outside its tiles, and ~3 more for the merge), counted on the blocks' mean causal range.  At least
 // four tiles a split.  333 queries x 4 heads over 30011 tokens on 8 kv-heads (88 row blocks on 152
-// SMs): one split 330 us, five 228 us with the merge; 78 queries over 60710 tokens (24 row blocks) 641
-// against 130 us.
+// SMs), a call: 356 us unsplit, 259 in five splits; 78 queries over 60710 tokens (24 row blocks) 699 and
+// 195 us.
 constexpr int kPMaxSplits = 16, kPCtaTiles = 8, kPMergeTiles = 3;
 int prefill_splits(long ctas, int mean_tiles, int num_sms, size_t room_rows) {
   int best = 1;
