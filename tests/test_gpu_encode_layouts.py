@@ -24,26 +24,36 @@ def flat(width, n=128):
     return np.where(np.arange(128) < n, width, 0)
 
 
+def packs_on_tensor_cores(bits):
+    """Whether a stream has a packing operand: digit blocks of 8 columns and half-words in sixteens share 128
+    columns, the record has at most 24 words, no channel more than 8 bits."""
+    blocks = sum(-(-int((bits >= 2 * k + 1).sum()) // 32) for k in range(4))
+    words = O.stream_words(bits)
+    return bits.max() <= 8 and words <= 24 and 8 * blocks + (2 * words + 15) // 16 * 16 <= 128
+
+
 CASES = [
-    # widths of the streams (key, value, key, ...), batch, n_tokens, start
-    ([0, 352], 1, 1, 0),                                       # one token; a stream without bits
-    ([37, 352, 97, 131], 2, 127, 3),                           # short records
-    ([352, 449, 255, 611, 700, 288], 1, 129, 250),             # differing records, a second tile of one token
-    ([flat(1), flat(2), flat(3), flat(4)], 1, 128, 64),        # top bits alone, whole layers
-    ([flat(1, 1), flat(3, 5), flat(8, 3), flat(7, 17)], 1, 300, 1),     # a few channels, odd counts
-    ([flat(6, 64) + flat(4) - flat(4, 64), 352], 1, 200, 0),    # 10 blocks and 48 half-word columns, the longest record
-    ([flat(7, 65), flat(7, 64)], 1, 200, 2),                   # 12 blocks and 32 columns, the most blocks
-    ([flat(6, 65) + flat(4) - flat(4, 65), 352], 1, 200, 0),   # 11 and 48: register packing
-    ([flat(8, 97), 352], 1, 200, 7),                           # 25 words: register packing
-    ([352] * 16, 1, 128 * 81 - 5, 11),                         # several items of each group
+    # widths of the streams (key, value, key, ...), batch, n_tokens, start; whether they pack on the tensor cores
+    ([0, 352], 1, 1, 0, True),                                 # one token; a stream without bits
+    ([37, 352, 97, 131], 2, 127, 3, True),                     # short records
+    ([352, 449, 255, 500, 400, 288], 1, 129, 250, True),       # differing records, a second tile of one token
+    ([352, 449, 255, 611, 700, 288], 1, 129, 250, False),      # one with 11 blocks and 48 columns: register packing
+    ([flat(1), flat(2), flat(3), flat(4)], 1, 128, 64, True),  # top bits alone, whole layers
+    ([flat(1, 1), flat(3, 5), flat(8, 3), flat(7, 17)], 1, 300, 1, True), # a few channels, odd counts
+    ([flat(6, 64) + flat(4) - flat(4, 64), 352], 1, 200, 0, True), # 10 blocks and 48 half-word columns, the longest record
+    ([flat(7, 65), flat(7, 64)], 1, 200, 2, True),             # 12 blocks and 32 columns, the most blocks
+    ([flat(6, 65) + flat(4) - flat(4, 65), 352], 1, 200, 0, False), # 11 and 48: register packing
+    ([flat(8, 97), 352], 1, 200, 7, False),                    # 25 words: register packing
+    ([352] * 16, 1, 128 * 81 - 5, 11, True),                   # several items of each group
 ]
 
 
-@pytest.mark.parametrize("widths,batch,n_tokens,start", CASES)
-def test_encode_record_layouts(aatc, widths, batch, n_tokens, start):
+@pytest.mark.parametrize("widths,batch,n_tokens,start,tensor_cores", CASES)
+def test_encode_record_layouts(aatc, widths, batch, n_tokens, start, tensor_cores):
     n_kv = len(widths) // 2
     rng = np.random.default_rng([n_tokens, n_kv])
     bits = np.stack([decaying(rng, w) if isinstance(w, int) else w for w in widths])
+    assert all(packs_on_tensor_cores(b) for b in bits) == tensor_cores
     bits = bits.reshape(1, n_kv, 2, 128).astype(np.uint8)
     basis = np.stack([np.linalg.qr(rng.standard_normal((128, 128)))[0] for _ in widths])
     basis = basis.reshape(1, n_kv, 2, 128, 128).astype(np.float32)

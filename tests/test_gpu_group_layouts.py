@@ -9,20 +9,30 @@ import pytest
 import torch
 
 import harness as Hn
+from oracle import aatc_oracle as O
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.mark.parametrize("g_h,n_groups,group,total,batch,n_ctx", [
-    (4, 2, 4, 250, 1, 1),                             # one token; six value tiles a warp
-    (4, 1, 2, 352, 3, 129),                           # eight; a second tile of one token; eight query rows
-    (4, 1, 4, 520, 1, 40001),                         # twelve; three tiles of one split
-    (2, 2, 8, 352, 1, 127),
-    (2, 1, 1, 300, 2, 30000),                         # two query rows, four tiles of one split
-    (2, 3, 5, 900, 1, 700),                           # twelve value tiles a warp
+def value_tiles_per_warp(bits, g_h):
+    """8-entry tiles of the widest value slice over the 16 / g_h warps of a slice (by the oracle's layout)."""
+    slices = [bits[0, g, 1, s::g_h].astype(np.int64) for g in range(bits.shape[1]) for s in range(g_h)]
+    tiles = max((sum(map(len, O.record_entries(b))) + 7) // 8 for b in slices)
+    return -(-tiles // (16 // g_h))
+
+
+@pytest.mark.parametrize("g_h,n_groups,group,total,batch,n_ctx,per_warp", [
+    (4, 2, 4, 250, 1, 1, 6),                          # one token; six value tiles a warp
+    (4, 1, 2, 352, 3, 129, 7),                        # seven; a second tile of one token; eight query rows
+    (4, 1, 4, 520, 1, 40001, 8),                      # eight; three tiles of one split
+    (4, 1, 4, 900, 1, 20001, 11),                     # eleven: the kernel for up to twelve
+    (2, 2, 8, 352, 1, 127, 4),
+    (2, 1, 1, 300, 2, 30000, 3),                      # two query rows, four tiles of one split
+    (2, 3, 5, 900, 1, 700, 6),                        # six value tiles a warp
+    (2, 1, 8, 2000, 1, 40000, 7),                     # seven: the kernel for up to twelve
 ])
-def test_group_decode_layouts(aatc, g_h, n_groups, group, total, batch, n_ctx):
+def test_group_decode_layouts(aatc, g_h, n_groups, group, total, batch, n_ctx, per_warp):
     n, n_kv = 128 * g_h, n_groups * g_h
     rng = np.random.default_rng([n_ctx, g_h])
     basis = np.stack([np.linalg.qr(rng.standard_normal((n, n)))[0] for _ in range(2 * n_groups)])
@@ -30,6 +40,7 @@ def test_group_decode_layouts(aatc, g_h, n_groups, group, total, batch, n_ctx):
     w = np.exp(-0.03 / g_h * np.arange(n)) * rng.uniform(0.3, 1.0, (1, n_groups, 2, n))
     bits = np.minimum(np.round(w / w.sum(-1, keepdims=True) * total * g_h), 8)
     bits = np.sort(bits, -1)[..., ::-1].astype(np.uint8)
+    assert value_tiles_per_warp(bits, g_h) == per_warp
     scales = (2.6 * np.arange(1, n + 1) ** -0.5 * np.ones((1, n_groups, 2, 1))).astype(np.float32)
     plan = aatc.GroupPlan(aatc.dims(1, n_kv, n_kv * group), g_h, basis, bits, scales)
     g = torch.Generator(DEV).manual_seed(n_ctx)
